@@ -105,9 +105,11 @@ struct TcArgs {
     // swizzled launches (SW): the state as a 2-D tensor of 128-byte rows (32 floats), boxes
     // of box_rows rows, `boxes` boxes per segment, 128-byte swizzle in shared memory
     CUtensorMap tmap;                      // 128-byte aligned by its type
+    // U on a fixed-point grid: entry (r, c) = (bx[..].x + i bx[..].y) 2^-18 b_inv_scale, row-major;
+    // |bx| <= 2^26.  The prologue cuts each into three 9-bit slices (cut_b).
+    alignas(16) int2 bx[(1u << K) * (1u << K)];
     uint32_t box_rows, boxes;
-    int16_t b[3][(2u << K) * (2u << K)];   // slices of R (row-major n x kk), |b| <= 256
-    float b_inv_scale;                     // R = (b1 + b2 2^-9 + b3 2^-18) * b_inv_scale
+    float b_inv_scale;
     void *psi;
     int *err;
     unsigned long long ntiles;
@@ -167,6 +169,49 @@ __device__ __forceinline__ void slice3(float2 v, float scale, uint32_t &w1, uint
     w1 = pack_half2(r1, i1);
     w2 = pack_half2(r2, i2);
     w3 = pack_half2(r3 * (1.f / 512.f), i3 * (1.f / 512.f));
+}
+
+// Three 9-bit slices of a fixed-point entry, x = b1 2^18 + b2 2^9 + b3, |b1|, |b2|, |b3| <= 256.
+__device__ __forceinline__ void cut_b(int x, float &b1, float &b2, float &b3) {
+    const int i1 = (x + (1 << 17)) >> 18;
+    x -= i1 << 18;
+    const int i2 = (x + (1 << 8)) >> 9;
+    b1 = (float)i1;
+    b2 = (float)i2;
+    b3 = (float)(x - (i2 << 9));
+}
+
+// B = the FP16 slices (B1, B2, B3 2^-9 [, B2 2^-9]) of R, from the fixed-point entries in the
+// kernel's parameters: complex entry (r, c) fills R's rows 2r (re, -im) and 2r + 1 (im, re) at
+// columns 2c, 2c + 1, one FP16 pair each.  Entries i0, i0 + stride, ... two at a time.
+// Why here and in this form: the operand used to travel as three int16 copies of all of R
+// (24 KiB of parameters) read entry by entry, i.e. as constant-bank loads that serialise over
+// a warp's 16 different words and miss line by line.  That was most of a launch on a small
+// state: a 20-qubit pass took 25.0 us (12 qubits: 21.0) and takes 11.1 (7.8) with 8 KiB of
+// parameters, 16-byte generic loads and the first tiles already in flight meanwhile; a
+// 28-qubit pass 693 -> 678 us.
+template <int K, int NB>
+__device__ __forceinline__ void expand_b(unsigned char *sB, const int2 *bx, uint32_t b_bytes, uint32_t sbo,
+                                         uint32_t i0, uint32_t stride) {
+    for (uint32_t e = 2u * i0; e < (1u << (2 * K)); e += 2u * stride) {
+        const int4 v = ld_param16(bx + e);
+        const uint32_t r = e >> K, c = e & ((1u << K) - 1u);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            float re[3], im[3];
+            cut_b(q ? v.z : v.x, re[0], re[1], re[2]);
+            cut_b(q ? v.w : v.y, im[0], im[1], im[2]);
+            const uint32_t o0 = kmajor_off16(2u * r, 2u * (c + q), sbo);
+            const uint32_t o1 = kmajor_off16(2u * r + 1u, 2u * (c + q), sbo);
+#pragma unroll
+            for (int s = 0; s < NB; ++s) {
+                const int d = s == 3 ? 1 : s;                     // slice 3: B2 again
+                const float f = s >= 2 ? 1.f / 512.f : 1.f;       // exact: 9-bit integers
+                *reinterpret_cast<uint32_t *>(sB + s * b_bytes + o0) = pack_half2(re[d] * f, -im[d] * f);
+                *reinterpret_cast<uint32_t *>(sB + s * b_bytes + o1) = pack_half2(im[d] * f, re[d] * f);
+            }
+        }
+    }
 }
 
 // Batched launches build B in shared memory from a state's FP32 matrix (width kin, or
@@ -310,23 +355,19 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
         b_grid(m, sb, inv);
         build_b<K>(sB, U0, a.kin, a.jw, sb, tid, blockDim.x);
         if (tid == 0) b_scale[0] = inv;
-    } else {
-        for (uint32_t e = tid; e < KD * KD; e += blockDim.x) {
-            const uint32_t n = e / KD, kk = e % KD, off = kmajor_off16(n, kk, S::SBO);
-            *reinterpret_cast<__half *>(sB + 0 * S::B_BYTES + off) = __int2half_rn(a.b[0][e]);
-            *reinterpret_cast<__half *>(sB + 1 * S::B_BYTES + off) = __int2half_rn(a.b[1][e]);
-            // exact: integers below 2^9 times 2^-9
-            *reinterpret_cast<__half *>(sB + 2 * S::B_BYTES + off) = __float2half_rn(a.b[2][e] * (1.f / 512.f));
-            if constexpr (SUB == 1)
-                *reinterpret_cast<__half *>(sB + 3 * S::B_BYTES + off) = __float2half_rn(a.b[1][e] * (1.f / 512.f));
-        }
     }
-    fence_proxy_async_smem();
+    if constexpr (BT) fence_proxy_async_smem();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     if constexpr (BT) {
         if (tid == 0) mbar_arrive(smem_u32(&b_full[0]));   // set 0: its first use
+    } else if (warp != S::W_PROD) {
+        // every warp but the producer, which is already loading the first tiles
+        const uint32_t i = tid < S::W_PROD * 32u ? tid : tid - 32u;
+        expand_b<K, (int)S::NB>(sB, a.bx, S::B_BYTES, S::SBO, i, S::THREADS - 32u);
+        fence_proxy_async_smem();
+        named_bar(3, S::THREADS - 32u);
     }
     const uint32_t tmem = tmem_slot;
     volatile int *abort = &abort_flag;
@@ -690,7 +731,7 @@ template <int K>
 sv_status launch_tc_t(sv_state *s, const svi::Gate &g) {
     using S = TcShape<K, 1>;
     using S2 = TcShape<K, 2>;
-    constexpr uint32_t D = S::D, KD = S::KD;
+    constexpr uint32_t D = S::D;
     static std::once_flag once;
     static cudaError_t init_err = cudaSuccess;
     std::call_once(once, [] {
@@ -730,27 +771,16 @@ sv_status launch_tc_t(sv_state *s, const svi::Gate &g) {
         const sv_status st = encode_rows_map(s->buf, 8ull << s->n, 8u << p.L, &a.tmap, &a.box_rows, &a.boxes);
         if (st != SV_OK) return st;
     }
-    // R (real embedding of U) and its fixed-point slices, in FP64 on the host
+    // U on its fixed-point grid, in FP64 on the host
     double rmax = 0.0;
     for (uint32_t i = 0; i < D * D; ++i)
         rmax = std::max(rmax, std::max(std::fabs(g.u[i].real()), std::fabs(g.u[i].imag())));
     int eb = 0;
     std::frexp(rmax, &eb);                                   // rmax < 2^eb
     const double sb = std::ldexp(1.0, 8 - eb);
-    for (uint32_t n = 0; n < KD; ++n)
-        for (uint32_t kk = 0; kk < KD; ++kk) {
-            const svi::cplx u = g.u[(n >> 1) * D + (kk >> 1)];
-            double r = ((n & 1) == (kk & 1)) ? u.real() : ((n & 1) ? u.imag() : -u.imag());
-            double x = r * sb;
-            const double b1 = std::nearbyint(x);
-            x = (x - b1) * 512.0;
-            const double b2 = std::nearbyint(x);
-            x = (x - b2) * 512.0;
-            const double b3 = std::nearbyint(x);
-            a.b[0][n * KD + kk] = (int16_t)b1;
-            a.b[1][n * KD + kk] = (int16_t)b2;
-            a.b[2][n * KD + kk] = (int16_t)b3;
-        }
+    const double sx = std::ldexp(sb, 18);
+    for (uint32_t i = 0; i < D * D; ++i)
+        a.bx[i] = make_int2((int)std::lrint(g.u[i].real() * sx), (int)std::lrint(g.u[i].imag() * sx));
     a.b_inv_scale = (float)std::ldexp(1.0, eb - 8);
     a.psi = s->buf;
     a.err = reinterpret_cast<int *>(s->ws + svi::WS_ERR);
@@ -827,7 +857,7 @@ sv_status launch_tc_batch(const sv_batch_launch &L) {
     const sv_status st = encode_rows_map(L.psi, (8ull * L.states) << L.n, 8u << p.L, &a.tmap, &a.box_rows,
                                          &a.boxes);
     if (st != SV_OK) return st;
-    std::memset(a.b, 0, sizeof(a.b));
+    std::memset(a.bx, 0, sizeof(a.bx));
     a.b_inv_scale = 1.f;
     a.psi = L.psi;
     a.err = L.err;

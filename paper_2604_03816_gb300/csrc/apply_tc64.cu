@@ -78,9 +78,11 @@ struct Tc64Args {
     // swizzled launches (SW): the state as a 2-D tensor of 128-byte rows (8 amplitudes),
     // `boxes` boxes of box_rows rows per segment, 128-byte swizzle in shared memory
     CUtensorMap tmap;
+    // U on the fixed-point grid of its largest entry: (re, im) of entry (r, c), row-major; the
+    // prologue cuts each into six digits (expand_b64)
+    alignas(16) longlong2 bx[16 * 16];
     uint32_t box_rows, boxes;
-    int16_t b[6][32 * 32];   // digits of R (row-major n x kk), most significant first
-    int b_exp;               // max |R| < 2^b_exp
+    int b_exp;               // max |U| < 2^b_exp
     void *psi;
     int *err;
     unsigned long long ntiles;
@@ -125,6 +127,33 @@ __device__ __forceinline__ uint32_t digit_pair(uint32_t word) {
     const __half2 h = __hfma2(*reinterpret_cast<const __half2 *>(&word), __float2half2_rn(0.5f),
                               __float2half2_rn(-1280.f));
     return *reinterpret_cast<const uint32_t *>(&h);
+}
+
+// The twelve FP16 slices of R (B_j, then B_j 2^-9) from the fixed-point entries in the
+// kernel's parameters: complex entry (r, c) fills R's rows 2r (re, -im) and 2r + 1 (im, re)
+// at columns 2c, 2c + 1, one FP16 pair each.  Entries i0, i0 + stride, ...  4 KiB of
+// parameters in 16-byte generic loads instead of 12 KiB of int16 digits in constant-bank
+// loads (see expand_b in apply_tc.cu): a 12-qubit pass 17.2 -> 9.4 us, a 23-qubit one 97 -> 90.
+__device__ __forceinline__ void expand_b64(unsigned char *sB, const longlong2 *bx, uint32_t i0, uint32_t stride) {
+    using S = Tc64;
+    for (uint32_t e = i0; e < 256u; e += stride) {
+        const int4 v = ld_param16(bx + e);
+        const uint64_t re = ((uint64_t)(uint32_t)v.y << 32 | (uint32_t)v.x) + fxp::OFFSET;
+        const uint64_t im = ((uint64_t)(uint32_t)v.w << 32 | (uint32_t)v.z) + fxp::OFFSET;
+        const uint32_t r = e >> 4, c = e & 15u;
+        const uint32_t o0 = kmajor_off16(2u * r, 2u * c, S::SBO), o1 = kmajor_off16(2u * r + 1u, 2u * c, S::SBO);
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            const float dr = (float)((int)fxp::field(re, j) - 256), di = (float)((int)fxp::field(im, j) - 256);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float f = h ? 1.f / 512.f : 1.f;      // exact: an integer of at most 9 bits
+                const __half2 w0 = __floats2half2_rn(dr * f, -di * f), w1 = __floats2half2_rn(di * f, dr * f);
+                *reinterpret_cast<__half2 *>(sB + (6 * h + j) * S::B_BYTES + o0) = w0;
+                *reinterpret_cast<__half2 *>(sB + (6 * h + j) * S::B_BYTES + o1) = w1;
+            }
+        }
+    }
 }
 
 // Levels as integers (L0, L1 below 2^22 by the bit-pattern trick, the others by
@@ -198,20 +227,15 @@ __global__ void __launch_bounds__(576, 1) apply_tc64(const __grid_constant__ Tc6
         abort_flag = 0;
         fence_mbar_init();
     }
-    for (uint32_t e = tid; e < KD * KD; e += blockDim.x) {
-        const uint32_t n = e / KD, kk = e % KD, off = kmajor_off16(n, kk, S::SBO);
-#pragma unroll
-        for (int j = 0; j < 6; ++j) {
-            *reinterpret_cast<__half *>(sB + j * S::B_BYTES + off) = __int2half_rn(a.b[j][e]);
-            // exact: an integer of at most 9 bits times 2^-9
-            *reinterpret_cast<__half *>(sB + (6 + j) * S::B_BYTES + off) =
-                __float2half_rn((float)a.b[j][e] * (1.f / 512.f));
-        }
-    }
-    fence_proxy_async_smem();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (warp != S::W_PROD) {
+        // every warp but the producer, which is already loading the first tiles
+        expand_b64(sB, a.bx, tid < S::W_PROD * 32u ? tid : tid - 32u, S::THREADS - 32u);
+        fence_proxy_async_smem();
+        named_bar(3, S::THREADS - 32u);
+    }
     const uint32_t tmem = tmem_slot;
     volatile int *abort = &abort_flag;
     const unsigned long long first = blockIdx.x, step = gridDim.x;
@@ -505,21 +529,16 @@ sv_status launch_tc64(sv_state *s, const svi::Gate &g0) {
         const sv_status st = encode_rows_map(s->buf, 16ull << s->n, 16u << p.L, &a.tmap, &a.box_rows, &a.boxes);
         if (st != SV_OK) return st;
     }
-    // R (real embedding of U) and its six digits, exactly, on the host
+    // U on its fixed-point grid, exactly, on the host (the kernel cuts the digits)
     double rmax = 0.0;
     for (uint32_t i = 0; i < 256; ++i)
         rmax = std::max(rmax, std::max(std::fabs(g->u[i].real()), std::fabs(g->u[i].imag())));
     int eb = 0;
     std::frexp(rmax, &eb);                                   // rmax < 2^eb
     const uint32_t ebias = (uint32_t)std::max(eb + 1022, 1);    // as a biased exponent field
-    for (uint32_t n = 0; n < 32; ++n)
-        for (uint32_t kk = 0; kk < 32; ++kk) {
-            const svi::cplx u = g->u[(n >> 1) * 16 + (kk >> 1)];
-            const double r = ((n & 1) == (kk & 1)) ? u.real() : ((n & 1) ? u.imag() : -u.imag());
-            int d[6];
-            fxp::digits(fxp::to_fixed(fxp::bits_of(r), ebias), d);
-            for (int i = 0; i < 6; ++i) a.b[i][n * 32 + kk] = (int16_t)d[i];
-        }
+    for (uint32_t i = 0; i < 256; ++i)
+        a.bx[i] = make_longlong2(fxp::to_fixed(fxp::bits_of(g->u[i].real()), ebias),
+                                 fxp::to_fixed(fxp::bits_of(g->u[i].imag()), ebias));
     a.b_exp = (int)ebias - 1022;
     a.psi = s->buf;
     a.err = reinterpret_cast<int *>(s->ws + svi::WS_ERR);

@@ -169,6 +169,15 @@ __device__ __forceinline__ void tma_store_2d(const void *tmap, int32_t x, int32_
                  : "memory");
 }
 
+// 16 bytes of a kernel parameter through its generic address (16-byte aligned): an ordinary
+// coalesced load.  Indexing the parameter itself would become constant-bank loads, which
+// serialise over the different addresses of a warp and miss line by line.
+__device__ __forceinline__ int4 ld_param16(const void *p) {
+    int4 v;
+    asm volatile("ld.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+
 // The 128-byte swizzle of TMA tensor copies, for 8-byte elements at index f of a
 // 1024-byte-aligned shared-memory tile: the 16-byte chunk (index bits 1-3) is XORed with
 // the 128-byte row within the 1024-byte block (index bits 4-6).  It is linear over XOR, so
