@@ -72,9 +72,11 @@ __global__ void __launch_bounds__(256) apply_tile(const __grid_constant__ ApplyA
     SegLanes sl;
     sl.init(a.L, a.h, a.hi, threadIdx.x & 31u);
     if (threadIdx.x == 0) {
+        pass_trigger();
         mbar_init(barp, 1);
         fence_mbar_init();
     }
+    pass_wait();
     __syncthreads();
 
     uint32_t parity = 0;
@@ -171,8 +173,7 @@ sv_status launch_apply_t(sv_state *s, const svi::Gate &g) {
     const unsigned long long cap = (unsigned long long)blocks_per_sm * (unsigned long long)s->num_sms;
     const unsigned grid = (unsigned)std::min<unsigned long long>(p.ntiles, cap);
     const size_t bytes = size_t(1) << (p.L + p.h);
-    apply_tile<R, K><<<grid, 256, bytes * sizeof(C), s->stream>>>(a);
-    SV_CUDA(cudaGetLastError());
+    SV_CUDA(launch_pass(apply_tile<R, K>, grid, 256, bytes * sizeof(C), s->stream, a));
     return SV_OK;
 }
 

@@ -27,6 +27,7 @@
 #include <algorithm>
 #include <string>
 
+#include "ptx.cuh"
 #include "sv_internal.h"
 
 namespace svs {
@@ -105,8 +106,10 @@ __global__ void __launch_bounds__(256) apply_diag(const __grid_constant__ DiagAr
     using V = typename Vec<R, VEC>::T;
     constexpr int ILP = 4;
     __shared__ C tab[1 << SV_MAX_K];
+    svk::pass_trigger();
     if (threadIdx.x < (1u << a.k)) tab[threadIdx.x] = mk(a.d[2 * threadIdx.x], a.d[2 * threadIdx.x + 1]);
     __syncthreads();
+    svk::pass_wait();
     V *psi = reinterpret_cast<V *>(a.psi);
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
     for (unsigned long long e0 = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; e0 < a.items;
@@ -163,6 +166,8 @@ template <typename R, int K>
 __global__ void __launch_bounds__(256) apply_mono(const __grid_constant__ MonoArgs<R, K> a) {
     using C = typename Cx<R>::T;
     constexpr int D = 1 << K, ILP = mono_ilp<R, K>();
+    svk::pass_trigger();
+    svk::pass_wait();
     C *psi = reinterpret_cast<C *>(a.psi);
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
     for (unsigned long long g0 = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; g0 < a.count;
@@ -205,6 +210,8 @@ template <typename R, int K>
 __global__ void __launch_bounds__(256) apply_ctrl(const __grid_constant__ CtrlArgs<R, K> a) {
     using C = typename Cx<R>::T;
     constexpr int D = 1 << K;
+    svk::pass_trigger();
+    svk::pass_wait();
     C *psi = reinterpret_cast<C *>(a.psi);
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
     for (unsigned long long g = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; g < a.count;
@@ -270,8 +277,7 @@ template <typename R, int VEC>
 static sv_status launch_diag_v(sv_state *s, const DiagArgs<R> &a) {
     static int per_sm = 0;
     const unsigned grid = grid_for(apply_diag<R, VEC>, &per_sm, s, (a.items + 3) / 4);
-    apply_diag<R, VEC><<<grid, 256, 0, s->stream>>>(a);
-    SV_CUDA(cudaGetLastError());
+    SV_CUDA(svk::launch_pass(apply_diag<R, VEC>, grid, 256, 0, s->stream, a));
     return SV_OK;
 }
 
@@ -333,8 +339,7 @@ static sv_status launch_mono(sv_state *s, const svi::Structure &st, uint64_t *by
     if (bytes) *bytes = 2ull * sizeof(R) * 2ull * a.count * moved;
     if (moved == 0) return SV_OK;
     const unsigned grid = grid_for(apply_mono<R, K>, &per_sm, s, (a.count + mono_ilp<R, K>() - 1) / mono_ilp<R, K>());
-    apply_mono<R, K><<<grid, 256, 0, s->stream>>>(a);
-    SV_CUDA(cudaGetLastError());
+    SV_CUDA(svk::launch_pass(apply_mono<R, K>, grid, 256, 0, s->stream, a));
     return SV_OK;
 }
 
@@ -358,8 +363,7 @@ static sv_status launch_ctrl(sv_state *s, const svi::Structure &st, uint64_t *by
     a.sp = make_spread(st, true);
     if (bytes) *bytes = 2ull * sizeof(R) * 2ull * a.count * D;
     const unsigned grid = grid_for(apply_ctrl<R, K>, &per_sm, s, a.count);
-    apply_ctrl<R, K><<<grid, 256, 0, s->stream>>>(a);
-    SV_CUDA(cudaGetLastError());
+    SV_CUDA(svk::launch_pass(apply_ctrl<R, K>, grid, 256, 0, s->stream, a));
     return SV_OK;
 }
 

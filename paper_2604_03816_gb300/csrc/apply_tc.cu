@@ -309,6 +309,7 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
     const uint32_t seg_bytes = seg_amps * 8u;
     const uint32_t nseg = 1u << a.h;
 
+    if (tid == 0) pass_trigger();
     if (warp == S::W_MMA) {
         tmem_alloc(smem_u32(&tmem_slot), S::TMEM_COLS);
         tmem_relinquish();
@@ -406,6 +407,7 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
         // lane i issues the bulk copy of segment i of every tile
         SegLanes sl;
         sl.init(a.L, a.h, a.hi, lane);
+        pass_wait();
         uint32_t j = 0;
         unsigned long long cur = ~0ull;
         uint32_t nsw = 0;                         // state changes so far (B set = nsw & 1)
@@ -792,15 +794,16 @@ sv_status launch_tc_t(sv_state *s, const svi::Gate &g) {
     a.xs = 4u - tl;
     a.xt = std::min(tl, (uint32_t)K - 1u);   // permute within a worker's half of the members
     const unsigned grid = (unsigned)std::min<unsigned long long>(p.ntiles, (unsigned long long)s->num_sms);
+    cudaError_t e = cudaSuccess;
     // with eight worker warps per role the permutation costs less than even 2-way conflicts
     if (swz) {
-        if constexpr (K == 5) apply_tc<K, false, 2, false, true><<<grid, S2::THREADS, S2::SMEM, s->stream>>>(a);
+        if constexpr (K == 5) e = launch_pass(apply_tc<K, false, 2, false, true>, grid, S2::THREADS, S2::SMEM, s->stream, a);
     } else if (a.xt >= 1) {
-        apply_tc<K, true, 1><<<grid, S::THREADS, S::SMEM, s->stream>>>(a);
+        e = launch_pass(apply_tc<K, true, 1>, grid, S::THREADS, S::SMEM, s->stream, a);
     } else {
-        apply_tc<K, false, 1><<<grid, S::THREADS, S::SMEM, s->stream>>>(a);
+        e = launch_pass(apply_tc<K, false, 1>, grid, S::THREADS, S::SMEM, s->stream, a);
     }
-    SV_CUDA(cudaGetLastError());
+    SV_CUDA(e);
     return SV_OK;
 }
 
@@ -874,8 +877,7 @@ sv_status launch_tc_batch(const sv_batch_launch &L) {
     a.kin = L.k;
     a.jw = jw;
     const unsigned grid = (unsigned)std::min<unsigned long long>(a.ntiles, (unsigned long long)L.num_sms);
-    apply_tc<5, false, 1, true, true><<<grid, S::THREADS, S::SMEM, L.stream>>>(a);
-    SV_CUDA(cudaGetLastError());
+    SV_CUDA(launch_pass(apply_tc<5, false, 1, true, true>, grid, S::THREADS, S::SMEM, L.stream, a));
     return SV_OK;
 }
 

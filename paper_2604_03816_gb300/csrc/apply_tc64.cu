@@ -208,6 +208,7 @@ __global__ void __launch_bounds__(576, 1) apply_tc64(const __grid_constant__ Tc6
     const uint32_t seg_bytes = seg_amps * 16u;
     const uint32_t nseg = 1u << a.h;
 
+    if (tid == 0) pass_trigger();
     if (warp == S::W_MMA) {
         tmem_alloc(smem_u32(&tmem_slot), S::TMEM_COLS);
         tmem_relinquish();
@@ -263,6 +264,7 @@ __global__ void __launch_bounds__(576, 1) apply_tc64(const __grid_constant__ Tc6
         // ------------------------------------------------------------ TMA producer
         SegLanes sl;
         sl.init(a.L, a.h, a.hi, lane);
+        pass_wait();
         uint32_t j = 0;
         for (unsigned long long t = first; t < a.ntiles; t += step, ++j) {
             const uint32_t s = j % NS, u = j / NS;
@@ -552,10 +554,9 @@ sv_status launch_tc64(sv_state *s, const svi::Gate &g0) {
     const unsigned grid = (unsigned)std::min<unsigned long long>(p.ntiles, (unsigned long long)s->num_sms);
     // two targets in bits 0..2 (4-way conflicts and worse) take the swizzled staging; one
     // target there leaves 2-way conflicts, cheaper than either remedy
-    if (swz) apply_tc64<false, 1, true><<<grid, S::THREADS, S::SMEM, s->stream>>>(a);
-    else if (wide) apply_tc64<false, 2><<<grid, S2::THREADS, S2::SMEM, s->stream>>>(a);
-    else apply_tc64<false, 1><<<grid, S::THREADS, S::SMEM, s->stream>>>(a);
-    SV_CUDA(cudaGetLastError());
+    SV_CUDA(swz    ? launch_pass(apply_tc64<false, 1, true>, grid, S::THREADS, S::SMEM, s->stream, a)
+            : wide ? launch_pass(apply_tc64<false, 2>, grid, S2::THREADS, S2::SMEM, s->stream, a)
+                   : launch_pass(apply_tc64<false, 1>, grid, S::THREADS, S::SMEM, s->stream, a));
     return SV_OK;
 }
 

@@ -169,6 +169,13 @@ __device__ __forceinline__ void tma_store_2d(const void *tmap, int32_t x, int32_
                  : "memory");
 }
 
+// Programmatic dependent launch (launch_pass): let the stream's next pass start its prologue
+// now, and wait here until the previous kernel of the stream has completed and its writes are
+// visible.  Every kernel launched by launch_pass waits before it touches the state; what runs
+// before the wait reads only kernel parameters and tables uploaded before the first pass.
+__device__ __forceinline__ void pass_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pass_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // 16 bytes of a kernel parameter through its generic address (16-byte aligned): an ordinary
 // coalesced load.  Indexing the parameter itself would become constant-bank loads, which
 // serialise over the different addresses of a warp and miss line by line.

@@ -136,6 +136,26 @@ struct sv_batch_launch {
 };
 
 namespace svk {
+// Launch a pass kernel that begins with pass_trigger() and calls pass_wait() before its first
+// access to the state: its launch latency and prologue overlap the previous pass's tail.
+// Measured on whole circuits, in-order launches -> this: 350 gates on 12 qubits (complex128)
+// 3094 -> 2169 us, 50 passes on 20 qubits 573 -> 481 us, 74 on 28 qubits 50.21 -> 49.93 ms.
+template <typename Args>
+cudaError_t launch_pass(void (*kern)(Args), unsigned grid, unsigned block, size_t smem, cudaStream_t stream,
+                        const Args &args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args);
+}
+
 cudaError_t tc_batch_prepare();
 sv_status launch_tc_batch(const sv_batch_launch &L);
 // `bytes` bytes at buf as a 2-D tensor of 128-byte rows for TMA tensor copies with the
