@@ -188,7 +188,8 @@ sv_status launch_apply(sv_state *s, const Gate &g, uint64_t *bytes, int *kind) {
         const Structure st = classify(g);
         if (struct_preferred(s, st)) {
             if (kind) *kind = PASS_STRUCTURED;
-            return launch_apply_struct(s, st, bytes);
+            if (bytes) *bytes = struct_bytes(s, st);
+            return launch_apply_struct(s, st);
         }
     }
     if (bytes) *bytes = 2ull * ((s->dtype == SV_C64 ? 8ull : 16ull) << s->n);

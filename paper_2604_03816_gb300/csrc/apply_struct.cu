@@ -282,7 +282,7 @@ static sv_status launch_diag_v(sv_state *s, const DiagArgs<R> &a) {
 }
 
 template <typename R>
-static sv_status launch_diag(sv_state *s, const svi::Structure &st, uint64_t *bytes) {
+static sv_status launch_diag(sv_state *s, const svi::Structure &st) {
     DiagArgs<R> a;
     const uint32_t dv = 1u << st.v.k;
     uint32_t changed = 0;
@@ -299,7 +299,6 @@ static sv_status launch_diag(sv_state *s, const svi::Structure &st, uint64_t *by
     a.sp = make_spread(st, false);
     a.k = st.v.k;
     for (uint32_t j = 0; j < SV_MAX_K; ++j) a.t[j] = j < st.v.k ? st.v.t[j] : 0u;
-    if (bytes) *bytes = 2ull * sizeof(R) * 2ull * (count >> st.v.k) * changed;
     if (changed == 0) return SV_OK;
     // pairs of amplitudes unless a control sits at bit 0 (or the subspace is one amplitude)
     const bool pairs = count >= 2 && !(st.nctrl && st.ctrl_q[0] == 0);
@@ -308,7 +307,7 @@ static sv_status launch_diag(sv_state *s, const svi::Structure &st, uint64_t *by
 }
 
 template <typename R, int K>
-static sv_status launch_mono(sv_state *s, const svi::Structure &st, uint64_t *bytes) {
+static sv_status launch_mono(sv_state *s, const svi::Structure &st) {
     static int per_sm = 0;
     constexpr uint32_t D = 1u << K;
     MonoArgs<R, K> a;
@@ -336,7 +335,6 @@ static sv_status launch_mono(sv_state *s, const svi::Structure &st, uint64_t *by
     a.psi = s->buf;
     a.count = 1ull << (s->n - st.nctrl - K);
     a.sp = make_spread(st, true);
-    if (bytes) *bytes = 2ull * sizeof(R) * 2ull * a.count * moved;
     if (moved == 0) return SV_OK;
     const unsigned grid = grid_for(apply_mono<R, K>, &per_sm, s, (a.count + mono_ilp<R, K>() - 1) / mono_ilp<R, K>());
     SV_CUDA(svk::launch_pass(apply_mono<R, K>, grid, 256, 0, s->stream, a));
@@ -344,7 +342,7 @@ static sv_status launch_mono(sv_state *s, const svi::Structure &st, uint64_t *by
 }
 
 template <typename R, int K>
-static sv_status launch_ctrl(sv_state *s, const svi::Structure &st, uint64_t *bytes) {
+static sv_status launch_ctrl(sv_state *s, const svi::Structure &st) {
     static int per_sm = 0;
     constexpr uint32_t D = 1u << K;
     CtrlArgs<R, K> a;
@@ -361,34 +359,33 @@ static sv_status launch_ctrl(sv_state *s, const svi::Structure &st, uint64_t *by
     a.psi = s->buf;
     a.count = 1ull << (s->n - st.nctrl - K);
     a.sp = make_spread(st, true);
-    if (bytes) *bytes = 2ull * sizeof(R) * 2ull * a.count * D;
     const unsigned grid = grid_for(apply_ctrl<R, K>, &per_sm, s, a.count);
     SV_CUDA(svk::launch_pass(apply_ctrl<R, K>, grid, 256, 0, s->stream, a));
     return SV_OK;
 }
 
 template <typename R>
-static sv_status launch_struct_t(sv_state *s, const svi::Structure &st, uint64_t *bytes) {
-    if (st.kind == SV_STRUCT_DIAGONAL) return launch_diag<R>(s, st, bytes);
+static sv_status launch_struct_t(sv_state *s, const svi::Structure &st) {
+    if (st.kind == SV_STRUCT_DIAGONAL) return launch_diag<R>(s, st);
     if (st.kind == SV_STRUCT_MONOMIAL) {
         switch (st.v.k) {
-            case 1: return launch_mono<R, 1>(s, st, bytes);
-            case 2: return launch_mono<R, 2>(s, st, bytes);
-            case 3: return launch_mono<R, 3>(s, st, bytes);
-            case 4: return launch_mono<R, 4>(s, st, bytes);
-            case 5: return launch_mono<R, 5>(s, st, bytes);
+            case 1: return launch_mono<R, 1>(s, st);
+            case 2: return launch_mono<R, 2>(s, st);
+            case 3: return launch_mono<R, 3>(s, st);
+            case 4: return launch_mono<R, 4>(s, st);
+            case 5: return launch_mono<R, 5>(s, st);
             default: break;
         }
     } else if (st.kind == SV_STRUCT_DENSE) {
         switch (st.v.k) {
-            case 1: return launch_ctrl<R, 1>(s, st, bytes);
-            case 2: return launch_ctrl<R, 2>(s, st, bytes);
+            case 1: return launch_ctrl<R, 1>(s, st);
+            case 2: return launch_ctrl<R, 2>(s, st);
             default: break;
         }
         // complex128 takes a dense remainder only with fewer targets than controls (<= 2)
         if constexpr (sizeof(R) == 4) switch (st.v.k) {
-            case 3: return launch_ctrl<R, 3>(s, st, bytes);
-            case 4: return launch_ctrl<R, 4>(s, st, bytes);
+            case 3: return launch_ctrl<R, 3>(s, st);
+            case 4: return launch_ctrl<R, 4>(s, st);
             default: break;
         }
     }
@@ -405,13 +402,26 @@ bool struct_preferred(const sv_state *s, const Structure &st) {
     return s->dtype == SV_C64 ? st.v.k <= 4 : st.v.k < st.nctrl;
 }
 
-sv_status launch_apply_struct(sv_state *s, const Structure &st, uint64_t *bytes) {
-    if (st.kind == SV_STRUCT_IDENTITY) {
-        if (bytes) *bytes = 0;
-        return SV_OK;
+template <typename R>
+static uint64_t struct_bytes_t(const sv_state *s, const Structure &st) {
+    const uint32_t D = 1u << st.v.k;
+    uint32_t rows = 0;                     // rows of V that change their amplitude
+    for (uint32_t r = 0; r < D; ++r) {
+        const bool alone = st.kind != SV_STRUCT_DENSE && svs::is_one<R>(st.v.u[(size_t)r * D + r]);
+        rows += !alone;
     }
-    return s->dtype == SV_C64 ? svs::launch_struct_t<float>(s, st, bytes)
-                              : svs::launch_struct_t<double>(s, st, bytes);
+    return 4ull * sizeof(R) * (1ull << (s->n - st.nctrl - st.v.k)) * rows;
+}
+
+uint64_t struct_bytes(const sv_state *s, const Structure &st) {
+    if (st.kind == SV_STRUCT_IDENTITY) return 0;
+    return s->dtype == SV_C64 ? struct_bytes_t<float>(s, st) : struct_bytes_t<double>(s, st);
+}
+
+sv_status launch_apply_struct(sv_state *s, const Structure &st) {
+    if (st.kind == SV_STRUCT_IDENTITY) return SV_OK;
+    return s->dtype == SV_C64 ? svs::launch_struct_t<float>(s, st)
+                              : svs::launch_struct_t<double>(s, st);
 }
 
 }  // namespace svi

@@ -556,8 +556,9 @@ static void plan_passes(const sv_state *s, const std::vector<Gate> &gates, size_
 // the events).
 static sv_status run_schedule(sv_state *s, const std::vector<Gate> &gates, size_t begin, size_t end,
                               bool timing, sv_apply_report *r) {
+    const bool small = small_state(s);
     std::vector<int> first, second;
-    plan_passes(s, gates, begin, end, &first, &second);
+    if (!small) plan_passes(s, gates, begin, end, &first, &second);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (timing) {
         SV_CUDA(cudaEventCreate(&e0));
@@ -565,6 +566,10 @@ static sv_status run_schedule(sv_state *s, const std::vector<Gate> &gates, size_
         SV_CUDA(cudaEventRecord(e0, s->stream));
     }
     sv_status st = SV_OK;
+    if (small) {
+        st = launch_small(s, gates, begin, end, &r->bytes);
+        for (size_t i = begin; i < end; ++i) r->max_k_used = std::max(r->max_k_used, gates[i].k);
+    }
     for (size_t i = 0; i < first.size() && st == SV_OK; ++i) {
         const Gate &g = gates[first[i]];
         if (second[i] >= 0) {
@@ -583,7 +588,7 @@ static sv_status run_schedule(sv_state *s, const std::vector<Gate> &gates, size_
         if (kind == PASS_TENSOR_CORE) ++r->tc_passes;
         r->max_k_used = std::max(r->max_k_used, g.k);
     }
-    r->passes += first.size();
+    r->passes += small ? end - begin : first.size();
     if (timing) {
         cudaError_t e = cudaEventRecord(e1, s->stream);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);

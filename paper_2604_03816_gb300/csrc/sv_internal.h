@@ -172,7 +172,12 @@ namespace svi {
 sv_status launch_apply(sv_state *s, const Gate &g, uint64_t *bytes = nullptr, int *kind = nullptr);
 // Structure-aware pass (apply_struct.cu): is it preferred over the dense kernels, and run it.
 bool struct_preferred(const sv_state *s, const Structure &st);
-sv_status launch_apply_struct(sv_state *s, const Structure &st, uint64_t *bytes);
+sv_status launch_apply_struct(sv_state *s, const Structure &st);
+uint64_t struct_bytes(const sv_state *s, const Structure &st);   // 2 s per amplitude it touches
+// States of up to 12 qubits without kernel-selection flags: gates [begin, end) in as few
+// launches as their matrices allow (apply_small.cu); *bytes is added to as by launch_apply.
+bool small_state(const sv_state *s);
+sv_status launch_small(sv_state *s, const std::vector<Gate> &gates, size_t begin, size_t end, uint64_t *bytes);
 bool tc_eligible(const sv_state *s, const Gate &g);        // apply_tc.cu
 sv_status launch_apply_tc(sv_state *s, const Gate &g);
 bool tc64_eligible(const sv_state *s, const Gate &g);      // apply_tc64.cu
