@@ -180,10 +180,6 @@ __device__ __forceinline__ double combine_levels(float f0, float f1, float f2, f
 // has targets among tile bits 0..2 and takes members in the lane's XOR
 // order; otherwise no permutation code at all.  The pipelines count tiles (j: raw stage,
 // output staging) and MMA subtiles (js = j SUB + sub: A and D buffers, row exponents).
-// 16-byte elements: the 128-byte swizzle XORs the 16-byte chunk (index bits 0-2) with the
-// 128-byte row within each 1 KiB (index bits 3-5); linear over XOR, its own inverse.
-__device__ __forceinline__ uint32_t swz128_16(uint32_t f) { return f ^ ((f >> 3) & 7u); }
-
 // SW: tiles move by 2-D tensor-map copies with the 128-byte swizzle and the roles address
 // them through it, so a warp's lanes reach different banks whatever the targets (no XOR
 // member order: XP = false).  The swizzle is applied to the group base and the target

@@ -193,6 +193,10 @@ __device__ __forceinline__ uint32_t swz128(uint32_t f) {
     return f ^ ((f >> 3) & 0xEu);
 }
 
+// 16-byte elements: the 128-byte swizzle XORs the 16-byte chunk (index bits 0-2) with the
+// 128-byte row within each 1 KiB (index bits 3-5); linear over XOR, its own inverse.
+__device__ __forceinline__ uint32_t swz128_16(uint32_t f) { return f ^ ((f >> 3) & 7u); }
+
 // Tile addressing for the warp that moves a tile: lane i (< 2^h) owns segment i of every
 // tile, whose offset from the tile's base it computes once; the tile base deposits the
 // tile index around the h high target bits.  The high-target positions live in

@@ -12,43 +12,10 @@
 #include <type_traits>
 
 #include "ptx.cuh"
+#include "reduce.cuh"
 #include "sv_internal.h"
 
 namespace svk {
-
-constexpr int RED_THREADS = 256;
-
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// Block-wide sum; result valid in thread 0.
-__device__ __forceinline__ double block_sum(double v) {
-    __shared__ double ws[RED_THREADS / 32];
-    v = warp_sum(v);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) ws[w] = v;
-    __syncthreads();
-    double r = 0.0;
-    if (w == 0) {
-        r = lane < RED_THREADS / 32 ? ws[lane] : 0.0;
-        r = warp_sum(r);
-    }
-    __syncthreads();
-    return r;
-}
-
-// |alpha|^2 in the state's precision: fl(fl(x*x) + fl(y*y)) with round-to-nearest and
-// no contraction, one fixed formula shared by probs, norm and top-k (so that a host
-// computing the same IEEE operations takes the same top-k decisions).
-__device__ __forceinline__ float prob_of(float x, float y) {
-    return __fadd_rn(__fmul_rn(x, x), __fmul_rn(y, y));
-}
-__device__ __forceinline__ double prob_of(double x, double y) {
-    return __dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y));
-}
 
 // ---------------------------------------------------------------- norm
 
@@ -176,12 +143,12 @@ __global__ void expect_kernel(const __grid_constant__ ExpectArgs a, const void *
     if (threadIdx.x == 0) partial[blockIdx.x] = r;
 }
 
-// complex64, up to NT terms of one X-part: per term FP32 partial sums over runs of eight
-// elements (pairs when x != 0), one FP64 step per run and term.  With s_t(k) = (-1)^{|k &
-// z_t|} and cc_t = ccr_t + i cci_t, a term contributes ccr_t sum_k s_t(k) |psi_k|^2 when
-// x = 0, and for x != 0, per pair (k, k2 = k ^ x) with bit hb of k clear and
-// c = conj(psi_k2) psi_k = re + i im:  ccr_t (s_t(k) + s_t(k2)) re - cci_t (s_t(k) - s_t(k2)) im.
-template <int NT, bool PAIRS>
+// complex64, up to NT terms of one X-part x != 0: per term FP32 partial sums over runs of
+// eight pairs, one FP64 step per run and term.  With s_t(k) = (-1)^{|k & z_t|} and
+// cc_t = ccr_t + i cci_t, the pair (k, k2 = k ^ x) with bit hb of k clear and
+// c = conj(psi_k2) psi_k = re + i im contributes ccr_t (s_t(k) + s_t(k2)) re - cci_t (s_t(k) -
+// s_t(k2)) im.
+template <int NT>
 __global__ void expect_c64(const __grid_constant__ ExpectArgs a, const float2 *__restrict__ psi,
                            double *partial) {
     double A[NT], B[NT];
@@ -197,23 +164,15 @@ __global__ void expect_c64(const __grid_constant__ ExpectArgs a, const float2 *_
         for (int r = 0; r < 8; ++r) {
             const unsigned long long i = i0 + r * stride;
             if (i >= a.npairs) break;
-            if constexpr (!PAIRS) {
-                const float2 v = psi[i];
-                const float pr = prob_of(v.x, v.y);
+            const unsigned long long k = insert_zero64(i, (uint32_t)a.hb), k2 = k ^ a.x;
+            const float2 p = psi[k], q = psi[k2];
+            const float re = __fadd_rn(__fmul_rn(q.x, p.x), __fmul_rn(q.y, p.y));
+            const float im = __fsub_rn(__fmul_rn(q.x, p.y), __fmul_rn(q.y, p.x));
 #pragma unroll
-                for (int t = 0; t < NT; ++t)
-                    sa[t] = __fadd_rn(sa[t], (__popcll(i & a.z[t]) & 1) ? -pr : pr);
-            } else {
-                const unsigned long long k = insert_zero64(i, (uint32_t)a.hb), k2 = k ^ a.x;
-                const float2 p = psi[k], q = psi[k2];
-                const float re = __fadd_rn(__fmul_rn(q.x, p.x), __fmul_rn(q.y, p.y));
-                const float im = __fsub_rn(__fmul_rn(q.x, p.y), __fmul_rn(q.y, p.x));
-#pragma unroll
-                for (int t = 0; t < NT; ++t) {
-                    const bool s1 = __popcll(k & a.z[t]) & 1, s2 = __popcll(k2 & a.z[t]) & 1;
-                    if (s1 == s2) sa[t] = __fadd_rn(sa[t], s1 ? -2.f * re : 2.f * re);
-                    else sb[t] = __fadd_rn(sb[t], s1 ? -2.f * im : 2.f * im);
-                }
+            for (int t = 0; t < NT; ++t) {
+                const bool s1 = __popcll(k & a.z[t]) & 1, s2 = __popcll(k2 & a.z[t]) & 1;
+                if (s1 == s2) sa[t] = __fadd_rn(sa[t], s1 ? -2.f * re : 2.f * re);
+                else sb[t] = __fadd_rn(sb[t], s1 ? -2.f * im : 2.f * im);
             }
         }
 #pragma unroll
@@ -488,68 +447,46 @@ sv_status launch_density_probs(sv_state *s, void *dev_out) {
     return SV_OK;
 }
 
-sv_status launch_expect(sv_state *s, const uint64_t *x, const uint64_t *z, const double *c,
-                        size_t nterms, double *host_out) {
-    // group terms by X-part; each launch handles up to EXP_MAX_TERMS terms of one group
-    std::vector<size_t> order(nterms);
-    for (size_t i = 0; i < nterms; ++i) order[i] = i;
-    std::stable_sort(order.begin(), order.end(), [&](size_t a, size_t b) { return x[a] < x[b]; });
-    double *partial = reinterpret_cast<double *>(s->ws + WS_PARTIAL);
-    double *results = reinterpret_cast<double *>(s->ws + WS_RESULT);
-    const int nb = red_blocks(s);
-    double total = 0.0;
-    size_t i = 0;
-    while (i < nterms) {
-        int nres = 0;
-        while (i < nterms && nres < 64) {
-            svk::ExpectArgs a;
-            std::memset(&a, 0, sizeof(a));
-            a.x = x[order[i]];
-            a.nterms = 0;
-            while (i < nterms && x[order[i]] == a.x && a.nterms < svk::EXP_MAX_TERMS) {
-                const size_t t = order[i++];
-                const int y = __builtin_popcountll(a.x & z[t]) & 3;   // i^y
-                const double re[4] = {1, 0, -1, 0}, im[4] = {0, 1, 0, -1};
-                a.z[a.nterms] = z[t];
-                a.ccr[a.nterms] = c[t] * re[y];
-                a.cci[a.nterms] = c[t] * im[y];
-                ++a.nterms;
-            }
-            if (a.x == 0) {
-                a.hb = 0;
-                a.npairs = 1ull << s->n;
-            } else {
-                a.hb = 63 - __builtin_clzll(a.x);
-                a.npairs = 1ull << (s->n - 1);
-            }
-            if (s->dtype == SV_C64) {
-                const float2 *v = reinterpret_cast<const float2 *>(s->buf);
-                const bool pr = a.x != 0;
-                switch (a.nterms) {
-                    case 1: pr ? svk::expect_c64<1, true><<<nb, svk::RED_THREADS, 0, s->stream>>>(a, v, partial)
-                               : svk::expect_c64<1, false><<<nb, svk::RED_THREADS, 0, s->stream>>>(a, v, partial); break;
-                    case 2: pr ? svk::expect_c64<2, true><<<nb, svk::RED_THREADS, 0, s->stream>>>(a, v, partial)
-                               : svk::expect_c64<2, false><<<nb, svk::RED_THREADS, 0, s->stream>>>(a, v, partial); break;
-                    case 3: pr ? svk::expect_c64<3, true><<<nb, svk::RED_THREADS, 0, s->stream>>>(a, v, partial)
-                               : svk::expect_c64<3, false><<<nb, svk::RED_THREADS, 0, s->stream>>>(a, v, partial); break;
-                    case 4: pr ? svk::expect_c64<4, true><<<nb, svk::RED_THREADS, 0, s->stream>>>(a, v, partial)
-                               : svk::expect_c64<4, false><<<nb, svk::RED_THREADS, 0, s->stream>>>(a, v, partial); break;
-                    default: svk::expect_kernel<float><<<nb, svk::RED_THREADS, 0, s->stream>>>(a, s->buf, partial);
-                }
-            } else
-                svk::expect_kernel<double><<<nb, svk::RED_THREADS, 0, s->stream>>>(a, s->buf, partial);
-            SV_CUDA(cudaGetLastError());
-            svk::sum_partials<<<1, svk::RED_THREADS, 0, s->stream>>>(partial, nb, results + nres);
-            SV_CUDA(cudaGetLastError());
-            ++nres;
-        }
-        double h[64];
-        SV_CUDA(cudaMemcpyAsync(h, results, sizeof(double) * nres, cudaMemcpyDeviceToHost, s->stream));
-        SV_CUDA(cudaStreamSynchronize(s->stream));
-        for (int r = 0; r < nres; ++r) total += h[r];
-    }
-    *host_out = total;
+sv_status enqueue_sum(sv_state *s, int n, double *dev_out) {
+    svk::sum_partials<<<1, svk::RED_THREADS, 0, s->stream>>>(reinterpret_cast<double *>(s->ws + WS_PARTIAL), n,
+                                                             dev_out);
+    SV_CUDA(cudaGetLastError());
     return SV_OK;
+}
+
+// One X-part's terms (at most 32) by the general kernels, the sum into *dev_out.
+sv_status enqueue_expect_group(sv_state *s, uint64_t x, const uint64_t *z, const double *c, int nterms,
+                               double *dev_out) {
+    double *partial = reinterpret_cast<double *>(s->ws + WS_PARTIAL);
+    const int nb = red_blocks(s);
+    svk::ExpectArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.x = x;
+    a.nterms = nterms;
+    for (int t = 0; t < nterms; ++t) {
+        const int y = __builtin_popcountll(x & z[t]) & 3;   // i^y
+        const double re[4] = {1, 0, -1, 0}, im[4] = {0, 1, 0, -1};
+        a.z[t] = z[t];
+        a.ccr[t] = c[t] * re[y];
+        a.cci[t] = c[t] * im[y];
+    }
+    a.hb = x ? 63 - __builtin_clzll(x) : 0;
+    a.npairs = x ? 1ull << (s->n - 1) : 1ull << s->n;
+    if (s->dtype == SV_C64 && x != 0 && nterms <= 4) {
+        const float2 *v = reinterpret_cast<const float2 *>(s->buf);
+        switch (nterms) {
+            case 1: svk::expect_c64<1><<<nb, svk::RED_THREADS, 0, s->stream>>>(a, v, partial); break;
+            case 2: svk::expect_c64<2><<<nb, svk::RED_THREADS, 0, s->stream>>>(a, v, partial); break;
+            case 3: svk::expect_c64<3><<<nb, svk::RED_THREADS, 0, s->stream>>>(a, v, partial); break;
+            default: svk::expect_c64<4><<<nb, svk::RED_THREADS, 0, s->stream>>>(a, v, partial);
+        }
+    } else if (s->dtype == SV_C64) {
+        svk::expect_kernel<float><<<nb, svk::RED_THREADS, 0, s->stream>>>(a, s->buf, partial);
+    } else {
+        svk::expect_kernel<double><<<nb, svk::RED_THREADS, 0, s->stream>>>(a, s->buf, partial);
+    }
+    SV_CUDA(cudaGetLastError());
+    return enqueue_sum(s, nb, dev_out);
 }
 
 // Enqueue the top-64 search and asynchronous copies of the 64 (p, index) pairs, best

@@ -191,6 +191,9 @@ sv_status launch_probs(sv_state *s, void *dev_out);
 sv_status launch_density_probs(sv_state *s, void *dev_out);   // Re v[x + 2^(n/2) x]
 sv_status launch_expect(sv_state *s, const uint64_t *x, const uint64_t *z, const double *c,
                         size_t nterms, double *host_out);
+sv_status enqueue_sum(sv_state *s, int n, double *dev_out);   // of the first n block partials
+sv_status enqueue_expect_group(sv_state *s, uint64_t x, const uint64_t *z, const double *c, int nterms,
+                               double *dev_out);
 sv_status launch_topk(sv_state *s, uint32_t k, uint64_t *idx, double *p);
 sv_status enqueue_topk(sv_state *s, double *host_p, unsigned long long *host_i);
 sv_status launch_widen(sv_state *s, const void *src_c64, void *dst_c128);
