@@ -173,7 +173,7 @@ sv_status launch_apply_t(sv_state *s, const svi::Gate &g) {
     const unsigned long long cap = (unsigned long long)blocks_per_sm * (unsigned long long)s->num_sms;
     const unsigned grid = (unsigned)std::min<unsigned long long>(p.ntiles, cap);
     const size_t bytes = size_t(1) << (p.L + p.h);
-    SV_CUDA(launch_pass(apply_tile<R, K>, grid, 256, bytes * sizeof(C), s->stream, a));
+    SV_CUDA(launch_pass(apply_tile<R, K>, dim3(grid), 256, bytes * sizeof(C), s->stream, a));
     return SV_OK;
 }
 

@@ -277,7 +277,7 @@ template <typename R, int VEC>
 static sv_status launch_diag_v(sv_state *s, const DiagArgs<R> &a) {
     static int per_sm = 0;
     const unsigned grid = grid_for(apply_diag<R, VEC>, &per_sm, s, (a.items + 3) / 4);
-    SV_CUDA(svk::launch_pass(apply_diag<R, VEC>, grid, 256, 0, s->stream, a));
+    SV_CUDA(svk::launch_pass(apply_diag<R, VEC>, dim3(grid), 256, 0, s->stream, a));
     return SV_OK;
 }
 
@@ -337,7 +337,7 @@ static sv_status launch_mono(sv_state *s, const svi::Structure &st) {
     a.sp = make_spread(st, true);
     if (moved == 0) return SV_OK;
     const unsigned grid = grid_for(apply_mono<R, K>, &per_sm, s, (a.count + mono_ilp<R, K>() - 1) / mono_ilp<R, K>());
-    SV_CUDA(svk::launch_pass(apply_mono<R, K>, grid, 256, 0, s->stream, a));
+    SV_CUDA(svk::launch_pass(apply_mono<R, K>, dim3(grid), 256, 0, s->stream, a));
     return SV_OK;
 }
 
@@ -360,7 +360,7 @@ static sv_status launch_ctrl(sv_state *s, const svi::Structure &st) {
     a.count = 1ull << (s->n - st.nctrl - K);
     a.sp = make_spread(st, true);
     const unsigned grid = grid_for(apply_ctrl<R, K>, &per_sm, s, a.count);
-    SV_CUDA(svk::launch_pass(apply_ctrl<R, K>, grid, 256, 0, s->stream, a));
+    SV_CUDA(svk::launch_pass(apply_ctrl<R, K>, dim3(grid), 256, 0, s->stream, a));
     return SV_OK;
 }
 

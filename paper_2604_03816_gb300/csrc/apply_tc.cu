@@ -805,11 +805,11 @@ sv_status launch_tc_t(sv_state *s, const svi::Gate &g) {
     cudaError_t e = cudaSuccess;
     // with eight worker warps per role the permutation costs less than even 2-way conflicts
     if (swz) {
-        if constexpr (K == 5) e = launch_pass(apply_tc<K, false, 2, false, true>, grid, S2::THREADS, S2::SMEM, s->stream, a);
+        if constexpr (K == 5) e = launch_pass(apply_tc<K, false, 2, false, true>, dim3(grid), S2::THREADS, S2::SMEM, s->stream, a);
     } else if (a.xt >= 1) {
-        e = launch_pass(apply_tc<K, true, 1>, grid, S::THREADS, S::SMEM, s->stream, a);
+        e = launch_pass(apply_tc<K, true, 1>, dim3(grid), S::THREADS, S::SMEM, s->stream, a);
     } else {
-        e = launch_pass(apply_tc<K, false, 1>, grid, S::THREADS, S::SMEM, s->stream, a);
+        e = launch_pass(apply_tc<K, false, 1>, dim3(grid), S::THREADS, S::SMEM, s->stream, a);
     }
     SV_CUDA(e);
     return SV_OK;
@@ -885,7 +885,7 @@ sv_status launch_tc_batch(const sv_batch_launch &L) {
     a.kin = L.k;
     a.jw = jw;
     const unsigned grid = (unsigned)std::min<unsigned long long>(a.ntiles, (unsigned long long)L.num_sms);
-    SV_CUDA(launch_pass(apply_tc<5, false, 1, true, true>, grid, S::THREADS, S::SMEM, L.stream, a));
+    SV_CUDA(launch_pass(apply_tc<5, false, 1, true, true>, dim3(grid), S::THREADS, S::SMEM, L.stream, a));
     return SV_OK;
 }
 

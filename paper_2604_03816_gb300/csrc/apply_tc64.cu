@@ -550,9 +550,9 @@ sv_status launch_tc64(sv_state *s, const svi::Gate &g0) {
     const unsigned grid = (unsigned)std::min<unsigned long long>(p.ntiles, (unsigned long long)s->num_sms);
     // two targets in bits 0..2 (4-way conflicts and worse) take the swizzled staging; one
     // target there leaves 2-way conflicts, cheaper than either remedy
-    SV_CUDA(swz    ? launch_pass(apply_tc64<false, 1, true>, grid, S::THREADS, S::SMEM, s->stream, a)
-            : wide ? launch_pass(apply_tc64<false, 2>, grid, S2::THREADS, S2::SMEM, s->stream, a)
-                   : launch_pass(apply_tc64<false, 1>, grid, S::THREADS, S::SMEM, s->stream, a));
+    SV_CUDA(swz    ? launch_pass(apply_tc64<false, 1, true>, dim3(grid), S::THREADS, S::SMEM, s->stream, a)
+            : wide ? launch_pass(apply_tc64<false, 2>, dim3(grid), S2::THREADS, S2::SMEM, s->stream, a)
+                   : launch_pass(apply_tc64<false, 1>, dim3(grid), S::THREADS, S::SMEM, s->stream, a));
     return SV_OK;
 }
 

@@ -88,6 +88,8 @@ struct ZTableArgs {
 // w[j][k] = sum of c_t (-1)^{|k & z_t|} over the terms with z_hi = zc[j] (and z_lo != 0, or
 // z = 0); one entry per thread.
 __global__ void z_table(const __grid_constant__ ZTableArgs a) {
+    svk::pass_trigger();
+    svk::pass_wait();
     const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= (1u << a.t)) return;
     const unsigned long long zc = a.zc[blockIdx.y];
@@ -131,6 +133,8 @@ __global__ void __launch_bounds__(THREADS, NC >= 2 ? 1 : 2) z_sum(const __grid_c
     for (uint32_t e = 0; e < E; ++e) U[e].clear();
 #pragma unroll
     for (uint32_t e = 0; e < (NC ? NC * E : 1u); ++e) X[e].clear();
+    svk::pass_trigger();
+    svk::pass_wait();
     double hi_acc = 0.0;
     V next[NV];
     auto load = [&](unsigned long long tile) {
@@ -315,6 +319,8 @@ __global__ void __launch_bounds__(THREADS, 2) x_sum(const __grid_constant__ XArg
     const unsigned long long my_z = lane < nterms ? a.term[lane].z : 0ull;
     svk::SegLanes sl;
     sl.init(a.L, a.h, a.hi, lane);
+    svk::pass_trigger();
+    svk::pass_wait();
     __syncthreads();
     constexpr uint32_t ROW = 128u / (uint32_t)sizeof(C);       // amplitudes per 128-byte row
     auto load = [&](unsigned long long t, uint32_t s) {        // warp 0
@@ -437,7 +443,7 @@ struct Partials {
     // a slot for one more sum
     sv_status slot(double **out) {
         const sv_status st = nres >= 60 ? collect() : SV_OK;
-        *out = reinterpret_cast<double *>(s->ws + WS_RESULT) + nres++;
+        *out = mail_results(s) + nres++;
         return st;
     }
     sv_status fold() {
@@ -452,8 +458,8 @@ struct Partials {
     sv_status collect() {
         double h[64];
         if (!nres) return SV_OK;
-        SV_CUDA(cudaMemcpyAsync(h, s->ws + WS_RESULT, sizeof(double) * nres, cudaMemcpyDeviceToHost, s->stream));
-        SV_CUDA(cudaStreamSynchronize(s->stream));
+        const sv_status st = read_results(s, h, sizeof(double) * nres);
+        if (st != SV_OK) return st;
         for (int r = 0; r < nres; ++r) total += h[r];
         nres = 0;
         return SV_OK;
@@ -511,16 +517,16 @@ sv_status z_group(sv_state *s, Partials &P, const Term *t, size_t n) {
             if (st != SV_OK) return st;
             a.partial = P.part();
             if (a.low || nc) {
-                z_table<<<dim3((unsigned)(((1u << T) + 127) / 128), ta.ntab), 128, 0, s->stream>>>(ta);
-                SV_CUDA(cudaGetLastError());
+                SV_CUDA(svk::launch_pass(z_table, dim3((unsigned)(((1u << T) + 127) / 128), ta.ntab), 128, 0, s->stream, ta));
             }
+            cudaError_t e = cudaSuccess;
             switch (nc) {
-                case 0: z_sum<R, 0><<<nb, THREADS, 0, s->stream>>>(a); break;
-                case 1: z_sum<R, 1><<<nb, THREADS, 0, s->stream>>>(a); break;
-                case 2: z_sum<R, 2><<<nb, THREADS, 0, s->stream>>>(a); break;
-                default: z_sum<R, 3><<<nb, THREADS, 0, s->stream>>>(a); break;
+                case 0: e = svk::launch_pass(z_sum<R, 0>, dim3(nb), THREADS, 0, s->stream, a); break;
+                case 1: e = svk::launch_pass(z_sum<R, 1>, dim3(nb), THREADS, 0, s->stream, a); break;
+                case 2: e = svk::launch_pass(z_sum<R, 2>, dim3(nb), THREADS, 0, s->stream, a); break;
+                default: e = svk::launch_pass(z_sum<R, 3>, dim3(nb), THREADS, 0, s->stream, a); break;
             }
-            SV_CUDA(cudaGetLastError());
+            SV_CUDA(e);
             P.used += nb;
             done += nc;
             first = false;
@@ -631,8 +637,7 @@ sv_status x_pass(sv_state *s, Partials &P, const std::vector<Term> &t, std::vect
         err = cudaFuncSetAttribute(x_sum<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     });
     SV_CUDA(err);
-    x_sum<R><<<nb, THREADS, smem, s->stream>>>(a);
-    SV_CUDA(cudaGetLastError());
+    SV_CUDA(svk::launch_pass(x_sum<R>, dim3(nb), THREADS, smem, s->stream, a));
     P.used += nb;
     return SV_OK;
 }

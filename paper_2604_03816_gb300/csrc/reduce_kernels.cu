@@ -19,7 +19,11 @@ namespace svk {
 
 // ---------------------------------------------------------------- norm
 
-__global__ void norm_c64(const float4 *__restrict__ v, unsigned long long nvec, double *partial) {
+// err, mail: a single block's sum is the result; the error word goes with it (else null).
+__global__ void norm_c64(const float4 *__restrict__ v, unsigned long long nvec, double *partial, const int *err,
+                         int *mail) {
+    pass_trigger();
+    pass_wait();
     double acc = 0.0;
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
     unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -38,10 +42,16 @@ __global__ void norm_c64(const float4 *__restrict__ v, unsigned long long nvec, 
         acc += (double)__fadd_rn(prob_of(a.x, a.y), prob_of(a.z, a.w));
     }
     const double r = block_sum(acc);
-    if (threadIdx.x == 0) partial[blockIdx.x] = r;
+    if (threadIdx.x == 0) {
+        partial[blockIdx.x] = r;
+        if (mail) *mail = *err;
+    }
 }
 
-__global__ void norm_c128(const double2 *__restrict__ v, unsigned long long n, double *partial) {
+__global__ void norm_c128(const double2 *__restrict__ v, unsigned long long n, double *partial, const int *err,
+                          int *mail) {
+    pass_trigger();
+    pass_wait();
     double acc = 0.0;
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
     unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -51,20 +61,30 @@ __global__ void norm_c128(const double2 *__restrict__ v, unsigned long long n, d
     }
     for (; i < n; i += stride) acc += prob_of(v[i].x, v[i].y);
     const double r = block_sum(acc);
-    if (threadIdx.x == 0) partial[blockIdx.x] = r;
+    if (threadIdx.x == 0) {
+        partial[blockIdx.x] = r;
+        if (mail) *mail = *err;
+    }
 }
 
-// out[0] = sum of partial[0..n) in a fixed order (one block).
-__global__ void sum_partials(const double *partial, int n, double *out) {
+// out[0] = sum of partial[0..n) in a fixed order (one block); *mail = *err if given.
+__global__ void sum_partials(const double *partial, int n, double *out, const int *err, int *mail) {
+    pass_trigger();
+    pass_wait();
     double acc = 0.0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) acc += partial[i];
     const double r = block_sum(acc);
-    if (threadIdx.x == 0) out[0] = r;
+    if (threadIdx.x == 0) {
+        out[0] = r;
+        if (mail) *mail = *err;
+    }
 }
 
 // ---------------------------------------------------------------- probabilities
 
 __global__ void probs_c64(const float4 *__restrict__ v, unsigned long long nvec, float2 *out) {
+    pass_trigger();
+    pass_wait();
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
     for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < nvec;
          i += stride) {
@@ -74,6 +94,8 @@ __global__ void probs_c64(const float4 *__restrict__ v, unsigned long long nvec,
 }
 
 __global__ void probs_c128(const double2 *__restrict__ v, unsigned long long n, double *out) {
+    pass_trigger();
+    pass_wait();
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
     for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += stride)
@@ -188,207 +210,26 @@ __global__ void expect_c64(const __grid_constant__ ExpectArgs a, const float2 *_
     if (threadIdx.x == 0) partial[blockIdx.x] = r;
 }
 
-// ---------------------------------------------------------------- top-k
-
-// (p, idx) order: larger p first, then smaller index.
-template <typename P>
-__device__ __forceinline__ bool better(P pa, unsigned long long ia, P pb, unsigned long long ib) {
-    return pa > pb || (pa == pb && ia < ib);
-}
-
-// Keys of the top-k lists.  complex64 probabilities are FP32 values, compared in FP32 (the
-// same decisions as on their exact FP64 widenings).  FP64 probabilities are compared as
-// their IEEE bit patterns, which order non-negative doubles like their values, in 64-bit
-// integer arithmetic: a warp-wide FP64 compare costs tens of cycles on this GPU.
-template <typename P> __device__ __forceinline__ P empty_key();
-template <> __device__ __forceinline__ float empty_key<float>() { return -1.f; }
-template <> __device__ __forceinline__ unsigned long long empty_key<unsigned long long>() { return 0ull; }
-
-__device__ __forceinline__ unsigned long long key_of(double p) {   // p >= 0
-    return (unsigned long long)__double_as_longlong(p);
-}
-__device__ __forceinline__ double value_of(unsigned long long k) { return __longlong_as_double((long long)k); }
-__device__ __forceinline__ double value_of(float k) { return (double)k; }
-
-// One warp's 64 entries, two per lane, plus the current worst.  Empty entries hold
-// (empty_key, ~0): they lose to every real entry.
-template <typename P>
-struct TopList {
-    P p0, p1;
-    unsigned long long i0, i1;
-    P wp;
-    unsigned long long wi;
-    int wl, ws;    // lane and slot of the worst entry
-
-    __device__ void init() {
-        p0 = p1 = empty_key<P>();
-        i0 = i1 = ~0ull;
-        find_worst();
-    }
-    __device__ void find_worst() {
-        const int lane = threadIdx.x & 31;
-        // this lane's worse entry
-        bool second = better(p0, i0, p1, i1);
-        P p = second ? p1 : p0;
-        unsigned long long ix = second ? i1 : i0;
-        int l = lane, s = second ? 1 : 0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const P op = __shfl_xor_sync(0xffffffffu, p, o);
-            const unsigned long long oi = __shfl_xor_sync(0xffffffffu, ix, o);
-            const int ol = __shfl_xor_sync(0xffffffffu, l, o);
-            const int os = __shfl_xor_sync(0xffffffffu, s, o);
-            if (better(p, ix, op, oi) || (p == op && ix == oi && (ol < l || (ol == l && os < s)))) {
-                p = op; ix = oi; l = ol; s = os;
-            }
-        }
-        wp = p; wi = ix; wl = l; ws = s;
-    }
-    // Offer one candidate per lane; all lanes of the warp must call.
-    __device__ void offer(P p, unsigned long long ix, bool valid) {
-        const int lane = threadIdx.x & 31;
-        unsigned mask = __ballot_sync(0xffffffffu, valid && better(p, ix, wp, wi));
-        while (mask) {
-            const int src = __ffs(mask) - 1;
-            mask &= mask - 1;
-            const P cp = __shfl_sync(0xffffffffu, p, src);
-            const unsigned long long ci = __shfl_sync(0xffffffffu, ix, src);
-            if (!better(cp, ci, wp, wi)) continue;     // uniform across the warp
-            if (lane == wl) {
-                if (ws == 0) { p0 = cp; i0 = ci; } else { p1 = cp; i1 = ci; }
-            }
-            find_worst();
-        }
-    }
-};
-
-// Pass 1: each warp scans a contiguous chunk (a multiple of 256 amplitudes), eight
-// amplitudes per lane per step from independent 16-byte loads; a step is offered to the
-// warp's list only if some lane holds a probability not below the list's current worst.
-// The block's warps then merge their lists, and the block writes 64 candidates.
-template <typename R>
-__global__ void __launch_bounds__(256) topk_pass1(const void *psi_, unsigned long long N,
-                                                  unsigned long long chunk, double *cand_p,
-                                                  unsigned long long *cand_i) {
-    using Key = typename std::conditional<sizeof(R) == 4, float, unsigned long long>::type;
-    __shared__ Key lp[8][64];
-    __shared__ unsigned long long li[8][64];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const unsigned long long warp = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    TopList<Key> L;
-    L.init();
-    const unsigned long long lo = warp * chunk, hi = min(N, lo + chunk);
-    for (unsigned long long b = lo; b < hi; b += 256) {
-        Key p[8];
-        unsigned long long k[8];
-        bool ok[8];
-        if constexpr (sizeof(R) == 4) {
-            // four float4 loads: amplitudes b + 2 (lane + 32 j) + {0, 1}
-            const float4 *v4 = reinterpret_cast<const float4 *>(psi_);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const unsigned long long k0 = b + 2ull * (lane + 32 * j);
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (k0 < hi) v = v4[k0 >> 1];
-                k[2 * j] = k0;
-                k[2 * j + 1] = k0 + 1;
-                ok[2 * j] = k0 < hi;
-                ok[2 * j + 1] = k0 + 1 < hi;
-                p[2 * j] = ok[2 * j] ? prob_of(v.x, v.y) : empty_key<Key>();
-                p[2 * j + 1] = ok[2 * j + 1] ? prob_of(v.z, v.w) : empty_key<Key>();
-            }
-        } else {
-            const double2 *v2 = reinterpret_cast<const double2 *>(psi_);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const unsigned long long k0 = b + lane + 32ull * j;
-                double2 v = make_double2(0.0, 0.0);
-                if (k0 < hi) v = v2[k0];
-                k[j] = k0;
-                ok[j] = k0 < hi;
-                p[j] = ok[j] ? key_of(prob_of(v.x, v.y)) : empty_key<Key>();
-            }
-        }
-        Key mx = p[0];
-#pragma unroll
-        for (int j = 1; j < 8; ++j) mx = mx > p[j] ? mx : p[j];
-        if (!__any_sync(0xffffffffu, mx >= L.wp)) continue;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) L.offer(p[j], k[j], ok[j]);
-    }
-    // merge the block's eight lists in warp 0
-    lp[w][2 * lane] = L.p0; li[w][2 * lane] = L.i0;
-    lp[w][2 * lane + 1] = L.p1; li[w][2 * lane + 1] = L.i1;
-    __syncthreads();
-    if (w == 0) {
-        for (int o = 1; o < 8; ++o)
-            for (int h = 0; h < 2; ++h) {
-                const unsigned long long ci = li[o][32 * h + lane];
-                L.offer(lp[o][32 * h + lane], ci, ci != ~0ull);
-            }
-        // candidates as doubles; empty entries as -1
-        const unsigned long long base = (unsigned long long)blockIdx.x * 64;
-        cand_p[base + 2 * lane] = L.i0 == ~0ull ? -1.0 : value_of(L.p0);
-        cand_i[base + 2 * lane] = L.i0;
-        cand_p[base + 2 * lane + 1] = L.i1 == ~0ull ? -1.0 : value_of(L.p1);
-        cand_i[base + 2 * lane + 1] = L.i1;
-    }
-}
-
-// Pass 2 (one block of 32 warps): each warp merges a strided share of the m candidates,
-// warp 0 merges the 32 lists and writes the best 64, sorted.
-__global__ void __launch_bounds__(1024) topk_pass2(const double *cand_p, const unsigned long long *cand_i,
-                                                   unsigned long long m, double *out_p,
-                                                   unsigned long long *out_i) {
-    __shared__ unsigned long long sp[32][64];
-    __shared__ unsigned long long si[32][64];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    TopList<unsigned long long> L;
-    L.init();
-    for (unsigned long long b = (unsigned long long)w * 32; b < m; b += 32ull * 32) {
-        const unsigned long long j = b + lane;
-        const bool ok = j < m;
-        const unsigned long long kb = ok ? (unsigned long long)__double_as_longlong(cand_p[j]) : 0ull;
-        const bool real = ok && !(kb >> 63);              // empty entries are -1
-        L.offer(real ? kb : 0ull, real ? cand_i[j] : ~0ull, real);
-    }
-    sp[w][2 * lane] = L.p0; si[w][2 * lane] = L.i0;
-    sp[w][2 * lane + 1] = L.p1; si[w][2 * lane + 1] = L.i1;
-    __syncthreads();
-    if (w != 0) return;
-    for (int o = 1; o < 32; ++o)
-        for (int h = 0; h < 2; ++h) {
-            const unsigned long long ci = si[o][32 * h + lane];
-            L.offer(sp[o][32 * h + lane], ci, ci != ~0ull);
-        }
-    sp[0][2 * lane] = L.p0; si[0][2 * lane] = L.i0;
-    sp[0][2 * lane + 1] = L.p1; si[0][2 * lane + 1] = L.i1;
-    __syncwarp();
-    if (lane == 0) {
-        unsigned long long *qp = sp[0];
-        unsigned long long *qi = si[0];
-        for (int a = 1; a < 64; ++a) {          // insertion sort, best first
-            const unsigned long long p = qp[a];
-            const unsigned long long ix = qi[a];
-            int b = a - 1;
-            while (b >= 0 && better(p, ix, qp[b], qi[b])) {
-                qp[b + 1] = qp[b]; qi[b + 1] = qi[b];
-                --b;
-            }
-            qp[b + 1] = p; qi[b + 1] = ix;
-        }
-        for (int a = 0; a < 64; ++a) {
-            out_p[a] = qi[a] == ~0ull ? -1.0 : value_of(qp[a]);
-            out_i[a] = qi[a];
-        }
-    }
-}
-
 // ---------------------------------------------------------------- init helpers
 
 __global__ void set_amp_one(void *psi, unsigned long long x, int is_c128) {
     if (is_c128) reinterpret_cast<double2 *>(psi)[x] = make_double2(1.0, 0.0);
     else reinterpret_cast<float2 *>(psi)[x] = make_float2(1.0f, 0.0f);
+}
+
+// |x> of a small state in one launch: 16-byte words, zero but for the amplitude of x.
+__global__ void set_basis_small(uint4 *psi, unsigned long long words, unsigned long long x, int is_c128) {
+    pass_trigger();
+    pass_wait();
+    const unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= words) return;
+    uint4 w = make_uint4(0, 0, 0, 0);
+    if (is_c128) {
+        if (i == x) w.y = (uint32_t)__double2hiint(1.0);
+    } else if (i == x >> 1) {
+        (x & 1 ? w.z : w.x) = __float_as_uint(1.f);
+    }
+    psi[i] = w;
 }
 
 __global__ void widen_kernel(const float2 *__restrict__ src, double2 *__restrict__ dst,
@@ -405,32 +246,39 @@ namespace svi {
 
 static int red_blocks(const sv_state *s) { return std::min(WS_NPARTIAL, s->num_sms * 8); }
 
+sv_status enqueue_sum(sv_state *s, int n, double *dev_out) {
+    SV_CUDA(svk::launch_pass(svk::sum_partials, dim3(1), svk::RED_THREADS, 0, s->stream,
+                             reinterpret_cast<double *>(s->ws + WS_PARTIAL), n, dev_out, device_error(s),
+                             mail_error(s)));
+    return SV_OK;
+}
+
 sv_status launch_norm(sv_state *s, double *dev_out) {
     double *partial = reinterpret_cast<double *>(s->ws + WS_PARTIAL);
     const unsigned long long N = 1ull << s->n;
-    const int nb = red_blocks(s);
+    // fixed by n, so the sum's order is; at least four 16-byte words per thread
+    const unsigned long long words = (N * (s->dtype == SV_C64 ? 8 : 16)) / 16;
+    const int nb = (int)std::min<unsigned long long>(red_blocks(s), std::max(1ull, words / (4 * svk::RED_THREADS)));
+    int *mail = nb == 1 ? mail_error(s) : nullptr;
+    if (nb == 1) partial = dev_out;
     if (s->dtype == SV_C64)
-        svk::norm_c64<<<nb, svk::RED_THREADS, 0, s->stream>>>(
-            reinterpret_cast<const float4 *>(s->buf), N / 2, partial);
+        SV_CUDA(svk::launch_pass(svk::norm_c64, dim3(nb), svk::RED_THREADS, 0, s->stream,
+                                 reinterpret_cast<const float4 *>(s->buf), N / 2, partial, device_error(s), mail));
     else
-        svk::norm_c128<<<nb, svk::RED_THREADS, 0, s->stream>>>(
-            reinterpret_cast<const double2 *>(s->buf), N, partial);
-    SV_CUDA(cudaGetLastError());
-    svk::sum_partials<<<1, svk::RED_THREADS, 0, s->stream>>>(partial, nb, dev_out);
-    SV_CUDA(cudaGetLastError());
-    return SV_OK;
+        SV_CUDA(svk::launch_pass(svk::norm_c128, dim3(nb), svk::RED_THREADS, 0, s->stream,
+                                 reinterpret_cast<const double2 *>(s->buf), N, partial, device_error(s), mail));
+    return nb == 1 ? SV_OK : enqueue_sum(s, nb, dev_out);
 }
 
 sv_status launch_probs(sv_state *s, void *dev_out) {
     const unsigned long long N = 1ull << s->n;
-    const int nb = s->num_sms * 8;
+    const int nb = (int)std::min<unsigned long long>(s->num_sms * 8, (N + 511) / 512);
     if (s->dtype == SV_C64)
-        svk::probs_c64<<<nb, 256, 0, s->stream>>>(reinterpret_cast<const float4 *>(s->buf), N / 2,
-                                                   reinterpret_cast<float2 *>(dev_out));
+        SV_CUDA(svk::launch_pass(svk::probs_c64, dim3(nb), 256, 0, s->stream, reinterpret_cast<const float4 *>(s->buf),
+                                 N / 2, reinterpret_cast<float2 *>(dev_out)));
     else
-        svk::probs_c128<<<nb, 256, 0, s->stream>>>(reinterpret_cast<const double2 *>(s->buf), N,
-                                                    reinterpret_cast<double *>(dev_out));
-    SV_CUDA(cudaGetLastError());
+        SV_CUDA(svk::launch_pass(svk::probs_c128, dim3(nb), 256, 0, s->stream,
+                                 reinterpret_cast<const double2 *>(s->buf), N, reinterpret_cast<double *>(dev_out)));
     return SV_OK;
 }
 
@@ -443,13 +291,6 @@ sv_status launch_density_probs(sv_state *s, void *dev_out) {
     else
         svk::density_diag<<<nb, 256, 0, s->stream>>>(reinterpret_cast<const double2 *>(s->buf), m,
                                                      reinterpret_cast<double *>(dev_out));
-    SV_CUDA(cudaGetLastError());
-    return SV_OK;
-}
-
-sv_status enqueue_sum(sv_state *s, int n, double *dev_out) {
-    svk::sum_partials<<<1, svk::RED_THREADS, 0, s->stream>>>(reinterpret_cast<double *>(s->ws + WS_PARTIAL), n,
-                                                             dev_out);
     SV_CUDA(cudaGetLastError());
     return SV_OK;
 }
@@ -487,47 +328,6 @@ sv_status enqueue_expect_group(sv_state *s, uint64_t x, const uint64_t *z, const
     }
     SV_CUDA(cudaGetLastError());
     return enqueue_sum(s, nb, dev_out);
-}
-
-// Enqueue the top-64 search and asynchronous copies of the 64 (p, index) pairs, best
-// first, into host_p / host_i (pinned memory for a truly asynchronous copy).
-sv_status enqueue_topk(sv_state *s, double *host_p, unsigned long long *host_i) {
-    const unsigned long long N = 1ull << s->n;
-    const int threads = 256, warps_per_block = threads / 32;
-    int blocks = std::min(s->num_sms * 4, TOPK_MAX_WARPS / warps_per_block);
-    unsigned long long nwarps = (unsigned long long)blocks * warps_per_block;
-    unsigned long long chunk = (N + nwarps - 1) / nwarps;
-    chunk = (chunk + 255) / 256 * 256;
-    double *cp = reinterpret_cast<double *>(s->ws + WS_TOPK);
-    unsigned long long *ci = reinterpret_cast<unsigned long long *>(s->ws + WS_TOPK) + TOPK_MAX_WARPS * 64;
-    double *op = reinterpret_cast<double *>(s->ws + WS_TOPK + WS_TOPK_BYTES);
-    unsigned long long *oi = reinterpret_cast<unsigned long long *>(op + 64);
-    if (s->dtype == SV_C64)
-        svk::topk_pass1<float><<<blocks, threads, 0, s->stream>>>(s->buf, N, chunk, cp, ci);
-    else
-        svk::topk_pass1<double><<<blocks, threads, 0, s->stream>>>(s->buf, N, chunk, cp, ci);
-    SV_CUDA(cudaGetLastError());
-    svk::topk_pass2<<<1, 1024, 0, s->stream>>>(cp, ci, (unsigned long long)blocks * 64, op, oi);
-    SV_CUDA(cudaGetLastError());
-    SV_CUDA(cudaMemcpyAsync(host_p, op, 64 * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
-    SV_CUDA(cudaMemcpyAsync(host_i, oi, 64 * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
-                            s->stream));
-    return SV_OK;
-}
-
-sv_status launch_topk(sv_state *s, uint32_t k, uint64_t *idx, double *p) {
-    const unsigned long long N = 1ull << s->n;
-    double hp[64];
-    unsigned long long hi[64];
-    sv_status st = enqueue_topk(s, hp, hi);
-    if (st != SV_OK) return st;
-    SV_CUDA(cudaStreamSynchronize(s->stream));
-    const uint32_t m = (uint32_t)std::min<unsigned long long>(k, N);
-    for (uint32_t j = 0; j < m; ++j) {
-        idx[j] = hi[j];
-        p[j] = hp[j];
-    }
-    return SV_OK;
 }
 
 // Enqueue sum_t coef[t] <P_t> for a raw device state into *out_dev, with block partials
@@ -585,7 +385,7 @@ sv_status enqueue_expect_sum(const void *psi, uint32_t n, sv_dtype dtype, const 
         SV_CUDA(cudaGetLastError());
     }
     svk::sum_partials<<<1, svk::RED_THREADS, 0, stream>>>(scratch, (int)(nbatches * nb_fixed),
-                                                          out_dev);
+                                                          out_dev, nullptr, nullptr);
     SV_CUDA(cudaGetLastError());
     return SV_OK;
 }
@@ -598,8 +398,19 @@ sv_status launch_widen(sv_state *s, const void *src_c64, void *dst_c128) {
     return SV_OK;
 }
 
-sv_status launch_set_one(sv_state *s, uint64_t x) {
-    svk::set_amp_one<<<1, 1, 0, s->stream>>>(s->buf, x, s->dtype == SV_C128);
+// The state becomes |x>.  Up to 16 qubits in one launch; larger states by a memset and a
+// one-amplitude kernel (the memset runs at copy speed).
+sv_status launch_set_basis(sv_state *s, uint64_t x) {
+    const int wide = s->dtype == SV_C128;
+    const unsigned long long bytes = (wide ? 16ull : 8ull) << s->n;
+    if (s->n <= 16) {
+        const unsigned long long words = bytes / 16;
+        SV_CUDA(svk::launch_pass(svk::set_basis_small, dim3((unsigned)((words + 255) / 256)), 256, 0, s->stream,
+                                 reinterpret_cast<uint4 *>(s->buf), words, (unsigned long long)x, wide));
+        return SV_OK;
+    }
+    SV_CUDA(cudaMemsetAsync(s->buf, 0, bytes, s->stream));
+    svk::set_amp_one<<<1, 1, 0, s->stream>>>(s->buf, x, wide);
     SV_CUDA(cudaGetLastError());
     return SV_OK;
 }

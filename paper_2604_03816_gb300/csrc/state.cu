@@ -24,16 +24,27 @@ void clear_error() { g_err.clear(); }
 static size_t elem_bytes(sv_dtype d) { return d == SV_C64 ? 8 : 16; }
 static size_t state_bytes(const sv_state *s) { return elem_bytes(s->dtype) << s->n; }
 
-sv_status check_device_error(sv_state *s) {
+static sv_status report_error(sv_state *s, int err) {
+    if (err == 0) return SV_OK;
+    SV_CUDA(cudaMemset(s->ws + WS_ERR, 0, sizeof(int)));
+    return set_error(SV_ERR_TIMEOUT, "a bounded device-side wait gave up (error word " +
+                                         std::to_string(err) + ")");
+}
+
+sv_status read_results(sv_state *s, void *dst, size_t bytes) {
     SV_CUDA(cudaStreamSynchronize(s->stream));
     int err = 0;
-    SV_CUDA(cudaMemcpy(&err, s->ws + WS_ERR, sizeof(int), cudaMemcpyDeviceToHost));
-    if (err != 0) {
-        SV_CUDA(cudaMemset(s->ws + WS_ERR, 0, sizeof(int)));
-        return set_error(SV_ERR_TIMEOUT, "a bounded device-side wait gave up (error word " +
-                                             std::to_string(err) + ")");
-    }
-    return SV_OK;
+    std::memcpy(&err, s->mail + WS_ERR, sizeof(int));
+    const sv_status st = report_error(s, err);
+    if (st == SV_OK) std::memcpy(dst, s->mail + WS_RESULT, bytes);
+    return st;
+}
+
+sv_status check_device_error(sv_state *s) {
+    int err = 0;
+    SV_CUDA(cudaMemcpyAsync(&err, s->ws + WS_ERR, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+    SV_CUDA(cudaStreamSynchronize(s->stream));
+    return report_error(s, err);
 }
 
 static sv_status validate_gate(const sv_gate *g, uint32_t n, const char *who) {
@@ -112,11 +123,8 @@ sv_status check_live(const sv_state *s, const char *who) {
 }
 
 static sv_status measure_norm(sv_state *s, double *out) {
-    double *res = reinterpret_cast<double *>(s->ws + WS_RESULT) + 63;
-    sv_status st = launch_norm(s, res);
-    if (st != SV_OK) return st;
-    SV_CUDA(cudaMemcpyAsync(out, res, sizeof(double), cudaMemcpyDeviceToHost, s->stream));
-    return check_device_error(s);
+    const sv_status st = launch_norm(s, mail_results(s));
+    return st != SV_OK ? st : read_results(s, out, sizeof(double));
 }
 
 }  // namespace svi
@@ -167,9 +175,13 @@ sv_status sv_alloc(uint32_t n, sv_dtype dtype, void *dev_buf, size_t bytes, void
     }
     e = cudaMalloc(reinterpret_cast<void **>(&s->ws), WS_BYTES);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->ws, 0, WS_BYTES, s->stream);
+    if (e == cudaSuccess)
+        e = cudaHostAlloc(reinterpret_cast<void **>(&s->mail), WS_RESULT + 1024, cudaHostAllocMapped | cudaHostAllocPortable);
+    if (e == cudaSuccess) e = cudaHostGetDevicePointer(reinterpret_cast<void **>(&s->mail_dev), s->mail, 0);
     if (e != cudaSuccess) {
         if (s->owned) cudaFree(s->buf);
         if (s->ws) cudaFree(s->ws);
+        if (s->mail) cudaFreeHost(s->mail);
         delete s;
         return set_error(SV_ERR_OOM, std::string("sv_alloc: workspace: ") + cudaGetErrorString(e));
     }
@@ -188,6 +200,7 @@ sv_status sv_free(sv_state *s) {
     cudaStreamSynchronize(s->stream);
     if (s->owned && s->buf) cudaFree(s->buf);
     if (s->ws) cudaFree(s->ws);
+    if (s->mail) cudaFreeHost(s->mail);
     if (s->snap) cudaFree(s->snap);
     if (s->samp) cudaFree(s->samp);
     if (s->probs_buf) cudaFree(s->probs_buf);
@@ -209,8 +222,7 @@ sv_status sv_set_basis(sv_state *s, uint64_t x) {
     if (!s) return set_error(SV_ERR_ARG, "sv_set_basis: null state");
     if (check_live(s, "sv_set_basis") != SV_OK) return SV_ERR_STATE;
     if (x >> s->n) return set_error(SV_ERR_ARG, "sv_set_basis: x >= 2^n");
-    SV_CUDA(cudaMemsetAsync(s->buf, 0, state_bytes(s), s->stream));
-    sv_status st = launch_set_one(s, x);
+    sv_status st = launch_set_basis(s, x);
     if (st != SV_OK) return st;
     s->basis_known = true;
     s->basis_x = x;
@@ -794,9 +806,7 @@ sv_status sv_expect(sv_state *s, const uint64_t *xmask, const uint64_t *zmask, c
         *out = 0.0;
         return SV_OK;
     }
-    sv_status st = launch_expect(s, xmask, zmask, coef, nterms, out);
-    if (st != SV_OK) return st;
-    return check_device_error(s);
+    return launch_expect(s, xmask, zmask, coef, nterms, out);
 }
 
 sv_status sv_topk(sv_state *s, uint32_t k, uint64_t *idx, double *p) {
@@ -804,9 +814,7 @@ sv_status sv_topk(sv_state *s, uint32_t k, uint64_t *idx, double *p) {
     if (!s || !idx || !p) return set_error(SV_ERR_ARG, "sv_topk: null argument");
     if (check_live(s, "sv_topk") != SV_OK) return SV_ERR_STATE;
     if (k < 1 || k > 64) return set_error(SV_ERR_ARG, "sv_topk: k must be 1..64");
-    sv_status st = launch_topk(s, k, idx, p);
-    if (st != SV_OK) return st;
-    return check_device_error(s);
+    return launch_topk(s, k, idx, p);
 }
 
 sv_status sv_debug_fail_allocs(uint32_t count) {

@@ -7,6 +7,7 @@
 #include <cstdint>
 #include <mutex>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "sv.h"
@@ -83,13 +84,13 @@ struct sv_circuit {
 // Device workspace layout (bytes), carved from one allocation.
 namespace svi {
 constexpr size_t WS_ERR = 0;                   // int error word (+ padding)
-constexpr size_t WS_PARTIAL = 256;             // double partials[WS_NPARTIAL]
+// 64 doubles, then the 64 indices of a top-k (server states; others use the mailbox)
+constexpr size_t WS_RESULT = 16;
+constexpr size_t WS_PARTIAL = 2048;            // double partials[WS_NPARTIAL]
 constexpr int WS_NPARTIAL = 8192;
-constexpr size_t WS_RESULT = WS_PARTIAL + WS_NPARTIAL * 8;   // double results[64]
-constexpr size_t WS_TOPK = WS_RESULT + 64 * 8;               // top-k candidates
-constexpr int TOPK_MAX_WARPS = 4096;
-constexpr size_t WS_TOPK_BYTES = size_t(TOPK_MAX_WARPS) * 64 * 16;
-constexpr size_t WS_BYTES = WS_TOPK + WS_TOPK_BYTES + 64 * 16;
+constexpr size_t WS_TOPK = WS_PARTIAL + WS_NPARTIAL * 8;   // chunk maxima of a top-k; tables of an expectation
+constexpr size_t WS_TOPK_BYTES = size_t(4) << 20;
+constexpr size_t WS_BYTES = WS_TOPK + WS_TOPK_BYTES;
 }  // namespace svi
 
 struct sv_state {
@@ -110,11 +111,19 @@ struct sv_state {
     uint32_t policy = 0;        // SV_POLICY_* flags (kernel selection)
     void *samp = nullptr;       // sampling scratch (sample.cu), kept across calls
     size_t samp_cap = 0;
+    // results and the error word in page-locked host memory that kernels write (sv_alloc): a
+    // call that returns a number then needs no copy.  Layout as WS_ERR / WS_RESULT.
+    unsigned char *mail = nullptr, *mail_dev = nullptr;
     void *probs_buf = nullptr;  // SV_POLICY_STAGED_PROBS: device probabilities, kept across calls
     size_t probs_cap = 0;
 };
 
 namespace svi {
+// Where a reduction's last kernel writes: results, and a copy of the error word.
+inline double *mail_results(const sv_state *s) { return reinterpret_cast<double *>(s->mail_dev + WS_RESULT); }
+inline int *mail_error(const sv_state *s) { return reinterpret_cast<int *>(s->mail_dev + WS_ERR); }
+inline const int *device_error(const sv_state *s) { return reinterpret_cast<const int *>(s->ws + WS_ERR); }
+
 // Which kernel family ran a pass (launch_apply's optional out-parameter).
 enum PassKind { PASS_CUDA_CORE = 0, PASS_TENSOR_CORE = 1, PASS_STRUCTURED = 2 };
 }  // namespace svi
@@ -136,24 +145,25 @@ struct sv_batch_launch {
 };
 
 namespace svk {
-// Launch a pass kernel that begins with pass_trigger() and calls pass_wait() before its first
-// access to the state: its launch latency and prologue overlap the previous pass's tail.
+// Launch a kernel that begins with pass_trigger() and calls pass_wait() before its first access
+// to memory that other kernels touch: its launch latency and prologue overlap the previous
+// kernel's tail.
 // Measured on whole circuits, in-order launches -> this: 350 gates on 12 qubits (complex128)
 // 3094 -> 2169 us, 50 passes on 20 qubits 573 -> 481 us, 74 on 28 qubits 50.21 -> 49.93 ms.
-template <typename Args>
-cudaError_t launch_pass(void (*kern)(Args), unsigned grid, unsigned block, size_t smem, cudaStream_t stream,
-                        const Args &args) {
+template <typename... P, typename... A>
+cudaError_t launch_pass(void (*kern)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t stream,
+                        A &&...args) {
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, args);
+    return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
 }
 
 cudaError_t tc_batch_prepare();
@@ -197,8 +207,11 @@ sv_status enqueue_expect_group(sv_state *s, uint64_t x, const uint64_t *z, const
 sv_status launch_topk(sv_state *s, uint32_t k, uint64_t *idx, double *p);
 sv_status enqueue_topk(sv_state *s, double *host_p, unsigned long long *host_i);
 sv_status launch_widen(sv_state *s, const void *src_c64, void *dst_c128);
-sv_status launch_set_one(sv_state *s, uint64_t x);
+sv_status launch_set_basis(sv_state *s, uint64_t x);
 sv_status check_device_error(sv_state *s);   // synchronises; reads and clears the error word
+// Synchronise and read the first `bytes` (<= 1024) of the results that the stream's last kernel
+// left in the state's mailbox, with the error word; one found set is cleared and reported.
+sv_status read_results(sv_state *s, void *dst, size_t bytes);
 // The circuit's input gates fused again at width <= 4 when its schedule has width-5 gates
 // (built once per circuit), else its schedule: what complex128 runs on the tensor cores.
 const std::vector<Gate> &narrow_schedule(const sv_circuit *c);
