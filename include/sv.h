@@ -183,14 +183,17 @@ typedef struct {
 typedef struct {
     int32_t dtype_used;         /* sv_dtype that produced the final state */
     uint32_t promotions;        /* 1 if the circuit was replayed in complex128 */
-    uint64_t passes;            /* HBM passes enqueued (including a replay); a two-gate
-                                   pass counts once */
+    uint64_t passes;            /* passes applied (including a replay); a two-gate pass
+                                   counts once, a gate that shares a launch or a read of the
+                                   state with others (small states; runs of diagonal gates or
+                                   of swaps) once each */
     double norm_before;         /* FP64 norms when adaptive (else 0); norm_before of a basis
                                    start is exactly 1 and takes no pass */
     double norm_after;
     double drift;               /* |norm_after - norm_before| of the reported run */
     uint64_t bytes;             /* algorithmic HBM bytes of the passes: 2 * 2^n * s per dense
-                                   pass, 2 * s per touched amplitude of a structured one */
+                                   pass and per run of structured gates that shares one,
+                                   2 * s per touched amplitude of a structured pass */
     double apply_ms;            /* with opts->timing: CUDA-event time of all passes (ms) */
     uint64_t tc_passes;         /* passes that ran on the tensor-core kernels */
     uint32_t max_k_used;        /* widest gate of the schedule that produced the final state */

@@ -181,11 +181,12 @@ sv_status launch_apply_t(sv_state *s, const svi::Gate &g) {
 
 namespace svi {
 
-sv_status launch_apply(sv_state *s, const Gate &g, uint64_t *bytes, int *kind) {
+sv_status launch_apply(sv_state *s, const Gate &g, uint64_t *bytes, int *kind, const Structure *given) {
     if (g.k < 1 || g.k > SV_MAX_K || g.k > s->n)
         return set_error(SV_ERR_ARG, "apply: gate width out of range");
     if (!(s->policy & SV_POLICY_DENSE_ONLY)) {
-        const Structure st = classify(g);
+        const Structure own = given ? Structure() : classify(g);
+        const Structure &st = given ? *given : own;
         if (struct_preferred(s, st)) {
             if (kind) *kind = PASS_STRUCTURED;
             if (bytes) *bytes = struct_bytes(s, st);

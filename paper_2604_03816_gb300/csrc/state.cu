@@ -582,7 +582,29 @@ static sv_status run_schedule(sv_state *s, const std::vector<Gate> &gates, size_
         st = launch_small(s, gates, begin, end, &r->bytes);
         for (size_t i = begin; i < end; ++i) r->max_k_used = std::max(r->max_k_used, gates[i].k);
     }
+    // runs of structured gates share a pass (not with the kernel-selection flags that ask for a
+    // pass per gate)
+    const bool runs = !small && !(s->policy & (SV_POLICY_DENSE_ONLY | SV_POLICY_TWO_GATE_PASSES));
+    std::vector<Structure> structure;      // of the gates looked at so far
+    structure.reserve(runs ? end - begin : 0);
+    auto kind_of = [&](size_t i) {
+        while (structure.size() <= i) structure.push_back(classify(gates[begin + structure.size()]));
+        return structure[i].kind;
+    };
     for (size_t i = 0; i < first.size() && st == SV_OK; ++i) {
+        if (runs) {
+            size_t e = i + 1;              // gates of one structured kind in a row
+            const uint32_t kind = kind_of(i);
+            if (kind == SV_STRUCT_DIAGONAL || kind == SV_STRUCT_MONOMIAL)
+                while (begin + e < end && kind_of(e) == kind) ++e;
+            const size_t m = e - i < 2 ? 0 : launch_run(s, gates, structure.data() + i, begin + i, begin + e, &st);
+            if (m) {
+                r->bytes += 2ull * state_bytes(s);
+                for (size_t q = 0; q < m; ++q) r->max_k_used = std::max(r->max_k_used, gates[begin + i + q].k);
+                i += m - 1;
+                continue;
+            }
+        }
         const Gate &g = gates[first[i]];
         if (second[i] >= 0) {
             const Gate &g2 = gates[second[i]];
@@ -595,7 +617,7 @@ static sv_status run_schedule(sv_state *s, const std::vector<Gate> &gates, size_
         }
         uint64_t b = 0;
         int kind = PASS_CUDA_CORE;
-        st = launch_apply(s, g, &b, &kind);
+        st = launch_apply(s, g, &b, &kind, runs ? &structure[i] : nullptr);
         r->bytes += b;
         if (kind == PASS_TENSOR_CORE) ++r->tc_passes;
         r->max_k_used = std::max(r->max_k_used, g.k);

@@ -179,7 +179,13 @@ namespace svi {
 // ---- kernels (apply_kernels.cu / reduce_kernels.cu); all enqueue on s->stream ----
 // One pass of g; *bytes (if given) gets the pass's algorithmic HBM bytes: a full read and
 // write of the state, or of the amplitudes a structure-aware pass touches.
-sv_status launch_apply(sv_state *s, const Gate &g, uint64_t *bytes = nullptr, int *kind = nullptr);
+// st: the gate's structure where the caller has it.
+sv_status launch_apply(sv_state *s, const Gate &g, uint64_t *bytes = nullptr, int *kind = nullptr,
+                       const Structure *st = nullptr);
+// Gates from `begin` on that share one pass (apply_runs.cu; st[i - begin]: gate i's structure):
+// how many it ran, 0 if there is no run there that pays.
+size_t launch_run(sv_state *s, const std::vector<Gate> &gates, const Structure *st, size_t begin, size_t end,
+                  sv_status *status);
 // Structure-aware pass (apply_struct.cu): is it preferred over the dense kernels, and run it.
 bool struct_preferred(const sv_state *s, const Structure &st);
 sv_status launch_apply_struct(sv_state *s, const Structure &st);
