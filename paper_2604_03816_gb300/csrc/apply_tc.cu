@@ -120,12 +120,12 @@ struct TcArgs {
     // takes group members in the order c ^ x(l), x(l) = (l >> xs) & (2^xt - 1)
     uint32_t xs, xt;
     // batched launches: ntiles = states x tiles_per_state, state i at amplitude offset
-    // i 2^n; state i's matrix is utab + i 2 4^kin (FP32 complex, row-major), of width kin
-    // = K, or K - 1 widened by an identity qubit at local bit jw (jw = -1: not widened)
-    const float *utab;
+    // i 2^n; state i's operand (the B set as it lies in shared memory) is images + i B_SET, its
+    // scale bscale[i] (pack_images)
+    const unsigned char *images;
+    const float *bscale;
     unsigned long long tiles_per_state;
-    uint32_t n, kin;
-    int jw;
+    uint32_t n;
 };
 
 // v[c] <- v[c ^ x] for the low xt bits of x: one conditional-swap stage per bit.
@@ -214,52 +214,6 @@ __device__ __forceinline__ void expand_b(unsigned char *sB, const int2 *bx, uint
     }
 }
 
-// Batched launches build B in shared memory from a state's FP32 matrix (width kin, or
-// K - 1 widened by an identity qubit at local bit jw): entry (r, c) of the K-qubit U.
-__device__ __forceinline__ float u_entry(const float *U, uint32_t kin, int jw, uint32_t r, uint32_t c,
-                                         uint32_t part) {
-    if (jw >= 0) {
-        if (((r ^ c) >> jw) & 1u) return 0.f;
-        const uint32_t lo = (1u << jw) - 1u;
-        r = (r & lo) | ((r >> (jw + 1)) << jw);
-        c = (c & lo) | ((c >> (jw + 1)) << jw);
-    }
-    return U[2u * ((r << kin) + c) + part];
-}
-
-// Largest |entry| of a state's stored matrix over the entries i0, i0 + stride, ...
-__device__ __forceinline__ float u_absmax_part(const float *U, uint32_t kin, uint32_t i0, uint32_t stride) {
-    float m = 0.f;
-    for (uint32_t i = i0; i < (2u << (2u * kin)); i += stride) m = fmaxf(m, fabsf(U[i]));
-    return m;
-}
-
-// B = the four FP16 slices (B1, B2, B3 2^-9, B2 2^-9) of R x sb, R the real embedding of
-// the state's U and sb = 2^(8 - eb) with max |R| < 2^eb, so |R sb| < 256 and the three
-// 9-bit slices of the FP32 value are exact; entries i0, i0 + stride, ...
-template <int K>
-__device__ void build_b(unsigned char *sB, const float *U, uint32_t kin, int jw, float sb, uint32_t i0,
-                        uint32_t stride) {
-    using S = TcShape<K, 1, true>;
-    constexpr uint32_t KD = S::KD;
-    for (uint32_t e = i0; e < KD * KD; e += stride) {
-        const uint32_t n = e / KD, kk = e % KD, r = n >> 1, c = kk >> 1;
-        float v;
-        if ((n & 1u) == (kk & 1u)) v = u_entry(U, kin, jw, r, c, 0);
-        else v = (n & 1u) ? u_entry(U, kin, jw, r, c, 1) : -u_entry(U, kin, jw, r, c, 1);
-        const float x = v * sb;
-        const float b1 = rintf(x);
-        const float x2 = (x - b1) * 512.f;
-        const float b2 = rintf(x2);
-        const float b3 = rintf((x2 - b2) * 512.f);
-        const uint32_t off = kmajor_off16(n, kk, S::SBO);
-        *reinterpret_cast<__half *>(sB + 0 * S::B_BYTES + off) = __float2half_rn(b1);
-        *reinterpret_cast<__half *>(sB + 1 * S::B_BYTES + off) = __float2half_rn(b2);
-        *reinterpret_cast<__half *>(sB + 2 * S::B_BYTES + off) = __float2half_rn(b3 * (1.f / 512.f));
-        *reinterpret_cast<__half *>(sB + 3 * S::B_BYTES + off) = __float2half_rn(b2 * (1.f / 512.f));
-    }
-}
-
 // sb = 2^(8 - eb) and 1 / sb for a matrix whose largest |entry| is m < 2^eb.
 __device__ __forceinline__ void b_grid(float m, float &sb, float &inv) {
     int eb = 0;
@@ -269,14 +223,95 @@ __device__ __forceinline__ void b_grid(float m, float &sb, float &inv) {
     inv = ldexpf(1.f, eb - 8);
 }
 
+// Operands of batched launches.  Every (gate, state) of a batch has its own matrix; pack_images
+// cuts them into B sets in global memory, laid out as in shared memory, before the passes, and a
+// pass then loads a state's set with one bulk copy.  (Built inside the pass by its producer
+// warp, a set cost about 20 us of stalled loads whenever a CTA met a new state: 18 qubits x 96
+// states 115 us per pass -> 79.)
+struct PackGate {
+    unsigned long long tab;          // offset of the gate's FP32 matrices in the table (bytes)
+    unsigned long long image;        // and of its images in units of B sets
+    uint32_t kin;
+    uint32_t idm;                    // identity bits of the width-5 gate it is widened to
+    uint8_t pos[SV_MAX_K];           // its local bits' places there
+};
+constexpr uint32_t PACK_GATES = 64;
+struct PackArgs {
+    const unsigned char *utab;       // matrices of the first state
+    unsigned char *images;
+    float *bscale;
+    PackGate g[PACK_GATES];
+};
+
+// One block per (state, gate).  R is the real embedding of the widened U times sb, so |R sb| <
+// 256 and the three 9-bit slices of the FP32 values are exact.  A thread writes 16-byte chunks of
+// the slices B1, B2, B3 2^-9, B2 2^-9: eight columns of one row.
+__global__ void __launch_bounds__(256) pack_images(const __grid_constant__ PackArgs a) {
+    using S = TcShape<5, 1, true>;
+    __shared__ float red[8];
+    const uint32_t tid = threadIdx.x;
+    const PackGate &g = a.g[blockIdx.y];
+    const uint32_t kin = g.kin, size = 2u << (2u * kin);
+    pass_trigger();
+    pass_wait();
+    const float *U = reinterpret_cast<const float *>(a.utab + g.tab) + (size_t)blockIdx.x * size;
+    float m = 0.f;
+    for (uint32_t i = tid; i < size; i += 256) m = fmaxf(m, fabsf(U[i]));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((tid & 31u) == 0) red[tid >> 5] = m;
+    __syncthreads();
+    m = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) m = fmaxf(m, red[w]);
+    float sb, inv;
+    b_grid(m, sb, inv);
+    const unsigned long long at = g.image + blockIdx.x;
+    if (tid == 0) a.bscale[at] = inv;
+    unsigned char *img = a.images + at * S::B_SET;
+    auto local = [&](uint32_t x) {                       // the gate's own local index of x
+        uint32_t l = 0;
+        for (uint32_t j = 0; j < kin; ++j) l |= ((x >> g.pos[j]) & 1u) << j;
+        return l;
+    };
+    for (uint32_t q = tid; q < S::B_BYTES / 16u; q += 256) {
+        // the chunk's place (kmajor_off16): row n, columns kk .. kk + 7
+        const uint32_t n = (q / (S::SBO / 16u)) * 8u + (q & 7u), kk = ((q >> 3) & 7u) * 8u;
+        const uint32_t r = n >> 1, lr = local(r);
+        uint32_t w[4][4];
+#pragma unroll
+        for (uint32_t i = 0; i < 4; ++i) {
+            const uint32_t c = (kk >> 1) + i;
+            float2 u = make_float2(0.f, 0.f);
+            if (!((r ^ c) & g.idm)) u = reinterpret_cast<const float2 *>(U)[(lr << kin) + local(c)];
+            const float x[2] = {(n & 1u ? u.y : u.x) * sb, (n & 1u ? u.x : -u.y) * sb};
+            float b[3][2];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                b[0][j] = rintf(x[j]);
+                const float x2 = (x[j] - b[0][j]) * 512.f;
+                b[1][j] = rintf(x2);
+                b[2][j] = rintf((x2 - b[1][j]) * 512.f) * (1.f / 512.f);
+            }
+            w[0][i] = pack_half2(b[0][0], b[0][1]);
+            w[1][i] = pack_half2(b[1][0], b[1][1]);
+            w[2][i] = pack_half2(b[2][0], b[2][1]);
+            w[3][i] = pack_half2(b[1][0] * (1.f / 512.f), b[1][1] * (1.f / 512.f));
+        }
+#pragma unroll
+        for (uint32_t s = 0; s < 4; ++s)
+            *reinterpret_cast<uint4 *>(img + s * S::B_BYTES + q * 16u) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
+    }
+}
+
 // XP: the launch has targets among tile bits 0..3 and takes members in the lane's XOR
 // order; otherwise every lane takes them in member order (no permutation code at all).
 // The pipelines count tiles (j: raw stage, output staging) and MMA subtiles (js = j SUB +
 // sub: A and D buffers, row scales).
 // BT: one launch over a batch of states, each with its own matrix: a CTA takes a
-// contiguous range of tiles (so it meets few states), B is double-buffered and rebuilt by
-// the producer warp from the next state's matrix when its first tile comes up (b_full:
-// built; b_empty: the MMAs of the state that last used the set have completed).
+// contiguous range of tiles (so it meets few states), B is double-buffered and the producer
+// loads the next state's set a few tiles into the current one (b_full: arrived; b_empty: the
+// MMAs of the state that last used the set have completed).
 // SW: tiles move by 2-D tensor-map copies that store them in shared memory with the
 // 128-byte swizzle (16-byte chunk index XOR the 128-byte row within each 1 KiB), and the
 // roles address the tile through the same swizzle.  A warp's lanes (consecutive groups)
@@ -297,8 +332,6 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
     __shared__ __align__(8) unsigned long long b_full[2], b_empty[2];   // batched launches
-    __shared__ float b_scale[2];
-    __shared__ float red[32];
     // B slices, the raw stages and the output staging tiles; B operand reads stay inside
     // the CTA's shared memory whatever the descriptor strides.
     unsigned char *sB = smem;
@@ -341,29 +374,10 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
         tend = min(a.ntiles, first + per);
         step = 1;
     }
-    if constexpr (BT) {
-        // B set 0 from the matrix of the range's first state, built by every thread
-        const unsigned long long st0 = first < tend ? first / a.tiles_per_state : 0;
-        const float *U0 = a.utab + st0 * (2ull << (2u * a.kin));
-        float m = u_absmax_part(U0, a.kin, tid, blockDim.x);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (lane == 0) red[warp] = m;
-        __syncthreads();
-        m = 0.f;
-        for (uint32_t w = 0; w < S::THREADS / 32u; ++w) m = fmaxf(m, red[w]);
-        float sb, inv;
-        b_grid(m, sb, inv);
-        build_b<K>(sB, U0, a.kin, a.jw, sb, tid, blockDim.x);
-        if (tid == 0) b_scale[0] = inv;
-    }
-    if constexpr (BT) fence_proxy_async_smem();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if constexpr (BT) {
-        if (tid == 0) mbar_arrive(smem_u32(&b_full[0]));   // set 0: its first use
-    } else if (warp != S::W_PROD) {
+    if (!BT && warp != S::W_PROD) {
         // every warp but the producer, which is already loading the first tiles
         const uint32_t i = tid < S::W_PROD * 32u ? tid : tid - 32u;
         expand_b<K, (int)S::NB>(sB, a.bx, S::B_BYTES, S::SBO, i, S::THREADS - 32u);
@@ -409,33 +423,32 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
         sl.init(a.L, a.h, a.hi, lane);
         pass_wait();
         uint32_t j = 0;
-        unsigned long long cur = ~0ull;
-        uint32_t nsw = 0;                         // state changes so far (B set = nsw & 1)
+        // batched: B sets are requested state by state, from the range's first one
+        const unsigned long long st0 = BT ? first / a.tiles_per_state : 0;
+        unsigned long long asked = st0;
+        auto ask = [&]() -> bool {
+            const uint32_t i = (uint32_t)(asked - st0), set = i & 1u, use = i >> 1;
+            bool okb = true;
+            if (lane == 0) {
+                if (use >= 1) okb = mbar_wait_or_abort(smem_u32(&b_empty[set]), (use - 1u) & 1u, abort);
+                if (okb) {
+                    const uint32_t bar = smem_u32(&b_full[set]);
+                    mbar_arrive_expect_tx(bar, S::B_SET);
+                    bulk_g2s(smem_u32(sB + set * S::B_SET), a.images + asked * S::B_SET, S::B_SET, bar);
+                }
+            }
+            ++asked;
+            return __shfl_sync(0xffffffffu, (int)okb, 0) != 0;
+        };
         for (unsigned long long t = first; t < tend; t += step, ++j) {
             if constexpr (BT) {
-                const unsigned long long st = t / a.tiles_per_state;
-                if (cur == ~0ull) {
-                    cur = st;                     // set 0 was built at the start
-                } else if (st != cur) {
-                    cur = st;
-                    ++nsw;
-                    const uint32_t set = nsw & 1u, use = nsw >> 1;
-                    bool okb = true;
-                    if (use >= 1 && lane == 0)
-                        okb = mbar_wait_or_abort(smem_u32(&b_empty[set]), (use - 1u) & 1u, abort);
-                    if (!__shfl_sync(0xffffffffu, (int)okb, 0)) break;
-                    const float *U = a.utab + st * (2ull << (2u * a.kin));
-                    float m = u_absmax_part(U, a.kin, lane, 32);
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-                    float sb, inv;
-                    b_grid(m, sb, inv);
-                    build_b<K>(sB + set * S::B_SET, U, a.kin, a.jw, sb, lane, 32);
-                    if (lane == 0) b_scale[set] = inv;
-                    fence_proxy_async_smem();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&b_full[set]));
-                }
+                const unsigned long long st = t / a.tiles_per_state, in = t - st * a.tiles_per_state;
+                if (asked <= st && !ask()) break;
+                // the next state's set, once the previous state's last MMAs must be done (its
+                // tiles left the raw stages), or at the last tile of this one
+                if (asked == st + 1 && (in >= 3 || in + 1 == a.tiles_per_state) && asked * a.tiles_per_state < tend &&
+                    !ask())
+                    break;
             }
             const uint32_t s = j % NS, u = j / NS;
             bool ok = true;
@@ -524,15 +537,15 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
         uint32_t j = 0;
         bool stop = false;
         unsigned long long cur = ~0ull;
-        uint32_t nsw = 0;
+        float bsc = a.b_inv_scale;
         for (unsigned long long t = first; t < tend && !stop; t += step, ++j) {
-            if constexpr (BT) {
-                const unsigned long long st = t / a.tiles_per_state;
-                if (cur != ~0ull && st != cur) ++nsw;
-                cur = st;
-            }
             const uint32_t s = j % NS;
             const bool okf = mbar_wait_or_abort(smem_u32(&full[s]), (j / NS) & 1u, abort);
+            if constexpr (BT) {
+                const unsigned long long st = t / a.tiles_per_state;
+                if (st != cur) bsc = __ldcg(a.bscale + st);       // after the first tile's arrival
+                cur = st;
+            }
             const float2 *rs = reinterpret_cast<const float2 *>(smem + S::OFF_RAW + s * S::TILE_BYTES);
 #pragma unroll
             for (uint32_t sub = 0; sub < SUB; ++sub) {
@@ -563,8 +576,7 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
                 // slot js & 3 was last read by the epilogue of subtile js - 4, which finished
                 // before the MMAs of subtile js - 2 were issued, whose completion released
                 // a_empty[ab]
-                // batched: the state's B scale, written by the producer before this tile's load
-                if (part == 0) row_scale[js & 3u][row] = ldexpf(BT ? b_scale[nsw & 1u] : a.b_inv_scale, ex - 8);
+                if (part == 0) row_scale[js & 3u][row] = ldexpf(bsc, ex - 8);
                 if constexpr (XP) xor_unpermute(v, xl, a.xt);   // back in member order (x < HALF)
                 // three 9-bit integer slices (and A2 2^-9 when SUB = 2), one FP16 pair
                 // (re, im) per 32-bit TMEM column, stored eight members at a time
@@ -815,11 +827,10 @@ sv_status launch_tc_t(sv_state *s, const svi::Gate &g) {
     return SV_OK;
 }
 
-// Batched launches (sv_batch_apply): complex64 gates of width 4 or 5 on states of at least
-// 12 qubits run as width-5 gates (a width-4 gate widened by an identity qubit, chosen as
-// in widen_gate) with one MMA subtile per stage; each state's B is built on the device
-// from the batch's FP32 matrix table.
-// Batched launches use the swizzled tensor-map staging (SW), like single states.
+// Batched launches (sv_batch_apply): complex64 gates on states of at least 13 qubits (12 for
+// widths 4 and 5) run as width-5 gates (a narrower gate widened by identity qubits, chosen as in
+// widen_gate) with one MMA subtile per stage and the swizzled tensor-map staging (SW), like single
+// states.
 static cudaError_t tc_batch_setup() {
     static std::once_flag once;
     static cudaError_t err = cudaSuccess;
@@ -837,31 +848,57 @@ cudaError_t tc_batch_prepare() {
     return e;
 }
 
+// The width-5 targets of a gate, and where its own local bits lie among them.
+static void widen_targets(uint32_t n, uint32_t k, const uint32_t *t, uint32_t (&t5)[5], uint8_t *pos, uint32_t *idm) {
+    uint64_t used = 0;
+    for (uint32_t j = 0; j < k; ++j) used |= 1ull << t[j];
+    uint32_t m = k;
+    for (uint32_t q = 5; q < n && m < 5; ++q)
+        if (!((used >> q) & 1ull)) { used |= 1ull << q; ++m; }
+    for (uint32_t q = 0; q < n && m < 5; ++q)
+        if (!((used >> q) & 1ull)) { used |= 1ull << q; ++m; }
+    uint32_t i = 0, own = 0;
+    *idm = 0;
+    for (uint32_t q = 0; q < n && i < 5; ++q)
+        if ((used >> q) & 1ull) {
+            t5[i] = q;
+            if (own < k && t[own] == q) pos[own++] = (uint8_t)i;
+            else *idm |= 1u << i;
+            ++i;
+        }
+}
+
+size_t tc_batch_image_bytes() { return TcShape<5, 1, true>::B_SET; }
+
+sv_status launch_tc_pack(const sv_batch_launch *L, const size_t *tab_off, uint32_t ngates, const void *utab,
+                         void *images, float *bscale) {
+    for (uint32_t g0 = 0; g0 < ngates; g0 += PACK_GATES) {
+        const uint32_t m = std::min(PACK_GATES, ngates - g0);
+        PackArgs a;
+        a.utab = static_cast<const unsigned char *>(utab);
+        a.images = static_cast<unsigned char *>(images);
+        a.bscale = bscale;
+        for (uint32_t i = 0; i < m; ++i) {
+            const sv_batch_launch &l = L[g0 + i];
+            uint32_t t5[5];
+            a.g[i].tab = tab_off[g0 + i];
+            a.g[i].image = (unsigned long long)(g0 + i) * l.states;
+            a.g[i].kin = l.k;
+            widen_targets(l.n, l.k, l.t, t5, a.g[i].pos, &a.g[i].idm);
+        }
+        SV_CUDA(launch_pass(pack_images, dim3(L[g0].states, m), 256, 0, L[g0].stream, a));
+    }
+    return SV_OK;
+}
+
 sv_status launch_tc_batch(const sv_batch_launch &L) {
     using S = TcShape<5, 1, true>;
     const cudaError_t e0 = tc_batch_prepare();
     if (e0 != cudaSuccess)
         return svi::set_error(SV_ERR_CUDA, std::string("batched tensor-core kernel setup: ") + cudaGetErrorString(e0));
-    uint32_t t5[5];
-    int jw = -1;
-    if (L.k == 5) {
-        for (int j = 0; j < 5; ++j) t5[j] = L.t[j];
-    } else {
-        // the identity qubit: the smallest non-target at or above bit 5, else below it
-        bool used[64] = {false};
-        for (uint32_t j = 0; j < 4; ++j) used[L.t[j]] = true;
-        uint32_t q = 64;
-        for (uint32_t c = 5; c < L.n && q == 64; ++c)
-            if (!used[c]) q = c;
-        for (uint32_t c = 0; c < L.n && q == 64; ++c)
-            if (!used[c]) q = c;
-        uint32_t m = 0;
-        for (uint32_t j = 0; j < 4; ++j) {
-            if (q < L.t[j] && jw < 0) { jw = (int)m; t5[m++] = q; }
-            t5[m++] = L.t[j];
-        }
-        if (jw < 0) { jw = (int)m; t5[m++] = q; }
-    }
+    uint32_t t5[5], idm;
+    uint8_t pos[SV_MAX_K];
+    widen_targets(L.n, L.k, L.t, t5, pos, &idm);
     const Plan p = make_plan(L.n, 5, t5, S::TB);
     TcArgs<5> a;
     // the whole batch (states back to back) as one tensor; the swizzle spreads the banks
@@ -879,11 +916,10 @@ sv_status launch_tc_batch(const sv_batch_launch &L) {
     for (int j = 0; j < 5; ++j) a.lp[j] = p.lp[j];
     a.xs = 0;
     a.xt = 0;
-    a.utab = static_cast<const float *>(L.utab);
+    a.images = static_cast<const unsigned char *>(L.images);
+    a.bscale = L.bscale;
     a.tiles_per_state = p.ntiles;
     a.n = L.n;
-    a.kin = L.k;
-    a.jw = jw;
     const unsigned grid = (unsigned)std::min<unsigned long long>(a.ntiles, (unsigned long long)L.num_sms);
     SV_CUDA(launch_pass(apply_tc<5, false, 1, true, true>, dim3(grid), S::THREADS, S::SMEM, L.stream, a));
     return SV_OK;

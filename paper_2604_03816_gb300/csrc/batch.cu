@@ -8,7 +8,7 @@
 // for each chunk every fused gate is one launch of a persistent tile kernel that strides
 // over all tiles of the chunk's states (the tile geometry is the one of the single-state
 // kernels: TMA 1-D bulk staging of 2^h segments, one HBM/L2 read + write per gate;
-// complex64 gates of width 4 and 5 run on the tensor-core kernel of apply_tc.cu).  The
+// complex64 gates run on the tensor-core kernel of apply_tc.cu where batch_tc says so).  The
 // whole launch sequence is captured once into a CUDA graph and replayed while the batch
 // object, the chunk size and the fused structure stay the same; only the matrix table is
 // refreshed (an H2D copy before the replay).
@@ -223,10 +223,8 @@ struct BatchExpectArgs {
     uint32_t n;
 };
 
-__device__ __forceinline__ float bprob(float x, float y) { return __fadd_rn(__fmul_rn(x, x), __fmul_rn(y, y)); }
-__device__ __forceinline__ double bprob(double x, double y) { return __dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y)); }
-
-// grid (BEXP_BLOCKS, states): partial[state * BEXP_BLOCKS + block]
+// Terms that share an X-part x != 0 (Z strings: expect.cu).  grid (BEXP_BLOCKS, states):
+// partial[state * BEXP_BLOCKS + block]
 template <typename R>
 __global__ void batch_expect_kernel(const __grid_constant__ BatchExpectArgs a, const void *psi_,
                                     double *partial) {
@@ -234,56 +232,20 @@ __global__ void batch_expect_kernel(const __grid_constant__ BatchExpectArgs a, c
     const C *psi = reinterpret_cast<const C *>(psi_) + ((unsigned long long)blockIdx.y << a.n);
     double acc = 0.0;
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-    // Z-only terms: runs of eight consecutive amplitudes per thread, the term weights and
-    // the run's sum in the state's precision (FP32 for complex64: GB300's FP64 pipe is
-    // narrow), one FP64 add per run
-    __shared__ R cw[BEXP_TERMS];
-    if (threadIdx.x < BEXP_TERMS) cw[threadIdx.x] = (R)a.ccr[threadIdx.x];
-    __syncthreads();
-    const unsigned long long nrun = a.x == 0 ? a.npairs / 8 : 0;
-    for (unsigned long long r = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; r < nrun;
-         r += stride) {
-        C v[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) v[q] = psi[r * 8 + q];
-        // terms outside, the eight amplitudes inside: eight independent weight sums
-        R w[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) w[q] = 0;
+    for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < a.npairs; i += stride) {
+        const unsigned long long k = insert_zero64(i, (uint32_t)a.hb), k2 = k ^ a.x;
+        const C p = psi[k], q = psi[k2];
+        const double re = (double)q.x * p.x + (double)q.y * p.y;
+        const double im = (double)q.x * p.y - (double)q.y * p.x;
+        double w1r = 0, w1i = 0, w2r = 0, w2i = 0;
         for (int t = 0; t < a.nterms; ++t) {
-            const unsigned long long z = a.z[t];
-            const R c = cw[t];
-            const int hi = __popcll((r * 8) & z);
-#pragma unroll
-            for (int q = 0; q < 8; ++q) w[q] += ((hi + __popc((uint32_t)q & (uint32_t)z)) & 1) ? -c : c;
+            const bool s1 = __popcll(k & a.z[t]) & 1, s2 = __popcll(k2 & a.z[t]) & 1;
+            w1r += s1 ? -a.ccr[t] : a.ccr[t];
+            w1i += s1 ? -a.cci[t] : a.cci[t];
+            w2r += s2 ? -a.ccr[t] : a.ccr[t];
+            w2i += s2 ? -a.cci[t] : a.cci[t];
         }
-        R run = 0;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) run += w[q] * bprob(v[q].x, v[q].y);
-        acc += (double)run;
-    }
-    for (unsigned long long i = nrun * 8 + (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
-         i < a.npairs; i += stride) {
-        if (a.x == 0) {
-            const C v = psi[i];
-            double w = 0.0;
-            for (int t = 0; t < a.nterms; ++t) w += (__popcll(i & a.z[t]) & 1) ? -a.ccr[t] : a.ccr[t];
-            acc += w * (double)bprob(v.x, v.y);
-        } else {
-            const unsigned long long k = insert_zero64(i, (uint32_t)a.hb), k2 = k ^ a.x;
-            const C p = psi[k], q = psi[k2];
-            const double re = (double)q.x * p.x + (double)q.y * p.y;
-            const double im = (double)q.x * p.y - (double)q.y * p.x;
-            double w1r = 0, w1i = 0, w2r = 0, w2i = 0;
-            for (int t = 0; t < a.nterms; ++t) {
-                const bool s1 = __popcll(k & a.z[t]) & 1, s2 = __popcll(k2 & a.z[t]) & 1;
-                w1r += s1 ? -a.ccr[t] : a.ccr[t];
-                w1i += s1 ? -a.cci[t] : a.cci[t];
-                w2r += s2 ? -a.ccr[t] : a.ccr[t];
-                w2i += s2 ? -a.cci[t] : a.cci[t];
-            }
-            acc += re * w1r - im * w1i + re * w2r + im * w2i;
-        }
+        acc += re * w1r - im * w1i + re * w2r + im * w2i;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
@@ -327,8 +289,11 @@ struct sv_batch {
     cudaStream_t stream = nullptr;
     int device = 0, num_sms = 0;
     int *err = nullptr;                 // device error word
-    double *partial = nullptr;          // count * BEXP_BLOCKS
+    double *partial = nullptr;          // partial_room doubles, then the tables of Z strings
+    size_t partial_room = 0;
     double *results = nullptr;          // count
+    void *images = nullptr;             // tensor-core operands of some gates (pack_images), then
+    size_t images_cap = 0;              // their scales: room for images_cap of them
     void *utab = nullptr;               // device matrix table
     size_t utab_cap = 0;
     void *utab_host = nullptr;          // pinned staging of the table
@@ -342,6 +307,8 @@ struct sv_batch {
 };
 
 namespace svi {
+
+constexpr size_t BATCH_Z_TABLES = 4u << 12;      // doubles (batch_z_terms)
 
 static size_t elem_bytes_b(sv_dtype d) { return d == SV_C64 ? 8 : 16; }
 
@@ -363,6 +330,13 @@ static sv_status batch_launch(const sv_batch_launch &L) {
         case 4: return svk::BatchKernel<double, 4>::launch(L);
         default: return svk::BatchKernel<double, 5>::launch(L);
     }
+}
+
+// The tensor cores serve complex64 gates of width 4 and 5 on states of at least 12 qubits, and
+// narrower ones from 13 (one tile more): 18 qubits x 96 states, width 3: 141 us on the CUDA
+// cores, 79 widened.
+static bool batch_tc(sv_dtype dt, uint32_t n, uint32_t k) {
+    return dt == SV_C64 && n >= (k >= 4 ? 12u : 13u);
 }
 
 static cudaError_t batch_prepare(sv_dtype dt, uint32_t k) {
@@ -423,8 +397,10 @@ sv_status sv_batch_alloc(uint32_t n, sv_dtype dtype, uint32_t count, void *dev_b
     }
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&b->err), 256);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->err, 0, 256, b->stream);
-    if (e == cudaSuccess)
-        e = cudaMalloc(reinterpret_cast<void **>(&b->partial), sizeof(double) * count * svk::BEXP_BLOCKS);
+    if (e == cudaSuccess) {
+        b->partial_room = std::max<size_t>((size_t)count * svk::BEXP_BLOCKS, 2 * (size_t)b->num_sms);
+        e = cudaMalloc(reinterpret_cast<void **>(&b->partial), sizeof(double) * (b->partial_room + BATCH_Z_TABLES));
+    }
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&b->results), sizeof(double) * count);
     if (e == cudaSuccess) e = cudaEventCreate(&b->ev0);
     if (e == cudaSuccess) e = cudaEventCreate(&b->ev1);
@@ -453,6 +429,7 @@ sv_status sv_batch_free(sv_batch *b) {
     if (b->partial) cudaFree(b->partial);
     if (b->results) cudaFree(b->results);
     if (b->utab) cudaFree(b->utab);
+    if (b->images) cudaFree(b->images);
     if (b->utab_host) cudaFreeHost(b->utab_host);
     if (b->ev0) cudaEventDestroy(b->ev0);
     if (b->ev1) cudaEventDestroy(b->ev1);
@@ -592,9 +569,35 @@ sv_status sv_batch_apply(sv_batch *b, const sv_circuit *const *circuits, const s
     const uint32_t tile_bits = opts ? opts->tile_bits : 0u;
     if (tile_bits && (tile_bits < svk::BATCH_TB_MIN || tile_bits > svk::BATCH_TB_MAX))
         return set_error(SV_ERR_ARG, "sv_batch_apply: tile_bits must be 0 or 10..13");
-    // complex64 gates of width 4 and 5 on the tensor cores (states of at least 12 qubits)
-    const bool tc_ok = b->dtype == SV_C64 && b->n >= 12 && !(opts && opts->no_tensor_cores);
-    auto use_tc = [&](const Gate &g) { return tc_ok && (g.k == 4 || g.k == 5); };
+    const bool tc_ok = !(opts && opts->no_tensor_cores);
+    auto use_tc = [&](const Gate &g) { return tc_ok && batch_tc(b->dtype, b->n, g.k); };
+    // room for the operands of as many (gate, state) pairs of a chunk as fit 256 MiB; less
+    // where memory is short, down to one pair at a time
+    size_t ntc = 0;
+    for (const Gate &g : c0->gates) ntc += use_tc(g);
+    if (ntc) {
+        const size_t one = svk::tc_batch_image_bytes() + sizeof(float);
+        size_t want = std::min<size_t>(ntc * chunk, (size_t(256) << 20) / one);
+        if (b->images_cap < want) {
+            SV_CUDA(cudaStreamSynchronize(b->stream));
+            if (b->images) cudaFree(b->images);
+            b->images = nullptr;
+            b->images_cap = 0;
+            if (b->graph) {                 // the graph holds the old address
+                cudaGraphExecDestroy(b->graph);
+                b->graph = nullptr;
+                b->graph_key.clear();
+            }
+            cudaError_t e = cudaMalloc(&b->images, want * one);
+            while (e == cudaErrorMemoryAllocation && want > 1) {
+                (void)cudaGetLastError();
+                want /= 2;
+                e = cudaMalloc(&b->images, want * one);
+            }
+            SV_CUDA(e);
+            b->images_cap = want;
+        }
+    }
 
     std::string key = std::to_string(b->n) + "/" + std::to_string(b->count) + "/" +
                       std::to_string(b->dtype) + "/" + std::to_string(chunk) + "/" +
@@ -603,26 +606,59 @@ sv_status sv_batch_apply(sv_batch *b, const sv_circuit *const *circuits, const s
         for (uint32_t j = 0; j < g.k; ++j) key += std::to_string(g.t[j]) + (j + 1 < g.k ? "," : ";");
 
     auto enqueue_all = [&](cudaStream_t stream) -> sv_status {
+        float *scales = reinterpret_cast<float *>(static_cast<char *>(b->images) +
+                                                  b->images_cap * svk::tc_batch_image_bytes());
+        auto launch_of = [&](size_t g, uint32_t s0, uint32_t ns) {
+            const Gate &gg = c0->gates[g];
+            sv_batch_launch L;
+            L.dtype = b->dtype;
+            L.k = gg.k;
+            L.n = b->n;
+            for (uint32_t j = 0; j < SV_MAX_K; ++j) L.t[j] = gg.t[j];
+            L.states = ns;
+            L.psi = static_cast<char *>(b->buf) + sbytes * s0;
+            L.utab = static_cast<char *>(b->utab) + goff[g] + (size_t)s0 * 2 * ((size_t)1 << (2 * gg.k)) * eb;
+            L.err = b->err;
+            L.stream = stream;
+            L.num_sms = b->num_sms;
+            L.tc = use_tc(gg);
+            L.tile_bits = tile_bits;
+            return L;
+        };
+        // states s0 .. s0 + ns - 1 through gates g0 .. g1 - 1, the tensor-core operands of all of
+        // them packed first
+        auto group = [&](uint32_t s0, uint32_t ns, size_t g0, size_t g1) -> sv_status {
+            std::vector<sv_batch_launch> tc, all;
+            std::vector<size_t> off;
+            for (size_t g = g0; g < g1; ++g) {
+                all.push_back(launch_of(g, s0, ns));
+                sv_batch_launch &L = all.back();
+                if (!L.tc) continue;
+                L.images = static_cast<char *>(b->images) + tc.size() * ns * svk::tc_batch_image_bytes();
+                L.bscale = scales + tc.size() * ns;
+                off.push_back((size_t)(static_cast<const char *>(L.utab) - static_cast<const char *>(b->utab)));
+                tc.push_back(L);
+            }
+            sv_status st = tc.empty() ? SV_OK
+                                      : svk::launch_tc_pack(tc.data(), off.data(), (uint32_t)tc.size(), b->utab,
+                                                            b->images, scales);
+            for (size_t i = 0; i < all.size() && st == SV_OK; ++i) st = batch_launch(all[i]);
+            return st;
+        };
         for (uint32_t s0 = 0; s0 < b->count; s0 += chunk) {
             const uint32_t ns = std::min(chunk, b->count - s0);
-            for (size_t g = 0; g < G; ++g) {
-                const Gate &gg = c0->gates[g];
-                sv_batch_launch L;
-                L.dtype = b->dtype;
-                L.k = gg.k;
-                L.n = b->n;
-                for (uint32_t j = 0; j < SV_MAX_K; ++j) L.t[j] = gg.t[j];
-                L.states = ns;
-                L.psi = static_cast<char *>(b->buf) + sbytes * s0;
-                L.utab = static_cast<char *>(b->utab) + goff[g] +
-                         (size_t)s0 * 2 * ((size_t)1 << (2 * gg.k)) * eb;
-                L.err = b->err;
-                L.stream = stream;
-                L.num_sms = b->num_sms;
-                L.tc = use_tc(gg);
-                L.tile_bits = tile_bits;
-                sv_status st = batch_launch(L);
-                if (st != SV_OK) return st;
+            for (size_t g0 = 0; g0 < G;) {
+                // as many gates as have room for their operands, at least one
+                size_t g1 = g0, pairs = 0;
+                while (g1 < G && (g1 == g0 || pairs + (use_tc(c0->gates[g1]) ? ns : 0) <= b->images_cap))
+                    pairs += use_tc(c0->gates[g1++]) ? ns : 0;
+                // a gate of more states than there is room for goes in parts
+                const uint32_t part = pairs > b->images_cap ? (uint32_t)b->images_cap : ns;
+                for (uint32_t s = 0; s < ns; s += part) {
+                    const sv_status st = group(s0 + s, std::min(part, ns - s), g0, g1);
+                    if (st != SV_OK) return st;
+                }
+                g0 = g1;
             }
         }
         return SV_OK;
@@ -693,7 +729,25 @@ sv_status sv_batch_expect(sv_batch *b, const uint64_t *xmask, const uint64_t *zm
     std::vector<size_t> order(nterms);
     for (size_t i = 0; i < nterms; ++i) order[i] = i;
     std::stable_sort(order.begin(), order.end(), [&](size_t a, size_t c) { return xmask[a] < xmask[c]; });
+    auto fold = [&](int per_state) -> sv_status {
+        svk::batch_sum_partials<<<(b->count + 127) / 128, 128, 0, b->stream>>>(b->partial, per_state, (int)b->count,
+                                                                              b->results);
+        SV_CUDA(cudaGetLastError());
+        return SV_OK;
+    };
     size_t i = 0;
+    if (nterms && xmask[order[0]] == 0) {              // the Z strings, all of them together
+        std::vector<uint64_t> z;
+        std::vector<double> c;
+        for (; i < nterms && xmask[order[i]] == 0; ++i) {
+            z.push_back(zmask[order[i]]);
+            c.push_back(coef[order[i]]);
+        }
+        const sv_status st = batch_z_terms(b->buf, b->n, b->dtype, b->count, b->num_sms, b->stream,
+                                           b->partial + b->partial_room, b->partial, b->partial_room, z.data(),
+                                           c.data(), z.size(), fold);
+        if (st != SV_OK) return st;
+    }
     while (i < nterms) {
         svk::BatchExpectArgs a;
         std::memset(&a, 0, sizeof(a));
@@ -707,8 +761,8 @@ sv_status sv_batch_expect(sv_batch *b, const uint64_t *xmask, const uint64_t *zm
             a.cci[a.nterms] = coef[t] * im[y];
             ++a.nterms;
         }
-        a.hb = a.x ? 63 - __builtin_clzll(a.x) : 0;
-        a.npairs = a.x ? (1ull << (b->n - 1)) : (1ull << b->n);
+        a.hb = 63 - __builtin_clzll(a.x);
+        a.npairs = 1ull << (b->n - 1);
         a.n = b->n;
         const dim3 grid(svk::BEXP_BLOCKS, b->count);
         if (b->dtype == SV_C64)
@@ -716,14 +770,13 @@ sv_status sv_batch_expect(sv_batch *b, const uint64_t *xmask, const uint64_t *zm
         else
             svk::batch_expect_kernel<double><<<grid, 256, 0, b->stream>>>(a, b->buf, b->partial);
         SV_CUDA(cudaGetLastError());
-        svk::batch_sum_partials<<<(b->count + 127) / 128, 128, 0, b->stream>>>(
-            b->partial, svk::BEXP_BLOCKS, (int)b->count, b->results);
-        SV_CUDA(cudaGetLastError());
+        const sv_status st = fold(svk::BEXP_BLOCKS);
+        if (st != SV_OK) return st;
     }
-    SV_CUDA(cudaMemcpyAsync(out, b->results, sizeof(double) * b->count, cudaMemcpyDeviceToHost, b->stream));
-    SV_CUDA(cudaStreamSynchronize(b->stream));
     int err = 0;
-    SV_CUDA(cudaMemcpy(&err, b->err, sizeof(int), cudaMemcpyDeviceToHost));
+    SV_CUDA(cudaMemcpyAsync(out, b->results, sizeof(double) * b->count, cudaMemcpyDeviceToHost, b->stream));
+    SV_CUDA(cudaMemcpyAsync(&err, b->err, sizeof(int), cudaMemcpyDeviceToHost, b->stream));
+    SV_CUDA(cudaStreamSynchronize(b->stream));
     if (err) {
         SV_CUDA(cudaMemset(b->err, 0, sizeof(int)));
         return set_error(SV_ERR_TIMEOUT, "a bounded device-side wait gave up in a batched pass");
@@ -764,7 +817,6 @@ sv_status sv_batch_tune(sv_batch *b, const sv_gate *gates, size_t ngates, uint32
     // (a fixed cost of about 20 us per launch) prefer few large launches
     const size_t sbytes = (b->dtype == SV_C64 ? size_t(8) : size_t(16)) << b->n;
     const size_t l2s[3] = {size_t(64) << 20, size_t(512) << 20, sbytes * b->count};
-    const bool tc_ok = b->dtype == SV_C64 && b->n >= 12;
     for (uint32_t k = kmin; k <= kmax; ++k) {
         sv_circuit *c = nullptr;
         sv_status st = sv_fuse(gates, ngates, b->n, k, &c);
@@ -803,7 +855,7 @@ sv_status sv_batch_tune(sv_batch *b, const sv_gate *gates, size_t ngates, uint32
         // the tile size of the CUDA-core passes, at this width's best chunking, when the
         // schedule has such passes (complex128, narrow gates, tensor cores not eligible)
         bool cuda_core = false;
-        for (const Gate &g : c->gates) cuda_core = cuda_core || !(tc_ok && (g.k == 4 || g.k == 5));
+        for (const Gate &g : c->gates) cuda_core = cuda_core || !batch_tc(b->dtype, b->n, g.k);
         if (cuda_core && st == SV_OK)
             for (uint32_t tb = svk::BATCH_TB_MIN; tb <= svk::BATCH_TB_MAX && st == SV_OK; ++tb)
                 kbest = std::min(kbest, time_it(kl2, tb));

@@ -32,6 +32,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <functional>
 #include <mutex>
 #include <type_traits>
 #include <vector>
@@ -114,7 +115,8 @@ struct ZArgs {
     double ch[Z_TERMS];
 };
 
-// Amplitude indices of a thread within the tile: e * 2 * THREADS + 2 tid + q for complex64
+// blockIdx.y: the state of a batch (states back to back, each of ntiles tiles; its partials follow
+// each other).  Amplitude indices of a thread within the tile: e * 2 * THREADS + 2 tid + q for complex64
 // (16-byte loads of two), e * THREADS + tid for complex128.
 template <typename R, int NC>
 __global__ void __launch_bounds__(THREADS, NC >= 2 ? 1 : 2) z_sum(const __grid_constant__ ZArgs a) {
@@ -125,9 +127,9 @@ __global__ void __launch_bounds__(THREADS, NC >= 2 ? 1 : 2) z_sum(const __grid_c
     using S = typename Sum<R>::T;
     __shared__ double wh_s[2][8];
     __shared__ uint32_t sg_s[2][8];
-    const V *psi = reinterpret_cast<const V *>(a.psi);
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const uint32_t tile_vec = (1u << a.t) / (F ? 2u : 1u);    // vectors per tile (>= 1: t >= 1)
+    const V *psi = reinterpret_cast<const V *>(a.psi) + (unsigned long long)blockIdx.y * a.ntiles * tile_vec;
     S U[E], X[NC ? NC * E : 1];
 #pragma unroll
     for (uint32_t e = 0; e < E; ++e) U[e].clear();
@@ -205,7 +207,7 @@ __global__ void __launch_bounds__(THREADS, NC >= 2 ? 1 : 2) z_sum(const __grid_c
         for (int c = 0; c < NC; ++c) acc += a.w[((size_t)(c + 1) << a.t) + k] * X[c * E + e].value();
     }
     const double r = block_sum(acc);
-    if (tid == 0) a.partial[blockIdx.x] = r;
+    if (tid == 0) a.partial[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = r;
 }
 
 // ---------------------------------------------------------------- strings with X or Y
@@ -466,14 +468,18 @@ struct Partials {
     }
 };
 
-int blocks_for(const sv_state *s, unsigned long long ntiles, unsigned per_sm = 2) {
-    return (int)std::min<unsigned long long>(ntiles, (unsigned long long)per_sm * (unsigned long long)s->num_sms);
+int blocks_for(const sv_state *s, unsigned long long ntiles) {
+    return (int)std::min<unsigned long long>(ntiles, 2ull * (unsigned long long)s->num_sms);
 }
 
-template <typename R>
-sv_status z_group(sv_state *s, Partials &P, const Term *t, size_t n) {
+// The Z strings t[0 .. n) on `states` states of nq qubits at psi, tables in `tables`: every pass
+// asks `reserve` where its partials go (blocks per state, state by state) and says with `ran`
+// that it has been enqueued.
+template <typename R, typename Reserve, typename Ran>
+sv_status z_passes(const void *psi, uint32_t nq, uint32_t states, int num_sms, cudaStream_t stream, double *tables,
+                   const Term *t, size_t n, Reserve reserve, Ran ran) {
     using namespace svx;
-    const uint32_t T = std::min(s->n, Geo<R>::T);
+    const uint32_t T = std::min(nq, Geo<R>::T);
     for (size_t b = 0; b < n; b += Z_TERMS) {
         const uint32_t m = (uint32_t)std::min<size_t>(Z_TERMS, n - b);
         const uint64_t lo = (1ull << T) - 1;
@@ -497,12 +503,11 @@ sv_status z_group(sv_state *s, Partials &P, const Term *t, size_t n) {
                 cls.push_back(z >> T);
             }
         }
-        a.psi = s->buf;
+        a.psi = psi;
         a.t = T;
-        a.ntiles = 1ull << (s->n - T);
-        // the tables lie in the top-k scratch (4 MiB), which no expectation uses
-        ta.w = reinterpret_cast<double *>(s->ws + WS_TOPK);
-        a.w = ta.w;
+        a.ntiles = 1ull << (nq - T);
+        ta.w = tables;
+        a.w = tables;
         size_t done = 0;
         bool first = true;
         while (first || done < cls.size()) {
@@ -512,27 +517,45 @@ sv_status z_group(sv_state *s, Partials &P, const Term *t, size_t n) {
             ta.ntab = 1 + nc;
             ta.zc[0] = 0;
             for (uint32_t c = 0; c < nc; ++c) ta.zc[1 + c] = a.zc[c] = cls[done + c];
-            const int nb = blocks_for(s, a.ntiles, nc >= 2 ? 1 : 2);
-            sv_status st = P.reserve(nb);
+            // as many blocks as the device holds, shared by the states
+            const unsigned long long slots = (unsigned long long)(nc >= 2 ? 1 : 2) * (unsigned long long)num_sms;
+            const int nb = (int)std::min<unsigned long long>(a.ntiles, std::max<unsigned long long>(1, slots / states));
+            sv_status st = reserve(nb, &a.partial);
             if (st != SV_OK) return st;
-            a.partial = P.part();
-            if (a.low || nc) {
-                SV_CUDA(svk::launch_pass(z_table, dim3((unsigned)(((1u << T) + 127) / 128), ta.ntab), 128, 0, s->stream, ta));
-            }
+            if (a.low || nc)
+                SV_CUDA(svk::launch_pass(z_table, dim3((unsigned)(((1u << T) + 127) / 128), ta.ntab), 128, 0, stream, ta));
+            const dim3 grid(nb, states);
             cudaError_t e = cudaSuccess;
             switch (nc) {
-                case 0: e = svk::launch_pass(z_sum<R, 0>, dim3(nb), THREADS, 0, s->stream, a); break;
-                case 1: e = svk::launch_pass(z_sum<R, 1>, dim3(nb), THREADS, 0, s->stream, a); break;
-                case 2: e = svk::launch_pass(z_sum<R, 2>, dim3(nb), THREADS, 0, s->stream, a); break;
-                default: e = svk::launch_pass(z_sum<R, 3>, dim3(nb), THREADS, 0, s->stream, a); break;
+                case 0: e = svk::launch_pass(z_sum<R, 0>, grid, THREADS, 0, stream, a); break;
+                case 1: e = svk::launch_pass(z_sum<R, 1>, grid, THREADS, 0, stream, a); break;
+                case 2: e = svk::launch_pass(z_sum<R, 2>, grid, THREADS, 0, stream, a); break;
+                default: e = svk::launch_pass(z_sum<R, 3>, grid, THREADS, 0, stream, a); break;
             }
             SV_CUDA(e);
-            P.used += nb;
+            st = ran(nb);
+            if (st != SV_OK) return st;
             done += nc;
             first = false;
         }
     }
     return SV_OK;
+}
+
+template <typename R>
+sv_status z_group(sv_state *s, Partials &P, const Term *t, size_t n) {
+    // the tables lie in the top-k scratch (4 MiB), which no expectation uses
+    return z_passes<R>(
+        s->buf, s->n, 1, s->num_sms, s->stream, reinterpret_cast<double *>(s->ws + WS_TOPK), t, n,
+        [&](int nb, double **out) {
+            const sv_status st = P.reserve(nb);
+            *out = P.part();
+            return st;
+        },
+        [&](int nb) {
+            P.used += nb;
+            return SV_OK;
+        });
 }
 
 // One x_sum pass: the tile's high bits H (ascending, above L), and the terms of `t` that are
@@ -678,6 +701,22 @@ sv_status x_group(sv_state *s, Partials &P, const std::vector<Term> &t) {
 }
 
 }  // namespace
+
+// Z strings on a batch: the tables (4 x 2^12 doubles) and `partial` (room for `room` doubles) are the
+// caller's; after each pass `fold` is called with the number of partials per state that lie there.
+sv_status batch_z_terms(const void *psi, uint32_t n, sv_dtype dtype, uint32_t states, int num_sms, cudaStream_t stream,
+                        double *tables, double *partial, size_t room, const uint64_t *z, const double *c, size_t nterms,
+                        const std::function<sv_status(int)> &fold) {
+    std::vector<Term> t(nterms);
+    for (size_t i = 0; i < nterms; ++i) t[i] = Term{0, z[i], c[i]};
+    auto reserve = [&](int nb, double **out) {
+        *out = partial;
+        return (size_t)nb * states <= room ? SV_OK : set_error(SV_ERR_ARG, "expectation: too few partials");
+    };
+    return dtype == SV_C64
+               ? z_passes<float>(psi, n, states, num_sms, stream, tables, t.data(), nterms, reserve, fold)
+               : z_passes<double>(psi, n, states, num_sms, stream, tables, t.data(), nterms, reserve, fold);
+}
 
 sv_status launch_expect(sv_state *s, const uint64_t *x, const uint64_t *z, const double *c,
                         size_t nterms, double *host_out) {

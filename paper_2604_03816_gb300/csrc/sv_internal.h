@@ -5,6 +5,7 @@
 
 #include <complex>
 #include <cstdint>
+#include <functional>
 #include <mutex>
 #include <string>
 #include <utility>
@@ -140,7 +141,9 @@ struct sv_batch_launch {
     int *err = nullptr;
     cudaStream_t stream = nullptr;
     int num_sms = 0;
-    bool tc = false;            // complex64 width 4/5 on the tensor cores (apply_tc.cu)
+    bool tc = false;            // complex64 on the tensor cores (apply_tc.cu): its operands
+    const void *images = nullptr;   // are packed first (launch_tc_pack)
+    const float *bscale = nullptr;
     uint32_t tile_bits = 0;     // CUDA-core passes: 2^tile_bits amplitudes per CTA (0: default)
 };
 
@@ -168,6 +171,12 @@ cudaError_t launch_pass(void (*kern)(P...), dim3 grid, unsigned block, size_t sm
 
 cudaError_t tc_batch_prepare();
 sv_status launch_tc_batch(const sv_batch_launch &L);
+// Operand images of `ngates` gates (L[i]; all with the same states and stream) into images,
+// gate by gate, tc_batch_image_bytes() each, and their scales into bscale; gate i's FP32 matrices
+// start tab_off[i] bytes into utab.
+size_t tc_batch_image_bytes();
+sv_status launch_tc_pack(const sv_batch_launch *L, const size_t *tab_off, uint32_t ngates, const void *utab,
+                         void *images, float *bscale);
 // `bytes` bytes at buf as a 2-D tensor of 128-byte rows for TMA tensor copies with the
 // 128-byte shared-memory swizzle; a segment of seg_bytes is *boxes boxes of *box_rows rows
 // (apply_tc.cu).  `map` points to a CUtensorMap.
@@ -210,6 +219,9 @@ sv_status launch_expect(sv_state *s, const uint64_t *x, const uint64_t *z, const
 sv_status enqueue_sum(sv_state *s, int n, double *dev_out);   // of the first n block partials
 sv_status enqueue_expect_group(sv_state *s, uint64_t x, const uint64_t *z, const double *c, int nterms,
                                double *dev_out);
+sv_status batch_z_terms(const void *psi, uint32_t n, sv_dtype dtype, uint32_t states, int num_sms, cudaStream_t stream,
+                        double *tables, double *partial, size_t room, const uint64_t *z, const double *c, size_t nterms,
+                        const std::function<sv_status(int)> &fold);
 sv_status launch_topk(sv_state *s, uint32_t k, uint64_t *idx, double *p);
 sv_status enqueue_topk(sv_state *s, double *host_p, unsigned long long *host_i);
 sv_status launch_widen(sv_state *s, const void *src_c64, void *dst_c128);

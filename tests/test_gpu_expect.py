@@ -93,3 +93,26 @@ def test_special_amplitudes(gpu, dtype):
     sv.sv_set_state(s, psi)
     assert sv.sv_expect(s, [0], [1], [1.0]) == np.inf
     s.free()
+
+
+@pytest.mark.parametrize("dtype", [0, 1])
+@pytest.mark.parametrize("n,count", [(3, 5), (11, 400), (13, 7), (15, 33)])
+def test_batch_energies(gpu, dtype, n, count):
+    """Z strings (inside, above and across a tile) and strings with X and Y, for every state."""
+    sv = gpu
+    import torch
+    import workloads as W
+    rng = np.random.default_rng(n)
+    fam = [W.hea(n, 2, rng=rng) for _ in range(min(count, 9))]
+    fused = [sv.sv_fuse(sv.gates_from_specs(f), n, 3) for f in fam]
+    b = sv.sv_batch_alloc(n, dtype, count, stream=torch.cuda.current_stream())
+    sv.sv_batch_apply(b, [fused[i % len(fused)] for i in range(count)])
+    z = [0] + [3 << i for i in range(n - 1)] + [int(v) for v in rng.integers(0, 1 << n, 40)] + [1, 0, 5]
+    x = [0] * (len(z) - 3) + [1, 1 << (n - 1), 3]
+    c = [float(v) for v in rng.normal(size=len(z))]
+    got = sv.sv_batch_expect(b, x, z, c)
+    tol = (2.0 ** -21 if dtype == 0 else 2.0 ** -45) * sum(abs(v) for v in c)
+    for i in list(range(min(count, 9))) + [count - 1]:
+        psi = sv.sv_batch_get_state(b, i).astype(np.complex128)
+        assert abs(got[i] - oracle.expect(psi, x, z, c)) < tol, i
+    b.free()
