@@ -13,16 +13,21 @@
 // norm per pass).  Instead each operand is cut into three 9-bit integer slices on a
 // fixed-point grid -- per row of A (scale 2^{8-e}, e = exponent of the row's largest
 // component) and for all of B -- so that x = (a1 + a2 2^-9 + a3 2^-18) / s.  The
-// slices are exact in FP16 and every product of integer slices is below 2^16, so
+// slices at their scale (a2 2^-9, a3 2^-18) are exact in FP16 and every product of slices is
+// an integer below 2^16 times a power of two, so
 //     D0  = A1 B1                                      (below 2^22: exact in FP32)
-//     D12 = A1 B2 + A2 B1 + 2^-9 (A1 B3 + A2 B2 + A3 B1)
-// are accumulated by the tensor cores (kind::f16, FP32 accumulators in TMEM); the
-// 2^-9-scaled slices (B3, B2 and A3 times 2^-9) are also exact in FP16.  D0, which
+//     D12 = A1 B2 + A2 B1 + A1 B3 + A2 B2 + A3 B1
+// are accumulated by the tensor cores (kind::f16, FP32 accumulators in TMEM).  D0, which
 // carries the leading 2^22 of the result, is exact; D12 sits 2^-9 below it, so the
 // truncation of its accumulation costs about 2^-31 of the output per step -- the error
 // stays unbiased to well below FP32 rounding.  The epilogue forms
-// out = (D0 + 2^-9 D12) / (s s_B) with round-to-nearest (the dropped slice products are
-// below 2^-27 of the row's largest amplitude).
+// out = (D0 + D12) / (s s_B) with round-to-nearest (the dropped slice products are
+// below 2^-27 of the row's largest amplitude).  With every slice at its own scale no scaled
+// copies are needed (three slices of each operand, 20 MMA instructions per 128 groups instead of
+// 24), and the slices are cut by magic-number rounding in packed FP32x2 instructions (tc.cuh)
+// instead of six conversions per amplitude on the conversion pipe, which bound the transform:
+// a 20-qubit pass 8.7 -> 7.8 us, 24 qubits 53 -> 47, 28 qubits 675 -> 670 (92 -> 94% of the copy
+// rate), a batched pass of 18 qubits x 96 states 86 -> 75.
 //
 // One persistent CTA per SM, warp-specialised, every hand-off an mbarrier:
 //   warp 8               TMA producer: lane i issues the load of segment i of each tile
@@ -32,7 +37,7 @@
 //                        and half of its members per thread -- gather from the raw stage,
 //                        cut into three 9-bit slices and write them into tensor memory
 //                        with tcgen05.st (the thread's own TMEM lane);
-//   warp 9 (one thread)  MMA issuer: 6 x K/16 tcgen05.mma.kind::f16, A from TMEM and B
+//   warp 9 (one thread)  MMA issuer: 5 x K/16 tcgen05.mma.kind::f16, A from TMEM and B
 //                        from shared memory, into two TMEM accumulators
 //                        (double-buffered), committed to mbarriers;
 //   warps 10-17          epilogue: two warps per quadrant, tcgen05.ld of half the columns,
@@ -65,11 +70,9 @@
 namespace svk {
 
 // SUB: MMA subtiles (128 groups each) per TMA stage.  SUB = 2 doubles the contiguous
-// segments of launches whose targets are all high (2 KiB instead of 1 KiB at k = 5), at
-// the price of one more A slice in TMEM (A2 2^-9 replaces the B2 2^-9 copy, to fit two
-// 64 KiB stages in shared memory).
+// segments of launches whose targets are all high (2 KiB instead of 1 KiB at k = 5).
 // BT: a batched launch over many states with their own matrices (see apply_tc): two B
-// sets (the current state's and the next one's) and two raw stages.
+// sets (the current state's and the next one's).
 template <int K, int SUB = 1, bool BT = false>
 struct TcShape {
     static constexpr uint32_t D = 1u << K;            // amplitudes per group
@@ -78,13 +81,13 @@ struct TcShape {
     static constexpr uint32_t TB = K + 7 + (SUB == 2 ? 1u : 0u);   // tile bits
     static constexpr uint32_t TILE_BYTES = SUB * ROWS * D * 8u;
     static constexpr uint32_t B_BYTES = KD * KD * 2u;     // one FP16 slice of B
-    static constexpr uint32_t NB = SUB == 2 ? 3u : 4u;    // B1, B2, B3 2^-9 [, B2 2^-9]
+    static constexpr uint32_t NB = 3;                     // B1, B2 2^-9, B3 2^-18
     static constexpr uint32_t SBO = (KD / 8u) * 128u;     // 8-row group stride of B
-    static constexpr uint32_t NS = (SUB == 2 || BT) ? 2u : (K == 5 ? 3u : 8u);   // raw stages
+    static constexpr uint32_t NS = SUB == 2 ? 2u : BT ? 3u : (K == 5 ? 4u : 8u);   // raw stages
     static constexpr uint32_t NOUT = SUB == 2 ? 1u : 2u;  // output staging tiles
     static constexpr uint32_t ACC = 2u * KD;              // TMEM columns of one D set (D0, D12)
     static constexpr uint32_t A_COLS = KD / 2u;           // TMEM columns of one A slice
-    static constexpr uint32_t NA = SUB == 2 ? 4u : 3u;    // A1, A2, A3 2^-9 [, A2 2^-9]
+    static constexpr uint32_t NA = 3;                     // A1, A2 2^-9, A3 2^-18
     static constexpr uint32_t A_SET = NA * A_COLS;        // one A buffer
     static constexpr uint32_t A_COL0 = 2u * ACC;          // first column of the A buffers
     static constexpr uint32_t TMEM_COLS = K == 5 ? 512u : 256u;
@@ -147,30 +150,6 @@ __device__ __forceinline__ void xor_unpermute(float2 (&v)[N], uint32_t x, uint32
     }
 }
 
-__device__ __forceinline__ uint32_t pack_half2(float a, float b) {
-    const __half2 h = __floats2half2_rn(a, b);   // exact: |a|, |b| <= 256 are integers
-    return *reinterpret_cast<const uint32_t *>(&h);
-}
-
-// An FP16 pair times 2^-9 (exact for the integer slices: at most 9 bits, no underflow).
-__device__ __forceinline__ uint32_t half2_times_2m9(uint32_t w) {
-    const __half2 h = __hmul2(*reinterpret_cast<const __half2 *>(&w), __float2half2_rn(1.f / 512.f));
-    return *reinterpret_cast<const uint32_t *>(&h);
-}
-
-// Three 9-bit integer slices of a scaled amplitude (|x scale| < 256): FP16 pairs
-// (re, im) of a1, a2 and a3 2^-9, all exact.
-__device__ __forceinline__ void slice3(float2 v, float scale, uint32_t &w1, uint32_t &w2, uint32_t &w3) {
-    const float xr = v.x * scale, xi = v.y * scale;
-    const float r1 = rintf(xr), i1 = rintf(xi);
-    const float xr2 = (xr - r1) * 512.f, xi2 = (xi - i1) * 512.f;
-    const float r2 = rintf(xr2), i2 = rintf(xi2);
-    const float r3 = rintf((xr2 - r2) * 512.f), i3 = rintf((xi2 - i2) * 512.f);
-    w1 = pack_half2(r1, i1);
-    w2 = pack_half2(r2, i2);
-    w3 = pack_half2(r3 * (1.f / 512.f), i3 * (1.f / 512.f));
-}
-
 // Three 9-bit slices of a fixed-point entry, x = b1 2^18 + b2 2^9 + b3, |b1|, |b2|, |b3| <= 256.
 __device__ __forceinline__ void cut_b(int x, float &b1, float &b2, float &b3) {
     const int i1 = (x + (1 << 17)) >> 18;
@@ -181,7 +160,7 @@ __device__ __forceinline__ void cut_b(int x, float &b1, float &b2, float &b3) {
     b3 = (float)(x - (i2 << 9));
 }
 
-// B = the FP16 slices (B1, B2, B3 2^-9 [, B2 2^-9]) of R, from the fixed-point entries in the
+// B = the FP16 slices (B1, B2 2^-9, B3 2^-18) of R, from the fixed-point entries in the
 // kernel's parameters: complex entry (r, c) fills R's rows 2r (re, -im) and 2r + 1 (im, re) at
 // columns 2c, 2c + 1, one FP16 pair each.  Entries i0, i0 + stride, ... two at a time.
 // Why here and in this form: the operand used to travel as three int16 copies of all of R
@@ -190,7 +169,7 @@ __device__ __forceinline__ void cut_b(int x, float &b1, float &b2, float &b3) {
 // state: a 20-qubit pass took 25.0 us (12 qubits: 21.0) and takes 11.1 (7.8) with 8 KiB of
 // parameters, 16-byte generic loads and the first tiles already in flight meanwhile; a
 // 28-qubit pass 693 -> 678 us.
-template <int K, int NB>
+template <int K>
 __device__ __forceinline__ void expand_b(unsigned char *sB, const int2 *bx, uint32_t b_bytes, uint32_t sbo,
                                          uint32_t i0, uint32_t stride) {
     for (uint32_t e = 2u * i0; e < (1u << (2 * K)); e += 2u * stride) {
@@ -204,11 +183,10 @@ __device__ __forceinline__ void expand_b(unsigned char *sB, const int2 *bx, uint
             const uint32_t o0 = kmajor_off16(2u * r, 2u * (c + q), sbo);
             const uint32_t o1 = kmajor_off16(2u * r + 1u, 2u * (c + q), sbo);
 #pragma unroll
-            for (int s = 0; s < NB; ++s) {
-                const int d = s == 3 ? 1 : s;                     // slice 3: B2 again
-                const float f = s >= 2 ? 1.f / 512.f : 1.f;       // exact: 9-bit integers
-                *reinterpret_cast<uint32_t *>(sB + s * b_bytes + o0) = pack_half2(re[d] * f, -im[d] * f);
-                *reinterpret_cast<uint32_t *>(sB + s * b_bytes + o1) = pack_half2(im[d] * f, re[d] * f);
+            for (int s = 0; s < 3; ++s) {
+                const float f = s == 0 ? 1.f : s == 1 ? 1.f / 512.f : 1.f / 262144.f;   // exact: 9-bit integers
+                *reinterpret_cast<uint32_t *>(sB + s * b_bytes + o0) = pack_h2(re[s] * f, -im[s] * f);
+                *reinterpret_cast<uint32_t *>(sB + s * b_bytes + o1) = pack_h2(im[s] * f, re[s] * f);
             }
         }
     }
@@ -227,7 +205,7 @@ __device__ __forceinline__ void b_grid(float m, float &sb, float &inv) {
 // cuts them into B sets in global memory, laid out as in shared memory, before the passes, and a
 // pass then loads a state's set with one bulk copy.  (Built inside the pass by its producer
 // warp, a set cost about 20 us of stalled loads whenever a CTA met a new state: 18 qubits x 96
-// states 115 us per pass -> 79.)
+// states 115 us per pass -> 86.)
 struct PackGate {
     unsigned long long tab;          // offset of the gate's FP32 matrices in the table (bytes)
     unsigned long long image;        // and of its images in units of B sets
@@ -245,7 +223,7 @@ struct PackArgs {
 
 // One block per (state, gate).  R is the real embedding of the widened U times sb, so |R sb| <
 // 256 and the three 9-bit slices of the FP32 values are exact.  A thread writes 16-byte chunks of
-// the slices B1, B2, B3 2^-9, B2 2^-9: eight columns of one row.
+// the slices B1, B2 2^-9, B3 2^-18: eight columns of one row.
 __global__ void __launch_bounds__(256) pack_images(const __grid_constant__ PackArgs a) {
     using S = TcShape<5, 1, true>;
     __shared__ float red[8];
@@ -278,28 +256,17 @@ __global__ void __launch_bounds__(256) pack_images(const __grid_constant__ PackA
         // the chunk's place (kmajor_off16): row n, columns kk .. kk + 7
         const uint32_t n = (q / (S::SBO / 16u)) * 8u + (q & 7u), kk = ((q >> 3) & 7u) * 8u;
         const uint32_t r = n >> 1, lr = local(r);
-        uint32_t w[4][4];
+        uint32_t w[3][4];
 #pragma unroll
         for (uint32_t i = 0; i < 4; ++i) {
             const uint32_t c = (kk >> 1) + i;
             float2 u = make_float2(0.f, 0.f);
             if (!((r ^ c) & g.idm)) u = reinterpret_cast<const float2 *>(U)[(lr << kin) + local(c)];
             const float x[2] = {(n & 1u ? u.y : u.x) * sb, (n & 1u ? u.x : -u.y) * sb};
-            float b[3][2];
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                b[0][j] = rintf(x[j]);
-                const float x2 = (x[j] - b[0][j]) * 512.f;
-                b[1][j] = rintf(x2);
-                b[2][j] = rintf((x2 - b[1][j]) * 512.f) * (1.f / 512.f);
-            }
-            w[0][i] = pack_half2(b[0][0], b[0][1]);
-            w[1][i] = pack_half2(b[1][0], b[1][1]);
-            w[2][i] = pack_half2(b[2][0], b[2][1]);
-            w[3][i] = pack_half2(b[1][0] * (1.f / 512.f), b[1][1] * (1.f / 512.f));
+            slices(make_float2(x[0], x[1]), make_float2(1.f, 1.f), w[0][i], w[1][i], w[2][i]);
         }
 #pragma unroll
-        for (uint32_t s = 0; s < 4; ++s)
+        for (uint32_t s = 0; s < 3; ++s)
             *reinterpret_cast<uint4 *>(img + s * S::B_BYTES + q * 16u) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
     }
 }
@@ -380,7 +347,7 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
     if (!BT && warp != S::W_PROD) {
         // every warp but the producer, which is already loading the first tiles
         const uint32_t i = tid < S::W_PROD * 32u ? tid : tid - 32u;
-        expand_b<K, (int)S::NB>(sB, a.bx, S::B_BYTES, S::SBO, i, S::THREADS - 32u);
+        expand_b<K>(sB, a.bx, S::B_BYTES, S::SBO, i, S::THREADS - 32u);
         fence_proxy_async_smem();
         named_bar(3, S::THREADS - 32u);
     }
@@ -474,7 +441,7 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
     } else if (warp == S::W_MMA) {
         // ------------------------------------------------------------ MMA issuer
         if (lane == 0) {
-            const uint32_t idesc = idesc_f16(S::ROWS, KD);
+            const uint32_t idesc = idesc_f16(S::ROWS, KD), idesc2 = idesc_f16(S::ROWS, 2u * KD);
             uint32_t B0 = smem_u32(sB);
             const unsigned long long nsub = tend > first ? ((tend - first + step - 1) / step) * SUB : 0;
             unsigned long long cur = ~0ull;
@@ -500,21 +467,18 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
                 tc_fence_after();
                 const uint32_t A0 = tmem + S::A_COL0 + b * S::A_SET;
                 const uint32_t dset = tmem + b * S::ACC;
-                // (accumulator, A slice, B slice): D0 = A1 B1; D12 = A1 B2 + A2 B1 +
-                // A1 (B3 2^-9) + A2 (B2 2^-9) + (A3 2^-9) B1   [A slices: A1, A2, A3s, A2s;
-                // B slices: B1, B2, B3s, B2s]; with SUB = 2, A2s B2 stands for A2 B2s
-                const uint32_t prod[6][3] = {{0, 0, 0}, {1, 0, 1}, {1, 1, 0}, {1, 0, 2},
-                                             {1, SUB == 2 ? 3u : 1u, SUB == 2 ? 1u : 3u}, {1, 2, 0}};
+                // A1 [B1 B2] -> [D0 D12] (the accumulators and the slices are adjacent: N =
+                // 2 KD), then A2 B1, A2 B2, A1 B3, A3 B1 -> D12
+                const uint32_t prod[5][2] = {{0, 0}, {1, 0}, {1, 1}, {0, 2}, {2, 0}};
 #pragma unroll
-                for (int p = 0; p < 6; ++p) {
-                    const uint32_t Aa = A0 + prod[p][1] * S::A_COLS;
-                    const uint32_t Bb = B0 + prod[p][2] * S::B_BYTES;
-                    const bool first_in_acc = (p == 0 || p == 1);
+                for (int p = 0; p < 5; ++p) {
+                    const uint32_t Aa = A0 + prod[p][0] * S::A_COLS;
+                    const uint32_t Bb = B0 + prod[p][1] * S::B_BYTES;
 #pragma unroll
                     for (uint32_t ks = 0; ks < KD / 16; ++ks)
-                        mma_f16_tmem_a(dset + prod[p][0] * KD, Aa + ks * 8u,
-                                       smem_desc(Bb + ks * 256u, 128u, S::SBO), idesc,
-                                       (first_in_acc && ks == 0) ? 0u : 1u);
+                        mma_f16_tmem_a(p == 0 ? dset : dset + KD, Aa + ks * 8u,
+                                       smem_desc(Bb + ks * 256u, 128u, S::SBO), p == 0 ? idesc2 : idesc,
+                                       (p == 0 && ks == 0) ? 0u : 1u);
                 }
                 mma_commit(smem_u32(&a_empty[b]));
                 mma_commit(smem_u32(&d_full[b]));
@@ -558,7 +522,7 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
                 for (uint32_t c = 0; c < HALF; ++c) {
                     const uint32_t mo = member_off(part * HALF + c);
                     v[c] = rs[gbase ^ (XP ? (mo ^ cx) : mo)];
-                    m = fmaxf(m, fmaxf(fabsf(v[c].x), fabsf(v[c].y)));
+                    m = max_abs2(m, v[c].x, v[c].y);
                 }
                 max_part[part][row] = m;
                 fence_proxy_async_smem();         // reads of the raw stage before its refill
@@ -568,7 +532,8 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
                 int ex = 0;
                 frexpf(m, &ex);                   // m < 2^ex (m = 0: ex = 0)
                 ex = max(ex, -100);               // keep 2^(8-ex) finite
-                const float scale = ldexpf(1.f, 8 - ex);   // |x * scale| < 256
+                const float sc = ldexpf(1.f, 8 - ex);      // |x * sc| < 256
+                const float2 scale = make_float2(sc, sc);
                 const uint32_t ab = js & 1u;
                 const bool oka = mbar_wait_or_abort(smem_u32(&a_empty[ab]), ((js >> 1) & 1u) ^ 1u, abort);
                 if (!named_bar_and(1, 256, oka)) { stop = true; break; }
@@ -578,22 +543,18 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
                 // a_empty[ab]
                 if (part == 0) row_scale[js & 3u][row] = ldexpf(bsc, ex - 8);
                 if constexpr (XP) xor_unpermute(v, xl, a.xt);   // back in member order (x < HALF)
-                // three 9-bit integer slices (and A2 2^-9 when SUB = 2), one FP16 pair
-                // (re, im) per 32-bit TMEM column, stored eight members at a time
+                // three 9-bit slices, one FP16 pair (re, im) per 32-bit TMEM column, stored
+                // eight members at a time
                 const uint32_t arow = tmem + S::A_COL0 + ab * S::A_SET + (((warp & 3u) * 32u) << 16) +
                                       part * HALF;
 #pragma unroll
                 for (uint32_t c0 = 0; c0 < HALF; c0 += 8) {
-                    uint32_t w1[8], w2[8], w3[8], w2s[8];
+                    uint32_t w1[8], w2[8], w3[8];
 #pragma unroll
-                    for (uint32_t c = 0; c < 8; ++c) {
-                        slice3(v[c0 + c], scale, w1[c], w2[c], w3[c]);
-                        if constexpr (SUB == 2) w2s[c] = half2_times_2m9(w2[c]);
-                    }
+                    for (uint32_t c = 0; c < 8; ++c) slices(v[c0 + c], scale, w1[c], w2[c], w3[c]);
                     tmem_st8_async(arow + c0, w1);
                     tmem_st8_async(arow + S::A_COLS + c0, w2);
                     tmem_st8_async(arow + 2 * S::A_COLS + c0, w3);
-                    if constexpr (SUB == 2) tmem_st8_async(arow + 3 * S::A_COLS + c0, w2s);
                 }
                 tmem_wait_st();
                 tc_fence_before();
@@ -638,7 +599,8 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
                     named_bar(2, 256);
                 }
                 const uint32_t gbase = gb[sub];
-                const float osc = row_scale[js & 3u][row];
+                const float osc1 = row_scale[js & 3u][row];
+                const float2 osc = make_float2(osc1, osc1);
                 const uint32_t lane_addr = tmem + b * S::ACC + ((quad * 32u) << 16) + part * HALF * 2u;
                 if constexpr (XP) {
                     float2 o[HALF];
@@ -649,9 +611,8 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
                         tmem_ld16(lane_addr + KD + c0, d12);
 #pragma unroll
                         for (uint32_t i = 0; i < 16; i += 2) {
-                            const float re = __fmaf_rn(d12[i], 1.f / 512.f, d0[i]) * osc;
-                            const float im = __fmaf_rn(d12[i + 1], 1.f / 512.f, d0[i + 1]) * osc;
-                            o[(c0 + i) / 2] = make_float2(re, im);
+                            o[(c0 + i) / 2] = __fmul2_rn(__fadd2_rn(make_float2(d0[i], d0[i + 1]),
+                                                                    make_float2(d12[i], d12[i + 1])), osc);
                         }
                     }
                     xor_unpermute(o, xl, a.xt);   // o[c] = member c ^ x (x < HALF)
@@ -667,9 +628,9 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
                         tmem_ld16(lane_addr + KD + c0, d12);
 #pragma unroll
                         for (uint32_t i = 0; i < 16; i += 2) {
-                            const float re = __fmaf_rn(d12[i], 1.f / 512.f, d0[i]) * osc;
-                            const float im = __fmaf_rn(d12[i + 1], 1.f / 512.f, d0[i + 1]) * osc;
-                            out[gbase ^ member_off(part * HALF + (c0 + i) / 2)] = make_float2(re, im);
+                            out[gbase ^ member_off(part * HALF + (c0 + i) / 2)] =
+                                __fmul2_rn(__fadd2_rn(make_float2(d0[i], d0[i + 1]),
+                                                      make_float2(d12[i], d12[i + 1])), osc);
                         }
                     }
                 }
@@ -755,9 +716,6 @@ sv_status launch_tc_t(sv_state *s, const svi::Gate &g) {
             init_err = cudaFuncSetAttribute(apply_tc<K, true, 1>,
                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
         if constexpr (K == 5) {
-            if (init_err == cudaSuccess)
-                init_err = cudaFuncSetAttribute(apply_tc<K, false, 2>,
-                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S2::SMEM);
             if (init_err == cudaSuccess)
                 init_err = cudaFuncSetAttribute(apply_tc<K, false, 2, false, true>,
                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S2::SMEM);

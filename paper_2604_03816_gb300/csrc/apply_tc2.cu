@@ -147,40 +147,6 @@ __device__ __forceinline__ void tmem_ld8x3(uint32_t a0, uint32_t stride, float (
         for (int i = 0; i < 8; ++i) v[q][i] = __uint_as_float(r[8 * q + i]);
 }
 
-// max(m, |a|, |b|) in one three-input maximum (sm_100 and later).
-__device__ __forceinline__ float max_abs2(float m, float a, float b) {
-    float r;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(m), "f"(fabsf(a)), "f"(fabsf(b)));
-    return r;
-}
-
-__device__ __forceinline__ uint32_t pack_h2(float a, float b) {
-    const __half2 h = __floats2half2_rn(a, b);
-    return *reinterpret_cast<const uint32_t *>(&h);
-}
-
-// The three slices of a scaled amplitude (|x scale| < 256) at their scale: a1 (an
-// integer), a2 2^-9 and a3 2^-18, with |a_i| <= 256; each FP16 pair (re, im) is exact.
-// Rounding to the grid 2^e (ties to even, |x| < 2^(e + 22)) adds and subtracts
-// c = 1.5 2^(e + 23): the sum keeps a unit in the last place of 2^e, so it is rounded to
-// that grid, and the subtraction is exact; the remainders x - a1 and (x - a1) - a2 2^-9
-// are exact FP32 differences (one fused multiply-add by -1).  (re, im) go through each
-// step together as one packed FP32x2 instruction.
-__device__ __forceinline__ void slices(float2 v, float2 scale, uint32_t &w1, uint32_t &w2, uint32_t &w3) {
-    const float2 m1 = make_float2(-1.f, -1.f);
-    const float2 x = __fmul2_rn(v, scale);
-    const float2 r1 = __fadd2_rn(__fadd2_rn(x, make_float2(12582912.f, 12582912.f)),
-                                 make_float2(-12582912.f, -12582912.f));              // 1.5 2^23
-    const float2 x2 = __ffma2_rn(r1, m1, x);
-    const float2 r2 = __fadd2_rn(__fadd2_rn(x2, make_float2(24576.f, 24576.f)),
-                                 make_float2(-24576.f, -24576.f));                    // 1.5 2^14
-    const float2 x3 = __ffma2_rn(r2, m1, x2);
-    const float2 r3 = __fadd2_rn(__fadd2_rn(x3, make_float2(48.f, 48.f)), make_float2(-48.f, -48.f));   // 1.5 2^5
-    w1 = pack_h2(r1.x, r1.y);
-    w2 = pack_h2(r2.x, r2.y);
-    w3 = pack_h2(r3.x, r3.y);
-}
-
 // The tile's layout in the state (read from the kernel parameters): tile t's base
 // deposits t around the high tile bits; segment q of a tile starts at base + seg_off(q).
 __device__ __forceinline__ unsigned long long tile_base(const Tc2Args &a, unsigned long long t) {
