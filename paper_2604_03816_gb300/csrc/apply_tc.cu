@@ -41,8 +41,12 @@
 //                        from shared memory, into two TMEM accumulators
 //                        (double-buffered), committed to mbarriers;
 //   warps 10-17          epilogue: two warps per quadrant, tcgen05.ld of half the columns,
-//                        combine, scatter into an output staging tile; warp 10 issues the
-//                        TMA bulk stores.
+//                        combine, scatter into an output staging tile;
+//   warp 18              issues the staging tiles' TMA bulk stores.
+// The epilogue warps never meet: they hand accumulators and staging tiles on by counted mbarrier
+// arrivals (an epilogue barrier and stores by one of its warps cost a batched pass of 18 qubits x
+// 96 states 4%, 75 -> 71 us).  The transform warps meet three times per subtile; letting them meet
+// in pairs instead measured the same within 1% (faster on 24-qubit states, slower on 28).
 // Targets among tile bits 0..3 (where 8-byte accesses pick their bank) would make the
 // lanes of a warp hit one bank.  Width-5 launches on states of 13 qubits or more, and
 // batched launches, avoid that with the swizzled staging (SW); the others (11- and
@@ -97,9 +101,9 @@ struct TcShape {
     static constexpr uint32_t OFF_RAW = NBSET * B_SET;
     static constexpr uint32_t OFF_OUT = OFF_RAW + NS * TILE_BYTES;
     static constexpr uint32_t SMEM = OFF_OUT + NOUT * TILE_BYTES;
-    static constexpr uint32_t THREADS = 576;              // 18 warps
-    // warps 0-7 transform, 8 TMA producer, 9 MMA issuer, 10-17 epilogue
-    static constexpr uint32_t W_PROD = 8, W_MMA = 9, W_EPI = 10;
+    static constexpr uint32_t THREADS = 608;              // 19 warps
+    // warps 0-7 transform, 8 TMA producer, 9 MMA issuer, 10-17 epilogue, 18 TMA stores
+    static constexpr uint32_t W_PROD = 8, W_MMA = 9, W_EPI = 10, W_STORE = 18;
     static constexpr uint32_t HALF = D / 2;               // group members per worker thread
 };
 
@@ -122,12 +126,12 @@ struct TcArgs {
     // bank-conflict avoidance: the xt lowest targets sit at tile bits below 4; lane l
     // takes group members in the order c ^ x(l), x(l) = (l >> xs) & (2^xt - 1)
     uint32_t xs, xt;
-    // batched launches: ntiles = states x tiles_per_state, state i at amplitude offset
+    // batched launches: ntiles = states x 2^tps tiles, state i at amplitude offset
     // i 2^n; state i's operand (the B set as it lies in shared memory) is images + i B_SET, its
     // scale bscale[i] (pack_images)
     const unsigned char *images;
     const float *bscale;
-    unsigned long long tiles_per_state;
+    uint32_t tps;                  // log2 of tiles_per_state
     uint32_t n;
 };
 
@@ -287,7 +291,7 @@ __global__ void __launch_bounds__(256) pack_images(const __grid_constant__ PackA
 // over XOR, so it is applied to the group base and to the target bits once, and member
 // offsets combine them by XOR.
 template <int K, bool XP, int SUB, bool BT = false, bool SW = false>
-__global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArgs<K> a) {
+__global__ void __launch_bounds__(608, 1) apply_tc(const __grid_constant__ TcArgs<K> a) {
     using S = TcShape<K, SUB, BT>;
     constexpr uint32_t KD = S::KD, NS = S::NS, NOUT = S::NOUT, HALF = S::HALF;
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -295,6 +299,7 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
     __shared__ __align__(8) unsigned long long a_full[2], a_empty[2], d_full[2], d_empty[2];
     __shared__ __align__(8) unsigned long long scale_full[4];   // row scales, tile j -> j & 3
     __shared__ float row_scale[4][128];
+    __shared__ __align__(8) unsigned long long out_full[NOUT], out_free[NOUT];   // staging tiles
     __shared__ float max_part[2][128];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
@@ -323,9 +328,13 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
             mbar_init(smem_u32(&a_full[b]), 1);
             mbar_init(smem_u32(&a_empty[b]), 1);
             mbar_init(smem_u32(&d_full[b]), 1);
-            mbar_init(smem_u32(&d_empty[b]), 1);
+            mbar_init(smem_u32(&d_empty[b]), 8);      // the epilogue warps
         }
         for (int q = 0; q < 4; ++q) mbar_init(smem_u32(&scale_full[q]), 1);
+        for (uint32_t o = 0; o < NOUT; ++o) {
+            mbar_init(smem_u32(&out_full[o]), 8);
+            mbar_init(smem_u32(&out_free[o]), 1);
+        }
         for (int q = 0; q < 2; ++q) {
             mbar_init(smem_u32(&b_full[q]), 1);
             mbar_init(smem_u32(&b_empty[q]), 1);
@@ -356,8 +365,8 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
     // amplitude offset of tile t (batched: the state's offset plus the tile's base)
     auto tile_base = [&](const SegLanes &sl, unsigned long long t) -> unsigned long long {
         if constexpr (BT) {
-            const unsigned long long st = t / a.tiles_per_state;
-            return (st << a.n) + sl.base(t - st * a.tiles_per_state);
+            const unsigned long long st = t >> a.tps;
+            return (st << a.n) + sl.base(t - (st << a.tps));
         } else {
             return sl.base(t);
         }
@@ -391,7 +400,7 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
         pass_wait();
         uint32_t j = 0;
         // batched: B sets are requested state by state, from the range's first one
-        const unsigned long long st0 = BT ? first / a.tiles_per_state : 0;
+        const unsigned long long st0 = BT ? first >> a.tps : 0;
         unsigned long long asked = st0;
         auto ask = [&]() -> bool {
             const uint32_t i = (uint32_t)(asked - st0), set = i & 1u, use = i >> 1;
@@ -409,11 +418,11 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
         };
         for (unsigned long long t = first; t < tend; t += step, ++j) {
             if constexpr (BT) {
-                const unsigned long long st = t / a.tiles_per_state, in = t - st * a.tiles_per_state;
+                const unsigned long long st = t >> a.tps, in = t - (st << a.tps);
                 if (asked <= st && !ask()) break;
                 // the next state's set, once the previous state's last MMAs must be done (its
                 // tiles left the raw stages), or at the last tile of this one
-                if (asked == st + 1 && (in >= 3 || in + 1 == a.tiles_per_state) && asked * a.tiles_per_state < tend &&
+                if (asked == st + 1 && (in >= 3 || in + 1 == 1ull << a.tps) && (asked << a.tps) < tend &&
                     !ask())
                     break;
             }
@@ -448,7 +457,7 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
             uint32_t nsw = 0;
             for (unsigned long long js = 0; js < nsub; ++js) {
                 if constexpr (BT) {
-                    const unsigned long long st = (first + (js / SUB) * step) / a.tiles_per_state;
+                    const unsigned long long st = (first + (js / SUB) * step) >> a.tps;
                     if (st != cur) {
                         if (cur != ~0ull) {
                             mma_commit(smem_u32(&b_empty[nsw & 1u]));   // the old state's MMAs
@@ -506,7 +515,7 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
             const uint32_t s = j % NS;
             const bool okf = mbar_wait_or_abort(smem_u32(&full[s]), (j / NS) & 1u, abort);
             if constexpr (BT) {
-                const unsigned long long st = t / a.tiles_per_state;
+                const unsigned long long st = t >> a.tps;
                 if (st != cur) bsc = __ldcg(a.bscale + st);       // after the first tile's arrival
                 cur = st;
             }
@@ -565,13 +574,12 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
                 }
             }
         }
-    } else if (warp >= S::W_EPI) {
+    } else if (warp < S::W_STORE) {
         // ------------------------------------------------------------ epilogue
         // Two warps per lane quadrant, each over half of the accumulator columns.
         const uint32_t quad = warp & 3u;          // TMEM lanes 32*quad .. 32*quad+31
         const uint32_t row = quad * 32u + lane;
-        const uint32_t et = tid - S::W_EPI * 32u; // 0..255 within the epilogue warps
-        const uint32_t part = et >> 7;
+        const uint32_t part = (warp - S::W_EPI) >> 2;
         uint32_t gb[SUB];
 #pragma unroll
         for (uint32_t sub = 0; sub < SUB; ++sub) gb[sub] = group_base(sub * S::ROWS + row);
@@ -580,82 +588,82 @@ __global__ void __launch_bounds__(576, 1) apply_tc(const __grid_constant__ TcArg
 #pragma unroll
         for (int q = 0; q < K; ++q)
             if ((xl >> q) & 1u) cx |= tbit[q];
-        SegLanes sl;                              // the first epilogue warp stores segments
-        sl.init(a.L, a.h, a.hi, lane);
         uint32_t j = 0;
-        bool stop = false;
-        for (unsigned long long t = first; t < tend && !stop; t += step, ++j) {
+        bool ok = true;
+        for (unsigned long long t = first; t < tend && ok; t += step, ++j) {
             const uint32_t ob = j % NOUT;
             float2 *out = reinterpret_cast<float2 *>(smem + S::OFF_OUT + ob * S::TILE_BYTES);
 #pragma unroll
             for (uint32_t sub = 0; sub < SUB; ++sub) {
                 const uint32_t js = j * SUB + sub, b = js & 1u;
-                bool ok = mbar_wait_or_abort(smem_u32(&d_full[b]), (js >> 1) & 1u, abort);
+                ok = ok && mbar_wait_or_abort(smem_u32(&d_full[b]), (js >> 1) & 1u, abort);
                 ok = ok && mbar_wait_or_abort(smem_u32(&scale_full[js & 3u]), (js >> 2) & 1u, abort);
-                if (!named_bar_and(2, 256, ok)) { stop = true; break; }
+                if (sub == 0) ok = ok && mbar_wait_or_abort(smem_u32(&out_free[ob]), ((j / NOUT) & 1u) ^ 1u, abort);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
                 tc_fence_after();
-                if (sub == 0) {
-                    if (et < 32) bulk_wait_read<(int)NOUT - 1>();   // this staging tile is free
-                    named_bar(2, 256);
-                }
                 const uint32_t gbase = gb[sub];
                 const float osc1 = row_scale[js & 3u][row];
                 const float2 osc = make_float2(osc1, osc1);
                 const uint32_t lane_addr = tmem + b * S::ACC + ((quad * 32u) << 16) + part * HALF * 2u;
-                if constexpr (XP) {
-                    float2 o[HALF];
+                float2 o[XP ? HALF : 1];
 #pragma unroll
-                    for (uint32_t c0 = 0; c0 < 2u * HALF; c0 += 16) {
-                        float d0[16], d12[16];
-                        tmem_ld16(lane_addr + c0, d0);
-                        tmem_ld16(lane_addr + KD + c0, d12);
+                for (uint32_t c0 = 0; c0 < 2u * HALF; c0 += 16) {
+                    float d0[16], d12[16];
+                    tmem_ld16x2(lane_addr + c0, lane_addr + KD + c0, d0, d12);
 #pragma unroll
-                        for (uint32_t i = 0; i < 16; i += 2) {
-                            o[(c0 + i) / 2] = __fmul2_rn(__fadd2_rn(make_float2(d0[i], d0[i + 1]),
-                                                                    make_float2(d12[i], d12[i + 1])), osc);
-                        }
-                    }
-                    xor_unpermute(o, xl, a.xt);   // o[c] = member c ^ x (x < HALF)
-#pragma unroll
-                    for (uint32_t c = 0; c < HALF; ++c) out[gbase ^ member_off(part * HALF + c) ^ cx] = o[c];
-                } else {
-                    // member order: each chunk of eight members is written as soon as it is
-                    // formed (fewer live registers than holding the half row)
-#pragma unroll
-                    for (uint32_t c0 = 0; c0 < 2u * HALF; c0 += 16) {
-                        float d0[16], d12[16];
-                        tmem_ld16(lane_addr + c0, d0);
-                        tmem_ld16(lane_addr + KD + c0, d12);
-#pragma unroll
-                        for (uint32_t i = 0; i < 16; i += 2) {
-                            out[gbase ^ member_off(part * HALF + (c0 + i) / 2)] =
-                                __fmul2_rn(__fadd2_rn(make_float2(d0[i], d0[i + 1]),
-                                                      make_float2(d12[i], d12[i + 1])), osc);
-                        }
+                    for (uint32_t i = 0; i < 16; i += 2) {
+                        const float2 x = __fmul2_rn(__fadd2_rn(make_float2(d0[i], d0[i + 1]),
+                                                               make_float2(d12[i], d12[i + 1])), osc);
+                        // in member order each chunk of eight members is written as soon as it
+                        // is formed (fewer live registers than holding the half row)
+                        if constexpr (XP) o[(c0 + i) / 2] = x;
+                        else out[gbase ^ member_off(part * HALF + (c0 + i) / 2)] = x;
                     }
                 }
                 tc_fence_before();
-                fence_proxy_async_smem();
-                named_bar(2, 256);
-                if (et == 0) mbar_arrive(smem_u32(&d_empty[b]));
-            }
-            if (stop) break;
-            if (et < 32) {
-                if (lane < nseg) {
-                    if constexpr (SW) {
-                        const int32_t row0 = (int32_t)((tile_base(sl, t) + sl.my_off) >> 4);
-                        const uint32_t s0 = smem_u32(out + (size_t)lane * seg_amps);
-                        for (uint32_t bx = 0; bx < a.boxes; ++bx)
-                            tma_store_2d(&a.tmap, 0, row0 + (int32_t)(bx * a.box_rows), s0 + bx * a.box_rows * 128u);
-                    } else {
-                        bulk_s2g(psi + tile_base(sl, t) + sl.my_off, smem_u32(out + (size_t)lane * seg_amps),
-                                 seg_bytes);
-                    }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&d_empty[b]));
+                if constexpr (XP) {
+                    xor_unpermute(o, xl, a.xt);   // o[c] = member c ^ x (x < HALF)
+#pragma unroll
+                    for (uint32_t c = 0; c < HALF; ++c) out[gbase ^ member_off(part * HALF + c) ^ cx] = o[c];
                 }
-                bulk_commit();
             }
+            if (!ok) break;
+            fence_proxy_async_smem();             // the bulk store reads them
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&out_full[ob]));
         }
-        if (et < 32) bulk_wait_all();
+    } else {
+        // ------------------------------------------------------------ TMA stores
+        // lane i stores segment i of every tile
+        SegLanes sl;
+        sl.init(a.L, a.h, a.hi, lane);
+        uint32_t j = 0;
+        for (unsigned long long t = first; t < tend; t += step, ++j) {
+            const uint32_t ob = j % NOUT;
+            const float2 *out = reinterpret_cast<const float2 *>(smem + S::OFF_OUT + ob * S::TILE_BYTES);
+            const bool ok = mbar_wait_or_abort(smem_u32(&out_full[ob]), (j / NOUT) & 1u, abort);
+            if (!__all_sync(0xffffffffu, ok)) break;
+            if (lane < nseg) {
+                if constexpr (SW) {
+                    const int32_t row0 = (int32_t)((tile_base(sl, t) + sl.my_off) >> 4);
+                    const uint32_t s0 = smem_u32(out + (size_t)lane * seg_amps);
+                    for (uint32_t bx = 0; bx < a.boxes; ++bx)
+                        tma_store_2d(&a.tmap, 0, row0 + (int32_t)(bx * a.box_rows), s0 + bx * a.box_rows * 128u);
+                } else {
+                    bulk_s2g(psi + tile_base(sl, t) + sl.my_off, smem_u32(out + (size_t)lane * seg_amps),
+                             seg_bytes);
+                }
+            }
+            bulk_commit();
+            // tile j - (NOUT - 1) has been read out
+            bulk_wait_read<(int)NOUT - 1>();
+            __syncwarp();
+            if (lane == 0 && j + 1 >= NOUT) mbar_arrive(smem_u32(&out_free[(j + 1u - NOUT) % NOUT]));
+        }
+        bulk_wait_all();
     }
     if (tid == 0 && abort_flag) atomicOr(a.err, 2);
     tc_fence_before();
@@ -876,7 +884,7 @@ sv_status launch_tc_batch(const sv_batch_launch &L) {
     a.xt = 0;
     a.images = static_cast<const unsigned char *>(L.images);
     a.bscale = L.bscale;
-    a.tiles_per_state = p.ntiles;
+    a.tps = (uint32_t)__builtin_ctzll(p.ntiles);
     a.n = L.n;
     const unsigned grid = (unsigned)std::min<unsigned long long>(a.ntiles, (unsigned long long)L.num_sms);
     SV_CUDA(launch_pass(apply_tc<5, false, 1, true, true>, dim3(grid), S::THREADS, S::SMEM, L.stream, a));
