@@ -725,6 +725,9 @@ sv_status launch_tc_t(sv_state *s, const svi::Gate &g) {
                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
         if constexpr (K == 5) {
             if (init_err == cudaSuccess)
+                init_err = cudaFuncSetAttribute(apply_tc<K, false, 1, false, true>,
+                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
+            if (init_err == cudaSuccess)
                 init_err = cudaFuncSetAttribute(apply_tc<K, false, 2, false, true>,
                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S2::SMEM);
         }
@@ -739,12 +742,13 @@ sv_status launch_tc_t(sv_state *s, const svi::Gate &g) {
     // width 5 on states of at least 13 qubits: two subtiles per stage (segments twice as
     // long, half the per-stage work) with the swizzled tensor-map staging, whatever the
     // targets (no XOR member order); otherwise one subtile, XOR order for bank-bit targets
+    // (one subtile while every SM has at most eight tiles, up to 22 qubits: a pass is then a few
+    // tiles' latency, and a second subtile adds to it: 18 qubits 7.25 -> 5.54 us per pass, 20
+    // qubits 7.83 -> 7.34, 22 qubits 15.1 -> 14.4; from 23 qubits two subtiles are as fast or faster)
     const bool swz = K == 5 && s->n >= S2::TB;
-    const bool wide = swz;
-    if (wide) {
-        p = make_plan(s->n, K, g.t, S2::TB);
-        tl = 0;
-    }
+    const bool wide = swz && p.ntiles > 8ull * (unsigned long long)s->num_sms;
+    if (wide) p = make_plan(s->n, K, g.t, S2::TB);
+    if (swz) tl = 0;
     TcArgs<K> a;
     a.box_rows = a.boxes = 0;
     if (swz) {
@@ -782,7 +786,9 @@ sv_status launch_tc_t(sv_state *s, const svi::Gate &g) {
     const unsigned grid = (unsigned)std::min<unsigned long long>(p.ntiles, (unsigned long long)s->num_sms);
     cudaError_t e = cudaSuccess;
     // with eight worker warps per role the permutation costs less than even 2-way conflicts
-    if (swz) {
+    if (swz && !wide) {
+        if constexpr (K == 5) e = launch_pass(apply_tc<K, false, 1, false, true>, dim3(grid), S::THREADS, S::SMEM, s->stream, a);
+    } else if (swz) {
         if constexpr (K == 5) e = launch_pass(apply_tc<K, false, 2, false, true>, dim3(grid), S2::THREADS, S2::SMEM, s->stream, a);
     } else if (a.xt >= 1) {
         e = launch_pass(apply_tc<K, true, 1>, dim3(grid), S::THREADS, S::SMEM, s->stream, a);
