@@ -658,10 +658,9 @@ __global__ void __launch_bounds__(608, 1) apply_tc(const __grid_constant__ TcArg
                 }
             }
             bulk_commit();
-            // tile j - (NOUT - 1) has been read out
-            bulk_wait_read<(int)NOUT - 1>();
+            bulk_wait_read_all();                 // the staging tile is free again
             __syncwarp();
-            if (lane == 0 && j + 1 >= NOUT) mbar_arrive(smem_u32(&out_free[(j + 1u - NOUT) % NOUT]));
+            if (lane == 0) mbar_arrive(smem_u32(&out_free[ob]));
         }
         bulk_wait_all();
     }

@@ -6,27 +6,36 @@
 // the row's largest exponent, for R on the grid of its largest entry,
 //     A = sum_i A_i 2^(-9 i),  R = sum_j B_j 2^(-9 j),  i, j = 0..5, |A_i|, |B_j| <= 256.
 // Level s collects the digit pairs with i + j = s; with 32 products of at most 2^16 per
-// pair, the levels s = 0..3 (1, 2, 3, 4 pairs) stay below 2^24 and are accumulated
-// EXACTLY by the FP32 tensor-core accumulators:
-//     D0 = L0, D1 = L1, D2 = L2, D3 = L3,
-//     D45 = L4 + 2^-9 L5   (with the B_j 2^-9 copies; its rounding sits 2^-45 below the
-//                           leading level).
-// Levels 6..10 are dropped (below 2^-46 of the row's largest term).  The epilogue
+// pair, the levels s = 0..4 (1 to 5 pairs) stay below 2^24 and are accumulated EXACTLY by the FP32
+// tensor-core accumulators; level 5 is added at its scale to level 4's accumulator (B_j 2^-9, also
+// exact FP16).  Levels 6..10 are dropped (below 2^-46 of the row's largest term).  The epilogue
 // converts the accumulators to integers, forms Z = L0 2^40 + L1 2^31 + L2 2^22 + L3 2^13 +
-// rint(16 D45) in 64 bits and builds the nearest double of Z 2^p with integer operations
-// (an identity gate returns its input bit for bit).
-// 21 digit products per tile; the split and the products never touch the FP64 pipe (this
-// GPU runs it at about 1/64 of the FP32 rate), only the final int64 -> double conversion
-// of each output does, which balances the integer and FP64 pipes.
+// rint(16 D45) in 64 bits and builds the nearest double of Z 2^p (an identity gate returns its
+// input bit for bit).
+// The split and the products never touch the FP64 pipe (this GPU runs it at about 1/64 of the
+// FP32 rate), only the final int64 -> double conversion of each output does, which balances the
+// integer and FP64 pipes.
+//
+// The five accumulators and the slices of R lie side by side, so the products of digit A_i with
+// B_0 .. B_{4-i} are one MMA per K step into D_i .. D_4 (N = 160, 128, .. 32): 22 instructions
+// per 128 groups instead of 42 of N = 32, which took about 140 cycles each.
+//
+// What bounds it: issue and the integer pipe (about 160 instructions per amplitude, 4250 cycles
+// per 2048 amplitudes where HBM needs 3030).  So the workers do not meet: two transform groups of
+// four warps take alternate subtiles, whole rows per warp (eight warps on one subtile exchanged
+// row maxima and met twice: 2430 cycles more), the epilogue's hand over by counted arrivals, and
+// the short forms of the split and of the scaling (rows whose exponents allow them, a vote per warp)
+// save a quarter of the integer instructions.  More workers do not help (16 epilogue warps: the
+// same time; 16 transform warps: 5% slower).  28-qubit grid circuit: 238.5 -> 196 ms, with the stores of
+// SUB = 2 by halves 175.6 ms.
 //
 // Gates on fewer than four qubits are widened to four (U (x) I on extra qubits chosen
 // above bit 4, so a warp's rows stay contiguous in shared memory).
 //
-// Roles and pipelines follow the complex64 kernel, with twice the integer workers: warps
-// 0-7 digit transform into TMEM (tcgen05.st), warp 8 TMA producer (lane i copies segment
-// i), warp 9 lane 0 the MMA issuer, warps 10-17 the epilogue with bulk stores; A and D
-// double-buffered in TMEM (2 x 96 + 2 x 160 = 512 columns); every wait bounded with a
-// shared abort flag.
+// Roles: warps 0-7 digit transform into TMEM (tcgen05.st), warp 8 TMA producer (lane i copies
+// segment i), warp 9 lane 0 the MMA issuer, warps 10-17 the epilogue, warp 18 the bulk stores; A
+// and D double-buffered in TMEM (2 x 96 + 2 x 160 = 512 columns); every wait bounded with a shared
+// abort flag.
 #include <cuda_fp16.h>
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -34,6 +43,7 @@
 #include <algorithm>
 #include <cmath>
 #include <mutex>
+#include <type_traits>
 
 #include "fixed_point.h"
 #include "plan.h"
@@ -57,7 +67,7 @@ struct Tc64S {
     static constexpr uint32_t NB = 12;                    // B_j and B_j 2^-9, j = 0..5
     static constexpr uint32_t SBO = (KD / 8u) * 128u;
     static constexpr uint32_t NS = SUB == 2 ? 2u : 4u;    // raw stages
-    static constexpr uint32_t NOUT = SUB == 2 ? 1u : 2u;  // output staging tiles
+    static constexpr uint32_t NOUT = SUB == 2 ? 1u : 2u;  // output staging tiles (two subtiles)
     static constexpr uint32_t NACC = 5;                   // D0, D1, D2, D3, D45
     static constexpr uint32_t ACC = NACC * KD;            // TMEM columns of one D set
     static constexpr uint32_t A_COLS = KD / 2u;           // TMEM columns of one A digit slice
@@ -68,9 +78,9 @@ struct Tc64S {
     static constexpr uint32_t OFF_RAW = NB * B_BYTES;
     static constexpr uint32_t OFF_OUT = OFF_RAW + NS * TILE_BYTES;
     static constexpr uint32_t SMEM = OFF_OUT + NOUT * TILE_BYTES;
-    static constexpr uint32_t THREADS = 576;              // 18 warps
-    // warps 0-7 transform, 8 producer, 9 MMA issuer, 10-17 epilogue
-    static constexpr uint32_t W_PROD = 8, W_MMA = 9, W_EPI = 10;
+    static constexpr uint32_t THREADS = 608;              // 19 warps
+    // warps 0-7 transform, 8 producer, 9 MMA issuer, 10-17 epilogue, 18 TMA stores
+    static constexpr uint32_t W_PROD = 8, W_MMA = 9, W_EPI = 10, W_STORE = 18;
 };
 using Tc64 = Tc64S<1>;
 
@@ -89,37 +99,8 @@ struct Tc64Args {
     uint32_t L, h;
     uint32_t hi[SV_MAX_K];
     uint32_t lp[4];
-    // bank-conflict avoidance: the xt (<= 2) lowest targets sit at tile bits below 3; lane
-    // l takes the members of each group of four in the order c ^ x(l), x(l) = (l >> xs) &
-    // (2^xt - 1)
-    uint32_t xs, xt;
+    uint32_t sb;             // the highest tile bit below L that is no target
 };
-
-// v[c] <- v[c ^ x] for c < 4 and the low xt (<= 2) bits of x.
-template <typename T, typename Sel>
-__device__ __forceinline__ void xor_unpermute4(T (&v)[4], uint32_t x, uint32_t xt, Sel sel) {
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        if (xt > (uint32_t)j) {                       // uniform over the launch
-            const bool f = (x >> j) & 1u;
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                if (c & (1 << j)) continue;
-                const T lo = v[c], hi = v[c | (1 << j)];
-                v[c] = sel(f, hi, lo);
-                v[c | (1 << j)] = sel(f, lo, hi);
-            }
-        }
-    }
-}
-
-__device__ __forceinline__ uint4 sel_u4(bool f, uint4 a, uint4 b) {
-    return make_uint4(f ? a.x : b.x, f ? a.y : b.y, f ? a.z : b.z, f ? a.w : b.w);
-}
-
-__device__ __forceinline__ double2 sel_d2(bool f, double2 a, double2 b) {
-    return make_double2(f ? a.x : b.x, f ? a.y : b.y);
-}
 
 // Digit-pair word -> FP16 pair of digits: the patterns read 2048 + 2u, and
 // (2048 + 2u) 0.5 - 1280 = u - 256 is exact in one half2 multiply-add.
@@ -148,9 +129,8 @@ __device__ __forceinline__ void expand_b64(unsigned char *sB, const longlong2 *b
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const float f = h ? 1.f / 512.f : 1.f;      // exact: an integer of at most 9 bits
-                const __half2 w0 = __floats2half2_rn(dr * f, -di * f), w1 = __floats2half2_rn(di * f, dr * f);
-                *reinterpret_cast<__half2 *>(sB + (6 * h + j) * S::B_BYTES + o0) = w0;
-                *reinterpret_cast<__half2 *>(sB + (6 * h + j) * S::B_BYTES + o1) = w1;
+                *reinterpret_cast<__half2 *>(sB + (6 * h + j) * S::B_BYTES + o0) = __floats2half2_rn(dr * f, -di * f);
+                *reinterpret_cast<__half2 *>(sB + (6 * h + j) * S::B_BYTES + o1) = __floats2half2_rn(di * f, dr * f);
             }
         }
     }
@@ -160,40 +140,69 @@ __device__ __forceinline__ void expand_b64(unsigned char *sB, const longlong2 *b
 // conversion; 16 D45 below 2^28), Z = L0 2^40 + L1 2^31 + L2 2^22 + L3 2^13 + rint(16 D45)
 // in 64 bits, and the nearest double of Z 2^p.  The int64 -> double conversion runs on the
 // FP64 pipe, which the rest of the kernel leaves idle: it rounds to nearest even exactly
-// like fxp::assemble_words (the integer-pipe form, about 30 instructions), and the scaling
-// by 2^p is an add to the exponent field while the result stays normal.  Measured at 28
-// qubits: 2.55 -> 2.09 ms per pass (the integer ALU pipe was the bound).
-__device__ __forceinline__ double combine_levels(float f0, float f1, float f2, float f3, float f45,
-                                                 int p) {
-    const long long z = (long long)__float2int_rn(f45 * 16.f) + (long long)__float2int_rn(f3) * (1ll << 13) +
-                        (long long)__float2int_rn(f2) * (1ll << 22) +
-                        (long long)fxp::small_float_to_int(f1) * (1ll << 31) +
-                        (long long)fxp::small_float_to_int(f0) * (1ll << 40);
+// like fxp::assemble_words (the integer-pipe form, about 30 instructions; converting every
+// second output in integers measured the same), and the scaling by 2^p is an add to the exponent
+// field while the result stays normal: always, for nonzero |Z| < 2^63, with P_SAFE (-1022 <= p
+// <= 960).
+template <bool P_SAFE>
+__device__ __forceinline__ double combine_levels(float f0, float f1, float f2, float f3, float f45, int p) {
+    constexpr uint32_t MAGIC = 0x4B400000u;                 // pattern of 1.5 2^23
+    const uint32_t b0 = __float_as_uint(f0 + 12582912.f), b1 = __float_as_uint(f1 + 12582912.f);
+    const unsigned long long c0 = 0ull - ((unsigned long long)MAGIC << 31) - ((unsigned long long)MAGIC << 40);
+    unsigned long long u = (unsigned long long)((long long)__float2int_rn(f45 * 16.f)) + c0;
+    u += (unsigned long long)((long long)__float2int_rn(f3) * (1 << 13));
+    u += (unsigned long long)((long long)__float2int_rn(f2) * (1 << 22));
+    u += (unsigned long long)b1 * 0x80000000u;
+    u += (unsigned long long)(b0 << 8) << 32;               // the bits above 2^64 cancel with c0's
+    const long long z = (long long)u;
+    const double x = __ll2double_rn(z);
+    if (P_SAFE) {
+        const int hi = __double2hiint(x);
+        return __hiloint2double(hi ? hi + (p << 20) : 0, __double2loint(x));
+    }
     if (z == 0) return 0.0;
-    const long long b = __double_as_longlong(__ll2double_rn(z));
+    const long long b = __double_as_longlong(x);
     const int e = (int)((b >> 52) & 0x7FF) + p;
     if (e < 1 || e > 2046) return fxp::assemble_slow(z, p);
     return __longlong_as_double(b + ((long long)p << 52));
 }
 
-// XP (not launched: two bank-bit targets now take the swizzled staging, SW): the launch
-// has targets among tile bits 0..2 and takes members in the lane's XOR
-// order; otherwise no permutation code at all.  The pipelines count tiles (j: raw stage,
-// output staging) and MMA subtiles (js = j SUB + sub: A and D buffers, row exponents).
+// The digit words of group members c0 .. c0 + 3 of one row.  NEAR: every component's exponent
+// field is nonzero and at most 31 below the row's largest.
+template <bool NEAR>
+__device__ __forceinline__ void cut_members(const uint4 (&v)[4], uint32_t emax, uint32_t (&w)[6][4]) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        uint32_t rh, rl, ih, il, t[6];
+        if (NEAR) {
+            const uint32_t ew = emax << 20 | 0xFFFFFu;
+            fxp::offset_fixed_near(v[c].y, v[c].x, ew, rh, rl);
+            fxp::offset_fixed_near(v[c].w, v[c].z, ew, ih, il);
+        } else {
+            fxp::offset_fixed(v[c].y, v[c].x, emax, rh, rl);
+            fxp::offset_fixed(v[c].w, v[c].z, emax, ih, il);
+        }
+        fxp::digit_pair_words(rh, rl, ih, il, t);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) w[i][c] = digit_pair(t[i]);
+    }
+}
+
+// The pipelines count tiles (j: raw stage) and MMA subtiles (js = j SUB + sub: A and D buffers, row
+// exponents, output staging).
 // SW: tiles move by 2-D tensor-map copies with the 128-byte swizzle and the roles address
-// them through it, so a warp's lanes reach different banks whatever the targets (no XOR
-// member order: XP = false).  The swizzle is applied to the group base and the target
+// them through it, so a warp's lanes reach different banks whatever the targets.  The swizzle is applied to the group base and the target
 // bits, which then combine by XOR.
-template <bool XP, int SUB = 1, bool SW = false>
-__global__ void __launch_bounds__(576, 1) apply_tc64(const __grid_constant__ Tc64Args a) {
+template <int SUB = 1, bool SW = false>
+__global__ void __launch_bounds__(608, 1) apply_tc64(const __grid_constant__ Tc64Args a) {
     using S = Tc64S<SUB>;
-    constexpr uint32_t KD = S::KD, NS = S::NS, NOUT = S::NOUT;
+    constexpr uint32_t KD = S::KD, NS = S::NS;
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) unsigned long long full[NS], empty[NS];
     __shared__ __align__(8) unsigned long long a_full[2], a_empty[2], d_full[2], d_empty[2];
-    __shared__ __align__(8) unsigned long long scale_full[4];   // row exponents, tile j -> j & 3
+    __shared__ __align__(8) unsigned long long scale_full[4];   // row exponents, subtile js -> js & 3
+    __shared__ __align__(8) unsigned long long out_full[2], out_free[2];   // staged subtiles
     __shared__ int row_exp[4][128];
-    __shared__ uint32_t emax_part[2][128];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
     unsigned char *sB = smem;
@@ -212,15 +221,17 @@ __global__ void __launch_bounds__(576, 1) apply_tc64(const __grid_constant__ Tc6
     if (tid == 0) {
         for (uint32_t s = 0; s < NS; ++s) {
             mbar_init(smem_u32(&full[s]), 1);
-            mbar_init(smem_u32(&empty[s]), 1);
+            mbar_init(smem_u32(&empty[s]), 4 * SUB);     // one transform group per subtile
         }
         for (int b = 0; b < 2; ++b) {
-            mbar_init(smem_u32(&a_full[b]), 1);
+            mbar_init(smem_u32(&a_full[b]), 4);       // one transform group
             mbar_init(smem_u32(&a_empty[b]), 1);
             mbar_init(smem_u32(&d_full[b]), 1);
-            mbar_init(smem_u32(&d_empty[b]), 1);
+            mbar_init(smem_u32(&d_empty[b]), 8);      // the epilogue warps
+            mbar_init(smem_u32(&out_full[b]), 8);
+            mbar_init(smem_u32(&out_free[b]), 1);
         }
-        for (int q = 0; q < 4; ++q) mbar_init(smem_u32(&scale_full[q]), 1);
+        for (int q = 0; q < 4; ++q) mbar_init(smem_u32(&scale_full[q]), 4);
         abort_flag = 0;
         fence_mbar_init();
     }
@@ -236,6 +247,8 @@ __global__ void __launch_bounds__(576, 1) apply_tc64(const __grid_constant__ Tc6
     const uint32_t tmem = tmem_slot;
     volatile int *abort = &abort_flag;
     const unsigned long long first = blockIdx.x, step = gridDim.x;
+    // this CTA's subtiles
+    const uint32_t nsub = a.ntiles > first ? (uint32_t)((a.ntiles - first + step - 1) / step) * SUB : 0u;
 
     auto group_base = [&](uint32_t row) {
         uint32_t g = row;
@@ -287,188 +300,179 @@ __global__ void __launch_bounds__(576, 1) apply_tc64(const __grid_constant__ Tc6
     } else if (warp == S::W_MMA) {
         // ------------------------------------------------------------ MMA issuer
         if (lane == 0) {
-            const uint32_t idesc = idesc_f16(S::ROWS, KD);
             const uint32_t B0 = smem_u32(sB);
-            const unsigned long long nsub = a.ntiles > first
-                                                ? ((a.ntiles - first + step - 1) / step) * SUB : 0;
-            for (unsigned long long js = 0; js < nsub; ++js) {
-                const uint32_t b = (uint32_t)js & 1u, u = (uint32_t)(js >> 1);
+            for (uint32_t js = 0; js < nsub; ++js) {
+                const uint32_t b = js & 1u, u = js >> 1;
                 if (!mbar_wait_or_abort(smem_u32(&a_full[b]), u & 1u, abort)) break;
                 if (!mbar_wait_or_abort(smem_u32(&d_empty[b]), (u & 1u) ^ 1u, abort)) break;
                 tc_fence_after();
                 const uint32_t A0 = tmem + S::A_COL0 + b * S::A_SET;
                 const uint32_t dset = tmem + b * S::ACC;
-                // (accumulator, A digit, B slice); slices 6 + j hold B_j 2^-9
-                const uint32_t prod[21][3] = {
-                    {0, 0, 0},
-                    {1, 0, 1}, {1, 1, 0},
-                    {2, 0, 2}, {2, 1, 1}, {2, 2, 0},
-                    {3, 0, 3}, {3, 1, 2}, {3, 2, 1}, {3, 3, 0},
-                    {4, 0, 4}, {4, 1, 3}, {4, 2, 2}, {4, 3, 1}, {4, 4, 0},
-                    {4, 0, 11}, {4, 1, 10}, {4, 2, 9}, {4, 3, 8}, {4, 4, 7}, {4, 5, 6}};
+                // A_i [B_0 .. B_{4-i}] -> [D_i .. D_4]: N rows from the first slice of B on
 #pragma unroll
-                for (int p = 0; p < 21; ++p) {
-                    const uint32_t acc = prod[p][0];
-                    const uint32_t Aa = A0 + prod[p][1] * S::A_COLS;
-                    const uint32_t Bb = B0 + prod[p][2] * S::B_BYTES;
-                    const bool first_in_acc = (p == 0 || p == 1 || p == 3 || p == 6 || p == 10);
+                for (uint32_t i = 0; i < 5; ++i)
 #pragma unroll
                     for (uint32_t ks = 0; ks < KD / 16; ++ks)
-                        mma_f16_tmem_a(dset + acc * KD, Aa + ks * 8u,
-                                       smem_desc(Bb + ks * 256u, 128u, S::SBO), idesc,
-                                       (first_in_acc && ks == 0) ? 0u : 1u);
-                }
+                        mma_f16_tmem_a(dset + i * KD, A0 + i * S::A_COLS + ks * 8u,
+                                       smem_desc(B0 + ks * 256u, 128u, S::SBO), idesc_f16(S::ROWS, (5u - i) * KD),
+                                       (i == 0 && ks == 0) ? 0u : 1u);
+                // level 5 at its scale, after the exact sums of level 4: A_i (B_{5-i} 2^-9) -> D_4
+#pragma unroll
+                for (uint32_t i = 0; i < 6; ++i)
+#pragma unroll
+                    for (uint32_t ks = 0; ks < KD / 16; ++ks)
+                        mma_f16_tmem_a(dset + 4u * KD, A0 + i * S::A_COLS + ks * 8u,
+                                       smem_desc(B0 + (11u - i) * S::B_BYTES + ks * 256u, 128u, S::SBO),
+                                       idesc_f16(S::ROWS, KD), 1u);
                 mma_commit(smem_u32(&a_empty[b]));
                 mma_commit(smem_u32(&d_full[b]));
             }
         }
     } else if (warp < S::W_PROD) {
         // ------------------------------------------------------------ digit transform
-        // Two warps per TMEM lane quadrant: warp w takes rows 32 (w & 3) .. + 31 and
-        // group members 8 (w >> 2) .. + 7.  Rolled loops over four members at a time keep
-        // the code small (the roles run different code on every SM sub-partition).
-        const uint32_t row = (warp & 3u) * 32u + lane;
-        const uint32_t part = warp >> 2;
+        // Two groups of four warps take alternate subtiles, one warp per TMEM lane quadrant and
+        // whole rows each, so that no warp waits for another.  Rolled loops over four members at
+        // a time keep the code small (the roles run different code on every SM sub-partition).
+        const uint32_t quad = warp & 3u, grp = warp >> 2;
+        const uint32_t row = quad * 32u + lane;
         const uint32_t lo_off[4] = {0u, tb[0], tb[1], tb[0] ^ tb[1]};
-        const uint32_t xl = (lane >> a.xs) & ((1u << a.xt) - 1u);
-        const uint32_t cx = ((xl & 1u) << a.lp[0]) | (((xl >> 1) & 1u) << a.lp[1]);
-        uint32_t j = 0;
-        bool stop = false;
-        for (unsigned long long t = first; t < a.ntiles && !stop; t += step, ++j) {
-            const uint32_t s = j % NS;
+        const uint32_t arow = tmem + S::A_COL0 + grp * S::A_SET + ((quad * 32u) << 16);
+        for (uint32_t js = grp; js < nsub; js += 2) {
+            const uint32_t j = js / SUB, sub = js % SUB, s = j % NS;
             const bool okf = mbar_wait_or_abort(smem_u32(&full[s]), (j / NS) & 1u, abort);
+            if (!__all_sync(0xffffffffu, okf)) break;
             const double2 *rs = reinterpret_cast<const double2 *>(smem + S::OFF_RAW + s * S::TILE_BYTES);
-#pragma unroll 1
-          for (uint32_t sub = 0; sub < (uint32_t)SUB; ++sub) {
-            const uint32_t js = j * SUB + sub;
             const uint32_t gbase = group_base(sub * S::ROWS + row);
-            const uint32_t ab = js & 1u;
-            const bool ok = okf && mbar_wait_or_abort(smem_u32(&a_empty[ab]), ((js >> 1) & 1u) ^ 1u, abort);
-            // the row's largest exponent field: each half over its members (high words)
-            uint32_t em = 0;                      // largest |high word|: its exponent field
-#pragma unroll
-            for (uint32_t c = 0; c < 8; ++c) {
-                const uint32_t *w = reinterpret_cast<const uint32_t *>(
-                    rs + (gbase ^ (XP ? (member_off(part * 8u + c) ^ cx) : member_off(part * 8u + c))));
-                em = max(em, max(w[1] & 0x7FFFFFFFu, w[3] & 0x7FFFFFFFu));
-            }
-            emax_part[part][row] = max(em >> 20, 1u);
-            if (!named_bar_and(1, 256, ok)) { stop = true; break; }
-            tc_fence_after();
-            const uint32_t emax = max(emax_part[0][row], emax_part[1][row]);
-            // slot js & 3 was last read by the epilogue of subtile js - 4, which finished
-            // before the MMAs of subtile js - 2 were issued, whose completion released
-            // a_empty[ab]
-            if (part == 0) row_exp[js & 3u][row] = (int)emax;
-            const uint32_t arow = tmem + S::A_COL0 + ab * S::A_SET + (((warp & 3u) * 32u) << 16);
+            uint32_t em = 0, mn = 0x7FFFFFFFu;    // largest and smallest |high word| of the row
 #pragma unroll 1
-            for (uint32_t c0 = part * 8u; c0 < part * 8u + 8u; c0 += 4) {
+            for (uint32_t c0 = 0; c0 < 16u; c0 += 4) {
+                const uint32_t hoff = gbase ^ (((c0 >> 2) & 1u) ? tb[2] : 0u) ^ (((c0 >> 3) & 1u) ? tb[3] : 0u);
+#pragma unroll
+                for (uint32_t c = 0; c < 4; ++c) {
+                    const uint4 v = *reinterpret_cast<const uint4 *>(rs + (hoff ^ lo_off[c]));
+                    const uint32_t r = v.y & 0x7FFFFFFFu, i = v.w & 0x7FFFFFFFu;
+                    em = max(em, max(r, i));
+                    mn = min(mn, min(r, i));
+                }
+            }
+            const uint32_t emax = max(em >> 20, 1u);
+            const uint32_t emin = mn >> 20;
+            const bool near = __all_sync(0xffffffffu, emin != 0u && emax - emin < 32u);
+            bool oka = true;
+#pragma unroll 1
+            for (uint32_t c0 = 0; c0 < 16u; c0 += 4) {
                 const uint32_t hoff = gbase ^ (((c0 >> 2) & 1u) ? tb[2] : 0u) ^ (((c0 >> 3) & 1u) ? tb[3] : 0u);
                 uint32_t w[6][4];
                 uint4 va[4];
 #pragma unroll
-                for (uint32_t c = 0; c < 4; ++c)
-                    va[c] = *reinterpret_cast<const uint4 *>(rs + (hoff ^ (XP ? (lo_off[c] ^ cx) : lo_off[c])));
-                if constexpr (XP) xor_unpermute4(va, xl, a.xt, sel_u4);
-#pragma unroll
-                for (uint32_t c = 0; c < 4; ++c) {
-                    const uint4 v = va[c];
-                    uint32_t rh, rl, ih, il, t[6];
-                    fxp::offset_fixed(v.y, v.x, emax, rh, rl);
-                    fxp::offset_fixed(v.w, v.z, emax, ih, il);
-                    fxp::digit_pair_words(rh, rl, ih, il, t);
-#pragma unroll
-                    for (int i = 0; i < 6; ++i) w[i][c] = digit_pair(t[i]);
+                for (uint32_t c = 0; c < 4; ++c) va[c] = *reinterpret_cast<const uint4 *>(rs + (hoff ^ lo_off[c]));
+                if (near) cut_members<true>(va, emax, w);
+                else cut_members<false>(va, emax, w);
+                if (c0 == 0) {
+                    // the A buffer is free once the MMAs of subtile js - 2 have completed
+                    oka = __all_sync(0xffffffffu,
+                                     mbar_wait_or_abort(smem_u32(&a_empty[grp]), ((js >> 1) & 1u) ^ 1u, abort));
+                    if (!oka) break;
+                    tc_fence_after();
+                    // slot js & 3 was last read by the epilogue of subtile js - 4, which finished
+                    // before the MMAs of subtile js - 2
+                    row_exp[js & 3u][row] = (int)emax;
                 }
 #pragma unroll
                 for (int i = 0; i < 6; ++i) tmem_st4_async(arow + i * S::A_COLS + c0, w[i]);
             }
+            if (!oka) break;
             fence_proxy_async_smem();             // reads of the raw stage before its refill
             tmem_wait_st();
             tc_fence_before();
-            named_bar(1, 256);                    // also: emax_part is free for the next subtile
-            if (tid == 0) {
-                if (sub == (uint32_t)SUB - 1u) mbar_arrive(smem_u32(&empty[s]));
-                mbar_arrive(smem_u32(&a_full[ab]));
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(smem_u32(&empty[s]));
+                mbar_arrive(smem_u32(&a_full[grp]));
                 mbar_arrive(smem_u32(&scale_full[js & 3u]));
             }
-          }
         }
-    } else if (warp >= S::W_EPI) {
+    } else if (warp < S::W_STORE) {
         // ------------------------------------------------------------ epilogue
         // Two warps per lane quadrant, each over 16 of the 32 accumulator columns.
         const uint32_t quad = warp & 3u;
         const uint32_t row = quad * 32u + lane;
-        const uint32_t et = tid - S::W_EPI * 32u;    // 0..255
-        const uint32_t part = et >> 7;
-        const uint32_t lo_off[4] = {0u, tb[0], tb[1], tb[0] ^ tb[1]};
-        const uint32_t xl = (lane >> a.xs) & ((1u << a.xt) - 1u);
-        const uint32_t cx = ((xl & 1u) << a.lp[0]) | (((xl >> 1) & 1u) << a.lp[1]);
-        SegLanes sl;
-        sl.init(a.L, a.h, a.hi, lane);
-        uint32_t j = 0;
-        bool stop = false;
-        for (unsigned long long t = first; t < a.ntiles && !stop; t += step, ++j) {
-            const uint32_t ob = j % NOUT;
-            double2 *out = reinterpret_cast<double2 *>(smem + S::OFF_OUT + ob * S::TILE_BYTES);
-#pragma unroll 1
-          for (uint32_t sub = 0; sub < (uint32_t)SUB; ++sub) {
-            const uint32_t js = j * SUB + sub, b = js & 1u;
-            const uint32_t gbase = group_base(sub * S::ROWS + row);
+        const uint32_t part = (warp - S::W_EPI) >> 2;
+        for (uint32_t js = 0; js < nsub; ++js) {
+            const uint32_t b = js & 1u;
+            double2 *out = reinterpret_cast<double2 *>(smem + S::OFF_OUT + (SUB == 1 ? b * S::TILE_BYTES : 0u));
+            const uint32_t gbase = group_base(js % SUB * S::ROWS + row);
             bool ok = mbar_wait_or_abort(smem_u32(&d_full[b]), (js >> 1) & 1u, abort);
             ok = ok && mbar_wait_or_abort(smem_u32(&scale_full[js & 3u]), (js >> 2) & 1u, abort);
-            if (!named_bar_and(2, 256, ok)) { stop = true; break; }
+            ok = ok && mbar_wait_or_abort(smem_u32(&out_free[b]), ((js >> 1) & 1u) ^ 1u, abort);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
             tc_fence_after();
-            if (sub == 0) {
-                if (et < 32) bulk_wait_read<(int)NOUT - 1>();   // this staging tile is free
-                named_bar(2, 256);
-            }
             const int p = row_exp[js & 3u][row] + a.b_exp - 1078;   // out = Z 2^p
             const uint32_t lane_addr = tmem + b * S::ACC + ((quad * 32u) << 16);
-            // eight columns (four members) of the five accumulators per step; the two steps
-            // are unrolled so that their recombinations overlap (28 qubits: 3.40 -> 3.47
-            // TB/s; unrolling the transform's member loop too measured slower)
-#pragma unroll
-            for (uint32_t c0 = part * 16u; c0 < part * 16u + 16u; c0 += 8) {
+            const bool p_safe = __all_sync(0xffffffffu, p >= -1022 && p <= 960);
+            // eight columns (four members) of the five accumulators per step, both steps
+            // unrolled so that their recombinations overlap
+            auto finish = [&](auto safe, uint32_t c0) {
                 float d[5][8];
-                tmem_ld8x5(lane_addr + c0, KD, d);
-                const uint32_t m0 = c0 >> 1;
-                const uint32_t hoff = gbase ^ (((m0 >> 2) & 1u) ? tb[2] : 0u) ^ (((m0 >> 3) & 1u) ? tb[3] : 0u);
-                double2 o[4];
+                tmem_ld8x5(lane_addr + part * 16u + c0, KD, d);
+                const uint32_t hoff = gbase ^ (c0 ? tb[2] : 0u) ^ (part ? tb[3] : 0u);
 #pragma unroll
                 for (uint32_t c = 0; c < 4; ++c) {
-                    const double re = combine_levels(d[0][2 * c], d[1][2 * c], d[2][2 * c],
-                                                     d[3][2 * c], d[4][2 * c], p);
-                    const double im = combine_levels(d[0][2 * c + 1], d[1][2 * c + 1], d[2][2 * c + 1],
-                                                     d[3][2 * c + 1], d[4][2 * c + 1], p);
-                    o[c] = make_double2(re, im);
+                    const double re = combine_levels<decltype(safe)::value>(
+                        d[0][2 * c], d[1][2 * c], d[2][2 * c], d[3][2 * c], d[4][2 * c], p);
+                    const double im = combine_levels<decltype(safe)::value>(
+                        d[0][2 * c + 1], d[1][2 * c + 1], d[2][2 * c + 1], d[3][2 * c + 1], d[4][2 * c + 1], p);
+                    out[hoff ^ member_off(c)] = make_double2(re, im);
                 }
-                if constexpr (XP) xor_unpermute4(o, xl, a.xt, sel_d2);   // o[c] = member c ^ x
-#pragma unroll
-                for (uint32_t c = 0; c < 4; ++c) out[hoff ^ (XP ? (lo_off[c] ^ cx) : lo_off[c])] = o[c];
+            };
+            if (p_safe) {
+                finish(std::true_type{}, 0u);
+                finish(std::true_type{}, 8u);
+            } else {
+#pragma unroll 1
+                for (uint32_t c0 = 0; c0 < 16u; c0 += 8) finish(std::false_type{}, c0);
             }
             tc_fence_before();
-            fence_proxy_async_smem();
-            named_bar(2, 256);
-            if (et == 0) mbar_arrive(smem_u32(&d_empty[b]));
-          }
-            if (stop) break;
-            if (et < 32) {
-                if (lane < nseg) {
-                    if constexpr (SW) {
-                        const int32_t row0 = (int32_t)((sl.base(t) + sl.my_off) >> 3);
-                        const uint32_t s0 = smem_u32(out + (size_t)lane * seg_amps);
-                        for (uint32_t bx = 0; bx < a.boxes; ++bx)
-                            tma_store_2d(&a.tmap, 0, row0 + (int32_t)(bx * a.box_rows), s0 + bx * a.box_rows * 128u);
-                    } else {
-                        bulk_s2g(psi + sl.base(t) + sl.my_off, smem_u32(out + (size_t)lane * seg_amps),
-                                 seg_bytes);
-                    }
-                }
-                bulk_commit();
+            fence_proxy_async_smem();                 // the bulk store reads what this thread wrote
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(smem_u32(&d_empty[b]));
+                mbar_arrive(smem_u32(&out_full[b]));
             }
         }
-        if (et < 32) bulk_wait_all();
+    } else {
+        // ------------------------------------------------------------ TMA stores
+        // One subtile at a time.  With SUB = 2 the two of a tile are the halves of its staging
+        // that differ in bit sb, the highest tile bit that is no target: pieces of 2^sb amplitudes,
+        // one per segment unless targets sit right below L.
+        SegLanes sl;
+        sl.init(a.L, a.h, a.hi, lane);
+        for (uint32_t js = 0; js < nsub; ++js) {
+            const uint32_t ob = js & 1u;
+            const unsigned long long t = first + (unsigned long long)(js / SUB) * step;
+            const double2 *out = reinterpret_cast<const double2 *>(smem + S::OFF_OUT + (SUB == 1 ? ob * S::TILE_BYTES : 0u));
+            const bool ok = mbar_wait_or_abort(smem_u32(&out_full[ob]), (js >> 1) & 1u, abort);
+            if (!__all_sync(0xffffffffu, ok)) break;
+            if (lane < nseg) {
+                if constexpr (SW) {
+                    const int32_t row0 = (int32_t)((sl.base(t) + sl.my_off) >> 3);
+                    const uint32_t s0 = smem_u32(out + (size_t)lane * seg_amps);
+                    for (uint32_t bx = 0; bx < a.boxes; ++bx)
+                        tma_store_2d(&a.tmap, 0, row0 + (int32_t)(bx * a.box_rows), s0 + bx * a.box_rows * 128u);
+                } else if constexpr (SUB == 2) {
+                    for (uint32_t o = ob << a.sb; o < seg_amps; o += 2u << a.sb)
+                        bulk_s2g(psi + sl.base(t) + sl.my_off + o, smem_u32(out + (size_t)lane * seg_amps + o), 16u << a.sb);
+                } else {
+                    bulk_s2g(psi + sl.base(t) + sl.my_off, smem_u32(out + (size_t)lane * seg_amps), seg_bytes);
+                }
+            }
+            bulk_commit();
+            bulk_wait_read_all();                 // the staging is free again
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&out_free[ob]));
+        }
+        bulk_wait_all();
     }
     if (tid == 0 && abort_flag) atomicOr(a.err, 2);
     tc_fence_before();
@@ -483,13 +487,13 @@ sv_status launch_tc64(sv_state *s, const svi::Gate &g0) {
     static std::once_flag once;
     static cudaError_t init_err = cudaSuccess;
     std::call_once(once, [] {
-        init_err = cudaFuncSetAttribute(apply_tc64<false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        init_err = cudaFuncSetAttribute(apply_tc64<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)S::SMEM);
         if (init_err == cudaSuccess)
-            init_err = cudaFuncSetAttribute(apply_tc64<false, 2>,
+            init_err = cudaFuncSetAttribute(apply_tc64<2>,
                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S2::SMEM);
         if (init_err == cudaSuccess)
-            init_err = cudaFuncSetAttribute(apply_tc64<false, 1, true>,
+            init_err = cudaFuncSetAttribute(apply_tc64<1, true>,
                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
     });
     if (init_err != cudaSuccess)
@@ -515,12 +519,7 @@ sv_status launch_tc64(sv_state *s, const svi::Gate &g0) {
     // stage); the others keep 1-D bulk copies, where the swizzled staging measured slower.
     const bool swz = std::min(tl, 2u) >= 2u;
     const bool wide = !swz && s->n >= S2::TB && p.h >= 3;
-    if (wide) {
-        p = make_plan(s->n, 4, g->t, S2::TB);
-        tl = 0;
-        while (tl < 3u && p.lp[tl] < 3u) ++tl;
-    }
-    if (swz) tl = 0;
+    if (wide) p = make_plan(s->n, 4, g->t, S2::TB);
     Tc64Args a;
     a.box_rows = a.boxes = 0;
     if (swz) {
@@ -545,14 +544,14 @@ sv_status launch_tc64(sv_state *s, const svi::Gate &g0) {
     a.h = p.h;
     for (int j = 0; j < SV_MAX_K; ++j) a.hi[j] = p.hi[j];
     for (int j = 0; j < 4; ++j) a.lp[j] = p.lp[j];
-    a.xs = 3u - tl;
-    a.xt = std::min(tl, 2u);
+    a.sb = p.L - 1;
+    for (int j = 3 - (int)p.h; j >= 0 && p.lp[j] == a.sb; --j) --a.sb;
     const unsigned grid = (unsigned)std::min<unsigned long long>(p.ntiles, (unsigned long long)s->num_sms);
     // two targets in bits 0..2 (4-way conflicts and worse) take the swizzled staging; one
     // target there leaves 2-way conflicts, cheaper than either remedy
-    SV_CUDA(swz    ? launch_pass(apply_tc64<false, 1, true>, dim3(grid), S::THREADS, S::SMEM, s->stream, a)
-            : wide ? launch_pass(apply_tc64<false, 2>, dim3(grid), S2::THREADS, S2::SMEM, s->stream, a)
-                   : launch_pass(apply_tc64<false, 1>, dim3(grid), S::THREADS, S::SMEM, s->stream, a));
+    SV_CUDA(swz    ? launch_pass(apply_tc64<1, true>, dim3(grid), S::THREADS, S::SMEM, s->stream, a)
+            : wide ? launch_pass(apply_tc64<2>, dim3(grid), S2::THREADS, S2::SMEM, s->stream, a)
+                   : launch_pass(apply_tc64<1>, dim3(grid), S::THREADS, S::SMEM, s->stream, a));
     return SV_OK;
 }
 

@@ -142,6 +142,20 @@ FXP_HD void offset_fixed(uint32_t hi, uint32_t lo, uint32_t emax, uint32_t &yh, 
     yh = (uint32_t)(y >> 32);
 }
 
+// offset_fixed for a nonzero exponent field at most 31 below emax (emax_word = emax << 20 |
+// 0xFFFFF): the implicit bit is there, the shift is below 32 and the sign can follow it
+// (bits 20..24 of emax_word - hi are the shift, whatever the sign bit adds above them).
+FXP_HD void offset_fixed_near(uint32_t hi, uint32_t lo, uint32_t emax_word, uint32_t &yh, uint32_t &yl) {
+    const uint32_t sh = ((emax_word - hi) >> 20) & 31u;
+    const uint32_t mh = (hi & 0xFFFFFu) | 0x100000u;
+    const uint32_t ah = funnel_l(lo, mh, 1), al = lo << 1;
+    const uint32_t sg = (uint32_t)((int32_t)hi >> 31);
+    const uint32_t xl = funnel_r(al, ah, sh) ^ sg, xh = funnel_r(ah, 0u, sh) ^ sg;
+    const uint64_t y = ((((uint64_t)xh) << 32) | xl) + (2ull * OFFSET + 1ull);
+    yl = (uint32_t)y;
+    yh = (uint32_t)(y >> 32);
+}
+
 // The six digit-pair words (most significant first) of the amplitude (re, im) from the
 // Y' words of both parts: fields of Y' at bits 46 (ten bits), 37, 28, 19, 10 and 1.  A
 // byte permute puts the two parts' 16-bit windows side by side, one shift and one
