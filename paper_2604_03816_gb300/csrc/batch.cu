@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <atomic>
 #include <chrono>
+#include <cmath>
 #include <cstring>
 #include <map>
 #include <mutex>
@@ -224,7 +225,11 @@ struct BatchExpectArgs {
     uint32_t n;
 };
 
-// Terms that share an X-part x != 0 (Z strings: expect.cu).  grid (BEXP_BLOCKS, states):
+__device__ __forceinline__ float bprob(float x, float y) { return __fadd_rn(__fmul_rn(x, x), __fmul_rn(y, y)); }
+__device__ __forceinline__ double bprob(double x, double y) { return __dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y)); }
+
+// Terms that share an X-part x (x = 0, Z strings, only where expect.cu's FP32 sums overflowed:
+// npairs counts amplitudes).  grid (BEXP_BLOCKS, states):
 // partial[state * BEXP_BLOCKS + block]
 template <typename R>
 __global__ void batch_expect_kernel(const __grid_constant__ BatchExpectArgs a, const void *psi_,
@@ -234,6 +239,13 @@ __global__ void batch_expect_kernel(const __grid_constant__ BatchExpectArgs a, c
     double acc = 0.0;
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
     for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < a.npairs; i += stride) {
+        if (a.x == 0) {
+            const C v = psi[i];
+            double w = 0.0;
+            for (int t = 0; t < a.nterms; ++t) w += (__popcll(i & a.z[t]) & 1) ? -a.ccr[t] : a.ccr[t];
+            acc += w * (double)bprob(v.x, v.y);
+            continue;
+        }
         const unsigned long long k = insert_zero64(i, (uint32_t)a.hb), k2 = k ^ a.x;
         const C p = psi[k], q = psi[k2];
         const double re = (double)q.x * p.x + (double)q.y * p.y;
@@ -730,15 +742,8 @@ sv_status sv_batch_apply(sv_batch *b, const sv_circuit *const *circuits, const s
     return SV_OK;
 }
 
-sv_status sv_batch_expect(sv_batch *b, const uint64_t *xmask, const uint64_t *zmask, const double *coef,
-                          size_t nterms, double *out) {
-    clear_error();
-    if (!b || !out || (nterms && (!xmask || !zmask || !coef)))
-        return set_error(SV_ERR_ARG, "sv_batch_expect: null argument");
-    const uint64_t lim = (1ull << b->n) - 1;
-    for (size_t t = 0; t < nterms; ++t)
-        if ((xmask[t] & ~lim) || (zmask[t] & ~lim))
-            return set_error(SV_ERR_ARG, "sv_batch_expect: Pauli mask names a qubit >= n");
+static sv_status batch_expect_terms(sv_batch *b, const uint64_t *xmask, const uint64_t *zmask, const double *coef,
+                                    size_t nterms, bool general, double *out) {
     SV_CUDA(cudaMemsetAsync(b->results, 0, sizeof(double) * b->count, b->stream));
     std::vector<size_t> order(nterms);
     for (size_t i = 0; i < nterms; ++i) order[i] = i;
@@ -750,7 +755,7 @@ sv_status sv_batch_expect(sv_batch *b, const uint64_t *xmask, const uint64_t *zm
         return SV_OK;
     };
     size_t i = 0;
-    if (nterms && xmask[order[0]] == 0) {              // the Z strings, all of them together
+    if (nterms && xmask[order[0]] == 0 && !general) {  // the Z strings, all of them together
         std::vector<uint64_t> z;
         std::vector<double> c;
         for (; i < nterms && xmask[order[i]] == 0; ++i) {
@@ -775,8 +780,8 @@ sv_status sv_batch_expect(sv_batch *b, const uint64_t *xmask, const uint64_t *zm
             a.cci[a.nterms] = coef[t] * im[y];
             ++a.nterms;
         }
-        a.hb = 63 - __builtin_clzll(a.x);
-        a.npairs = 1ull << (b->n - 1);
+        a.hb = a.x ? 63 - __builtin_clzll(a.x) : 0;
+        a.npairs = 1ull << (a.x ? b->n - 1 : b->n);
         a.n = b->n;
         const dim3 grid(svk::BEXP_BLOCKS, b->count);
         if (b->dtype == SV_C64)
@@ -796,6 +801,22 @@ sv_status sv_batch_expect(sv_batch *b, const uint64_t *xmask, const uint64_t *zm
         return set_error(SV_ERR_TIMEOUT, "a bounded device-side wait gave up in a batched pass");
     }
     return SV_OK;
+}
+
+sv_status sv_batch_expect(sv_batch *b, const uint64_t *xmask, const uint64_t *zmask, const double *coef,
+                          size_t nterms, double *out) {
+    clear_error();
+    if (!b || !out || (nterms && (!xmask || !zmask || !coef)))
+        return set_error(SV_ERR_ARG, "sv_batch_expect: null argument");
+    const uint64_t lim = (1ull << b->n) - 1;
+    for (size_t t = 0; t < nterms; ++t)
+        if ((xmask[t] & ~lim) || (zmask[t] & ~lim))
+            return set_error(SV_ERR_ARG, "sv_batch_expect: Pauli mask names a qubit >= n");
+    // FP32 sums that overflowed (launch_expect): once more with FP64 sums
+    const sv_status st = batch_expect_terms(b, xmask, zmask, coef, nterms, false, out);
+    if (st != SV_OK || b->dtype != SV_C64 || std::all_of(out, out + b->count, [](double v) { return std::isfinite(v); }))
+        return st;
+    return batch_expect_terms(b, xmask, zmask, coef, nterms, true, out);
 }
 
 sv_status sv_batch_tune(sv_batch *b, const sv_gate *gates, size_t ngates, uint32_t kmin, uint32_t kmax,

@@ -31,6 +31,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <functional>
 #include <mutex>
@@ -718,8 +719,9 @@ sv_status batch_z_terms(const void *psi, uint32_t n, sv_dtype dtype, uint32_t st
                : z_passes<double>(psi, n, states, num_sms, stream, tables, t.data(), nterms, reserve, fold);
 }
 
-sv_status launch_expect(sv_state *s, const uint64_t *x, const uint64_t *z, const double *c,
-                        size_t nterms, double *host_out) {
+// general: every term by the general kernel.
+static sv_status expect_terms(sv_state *s, const uint64_t *x, const uint64_t *z, const double *c, size_t nterms,
+                              bool general, double *host_out) {
     std::vector<Term> t(nterms);
     for (size_t i = 0; i < nterms; ++i) t[i] = Term{x[i], z[i], c[i]};
     std::stable_sort(t.begin(), t.end(), [](const Term &a, const Term &b) { return a.x < b.x; });
@@ -729,9 +731,9 @@ sv_status launch_expect(sv_state *s, const uint64_t *x, const uint64_t *z, const
         size_t e = i;
         while (e < nterms && t[e].x == t[i].x) ++e;
         sv_status st = SV_OK;
-        if (t[i].x == 0) {
+        if (t[i].x == 0 && !general) {
             st = s->dtype == SV_C64 ? z_group<float>(s, P, &t[i], e - i) : z_group<double>(s, P, &t[i], e - i);
-        } else if (s->n >= 4 && __builtin_popcountll(t[i].x) <= 4 && (s->dtype == SV_C128 || e - i <= 4)) {
+        } else if (!general && s->n >= 4 && __builtin_popcountll(t[i].x) <= 4 && (s->dtype == SV_C128 || e - i <= 4)) {
             xt.insert(xt.end(), t.begin() + i, t.begin() + e);
         } else {
             // general kernel, up to 32 terms per launch
@@ -760,6 +762,15 @@ sv_status launch_expect(sv_state *s, const uint64_t *x, const uint64_t *z, const
     if (st == SV_OK) st = P.collect();
     *host_out = P.total;
     return st;
+}
+
+// Two-float sums end at 3.4e38 where the general kernel's FP64 sums go on (amplitudes around 1e18):
+// a complex64 result that is not finite is formed again there.
+sv_status launch_expect(sv_state *s, const uint64_t *x, const uint64_t *z, const double *c,
+                        size_t nterms, double *host_out) {
+    const sv_status st = expect_terms(s, x, z, c, nterms, false, host_out);
+    if (st != SV_OK || s->dtype != SV_C64 || std::isfinite(*host_out)) return st;
+    return expect_terms(s, x, z, c, nterms, true, host_out);
 }
 
 }  // namespace svi
