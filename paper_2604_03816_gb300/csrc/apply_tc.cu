@@ -45,7 +45,7 @@
 //   warp 18              issues the staging tiles' TMA bulk stores.
 // The epilogue warps never meet: they hand accumulators and staging tiles on by counted mbarrier
 // arrivals (an epilogue barrier and stores by one of its warps cost a batched pass of 18 qubits x
-// 96 states 4%, 75 -> 71 us).  The transform warps meet three times per subtile; letting them meet
+// 96 states 4%, 75 -> 71 us).  The transform warps meet three times per tile; letting them meet
 // in pairs instead measured the same within 1% (faster on 24-qubit states, slower on 28).
 // Targets among tile bits 0..3 (where 8-byte accesses pick their bank) would make the
 // lanes of a warp hit one bank.  Width-5 launches on states of 13 qubits or more, and
@@ -73,22 +73,20 @@
 
 namespace svk {
 
-// SUB: MMA subtiles (128 groups each) per TMA stage.  SUB = 2 doubles the contiguous
-// segments of launches whose targets are all high (2 KiB instead of 1 KiB at k = 5).
-// BT: a batched launch over many states with their own matrices (see apply_tc): two B
+// One tile is one MMA (128 groups).  BT: a batched launch over many states with their own matrices (see apply_tc): two B
 // sets (the current state's and the next one's).
-template <int K, int SUB = 1, bool BT = false>
+template <int K, bool BT = false>
 struct TcShape {
     static constexpr uint32_t D = 1u << K;            // amplitudes per group
     static constexpr uint32_t KD = 2u * D;            // real K = N
-    static constexpr uint32_t ROWS = 128;             // groups per MMA subtile (MMA M)
-    static constexpr uint32_t TB = K + 7 + (SUB == 2 ? 1u : 0u);   // tile bits
-    static constexpr uint32_t TILE_BYTES = SUB * ROWS * D * 8u;
+    static constexpr uint32_t ROWS = 128;             // groups per tile (MMA M)
+    static constexpr uint32_t TB = K + 7;             // tile bits
+    static constexpr uint32_t TILE_BYTES = ROWS * D * 8u;
     static constexpr uint32_t B_BYTES = KD * KD * 2u;     // one FP16 slice of B
     static constexpr uint32_t NB = 3;                     // B1, B2 2^-9, B3 2^-18
     static constexpr uint32_t SBO = (KD / 8u) * 128u;     // 8-row group stride of B
-    static constexpr uint32_t NS = SUB == 2 ? 2u : BT ? 3u : (K == 5 ? 4u : 8u);   // raw stages
-    static constexpr uint32_t NOUT = SUB == 2 ? 1u : 2u;  // output staging tiles
+    static constexpr uint32_t NS = BT ? 3u : (K == 5 ? 4u : 8u);   // raw stages
+    static constexpr uint32_t NOUT = 2u;              // output staging tiles
     static constexpr uint32_t ACC = 2u * KD;              // TMEM columns of one D set (D0, D12)
     static constexpr uint32_t A_COLS = KD / 2u;           // TMEM columns of one A slice
     static constexpr uint32_t NA = 3;                     // A1, A2 2^-9, A3 2^-18
@@ -116,6 +114,7 @@ struct TcArgs {
     // |bx| <= 2^26.  The prologue cuts each into three 9-bit slices (cut_b).
     alignas(16) int2 bx[(1u << K) * (1u << K)];
     uint32_t box_rows, boxes;
+    uint32_t depth;                        // tile loads in flight, 1 .. NS
     float b_inv_scale;
     void *psi;
     int *err;
@@ -229,7 +228,7 @@ struct PackArgs {
 // 256 and the three 9-bit slices of the FP32 values are exact.  A thread writes 16-byte chunks of
 // the slices B1, B2 2^-9, B3 2^-18: eight columns of one row.
 __global__ void __launch_bounds__(256) pack_images(const __grid_constant__ PackArgs a) {
-    using S = TcShape<5, 1, true>;
+    using S = TcShape<5, true>;
     __shared__ float red[8];
     const uint32_t tid = threadIdx.x;
     const PackGate &g = a.g[blockIdx.y];
@@ -277,8 +276,7 @@ __global__ void __launch_bounds__(256) pack_images(const __grid_constant__ PackA
 
 // XP: the launch has targets among tile bits 0..3 and takes members in the lane's XOR
 // order; otherwise every lane takes them in member order (no permutation code at all).
-// The pipelines count tiles (j: raw stage, output staging) and MMA subtiles (js = j SUB +
-// sub: A and D buffers, row scales).
+// The pipelines count this CTA's tiles (j).
 // BT: one launch over a batch of states, each with its own matrix: a CTA takes a
 // contiguous range of tiles (so it meets few states), B is double-buffered and the producer
 // loads the next state's set a few tiles into the current one (b_full: arrived; b_empty: the
@@ -287,12 +285,17 @@ __global__ void __launch_bounds__(256) pack_images(const __grid_constant__ PackA
 // 128-byte swizzle (16-byte chunk index XOR the 128-byte row within each 1 KiB), and the
 // roles address the tile through the same swizzle.  A warp's lanes (consecutive groups)
 // then reach different banks whatever the targets, so no lane-dependent member order is
-// needed (XP = false) and every layout takes two subtiles per stage.  The swizzle is linear
+// needed (XP = false).  The swizzle is linear
 // over XOR, so it is applied to the group base and to the target bits once, and member
 // offsets combine them by XOR.
-template <int K, bool XP, int SUB, bool BT = false, bool SW = false>
+// P0 (with SW): the targets include index bits 0-3, so members c and c + 1 are neighbours, also
+// under the swizzle, and take 16-byte accesses: a group is then one or two whole 128-byte rows and the
+// swizzle spreads a warp's lanes over few chunks (8-way conflicts in 8-byte accesses).  Targets
+// 0-4: 28 qubits 848 -> 626 us per pass, 24 qubits 62.9 -> 46.1.  With only bit 0 or bits 0 and 1
+// among the targets 8-byte accesses are as fast.
+template <int K, bool XP, bool BT = false, bool SW = false, bool P0 = false>
 __global__ void __launch_bounds__(608, 1) apply_tc(const __grid_constant__ TcArgs<K> a) {
-    using S = TcShape<K, SUB, BT>;
+    using S = TcShape<K, BT>;
     constexpr uint32_t KD = S::KD, NS = S::NS, NOUT = S::NOUT, HALF = S::HALF;
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) unsigned long long full[NS], empty[NS];
@@ -428,7 +431,12 @@ __global__ void __launch_bounds__(608, 1) apply_tc(const __grid_constant__ TcArg
             }
             const uint32_t s = j % NS, u = j / NS;
             bool ok = true;
-            if (lane == 0) ok = mbar_wait_or_abort(smem_u32(&empty[s]), (u & 1u) ^ 1u, abort);
+            if (lane == 0) {
+                ok = mbar_wait_or_abort(smem_u32(&empty[s]), (u & 1u) ^ 1u, abort);
+                // at most `depth` tiles on their way (launch_tc_t)
+                const uint32_t i = j - a.depth;
+                if (ok && a.depth < NS && j >= a.depth) ok = mbar_wait_or_abort(smem_u32(&full[i % NS]), (i / NS) & 1u, abort);
+            }
             if (!__shfl_sync(0xffffffffu, (int)ok, 0)) break;
             const uint32_t bar = smem_u32(&full[s]);
             if (lane == 0) mbar_arrive_expect_tx(bar, S::TILE_BYTES);
@@ -452,12 +460,12 @@ __global__ void __launch_bounds__(608, 1) apply_tc(const __grid_constant__ TcArg
         if (lane == 0) {
             const uint32_t idesc = idesc_f16(S::ROWS, KD), idesc2 = idesc_f16(S::ROWS, 2u * KD);
             uint32_t B0 = smem_u32(sB);
-            const unsigned long long nsub = tend > first ? ((tend - first + step - 1) / step) * SUB : 0;
+            const unsigned long long ntile = tend > first ? (tend - first + step - 1) / step : 0;
             unsigned long long cur = ~0ull;
             uint32_t nsw = 0;
-            for (unsigned long long js = 0; js < nsub; ++js) {
+            for (unsigned long long j = 0; j < ntile; ++j) {
                 if constexpr (BT) {
-                    const unsigned long long st = (first + (js / SUB) * step) >> a.tps;
+                    const unsigned long long st = (first + j * step) >> a.tps;
                     if (st != cur) {
                         if (cur != ~0ull) {
                             mma_commit(smem_u32(&b_empty[nsw & 1u]));   // the old state's MMAs
@@ -470,7 +478,7 @@ __global__ void __launch_bounds__(608, 1) apply_tc(const __grid_constant__ TcArg
                         B0 = smem_u32(sB) + set * S::B_SET;
                     }
                 }
-                const uint32_t b = (uint32_t)js & 1u, u = (uint32_t)(js >> 1);
+                const uint32_t b = (uint32_t)j & 1u, u = (uint32_t)(j >> 1);
                 if (!mbar_wait_or_abort(smem_u32(&a_full[b]), u & 1u, abort)) break;
                 if (!mbar_wait_or_abort(smem_u32(&d_empty[b]), (u & 1u) ^ 1u, abort)) break;
                 tc_fence_after();
@@ -495,23 +503,20 @@ __global__ void __launch_bounds__(608, 1) apply_tc(const __grid_constant__ TcArg
         }
     } else if (warp < S::W_PROD) {
         // ------------------------------------------------------------ transform
-        // Two warps per TMEM lane quadrant: warp w takes rows 32 (w & 3) .. + 31 of each MMA
-        // subtile and group members HALF (w >> 2) .. + HALF - 1.
+        // Two warps per TMEM lane quadrant: warp w takes rows 32 (w & 3) .. + 31 of each
+        // tile and group members HALF (w >> 2) .. + HALF - 1.
         const uint32_t row = (warp & 3u) * 32u + lane;
         const uint32_t part = warp >> 2;
-        uint32_t gb[SUB];
-#pragma unroll
-        for (uint32_t sub = 0; sub < SUB; ++sub) gb[sub] = group_base(sub * S::ROWS + row);
+        const uint32_t gbase = group_base(row);
         const uint32_t xl = (lane >> a.xs) & ((1u << a.xt) - 1u);
         uint32_t cx = 0;
 #pragma unroll
         for (int q = 0; q < K; ++q)
             if ((xl >> q) & 1u) cx |= tbit[q];
         uint32_t j = 0;
-        bool stop = false;
         unsigned long long cur = ~0ull;
         float bsc = a.b_inv_scale;
-        for (unsigned long long t = first; t < tend && !stop; t += step, ++j) {
+        for (unsigned long long t = first; t < tend; t += step, ++j) {
             const uint32_t s = j % NS;
             const bool okf = mbar_wait_or_abort(smem_u32(&full[s]), (j / NS) & 1u, abort);
             if constexpr (BT) {
@@ -520,58 +525,60 @@ __global__ void __launch_bounds__(608, 1) apply_tc(const __grid_constant__ TcArg
                 cur = st;
             }
             const float2 *rs = reinterpret_cast<const float2 *>(smem + S::OFF_RAW + s * S::TILE_BYTES);
+            // this half of the row (members in the lane's order c ^ x), its largest component
+            float2 v[HALF];
+            float m = 0.f;
 #pragma unroll
-            for (uint32_t sub = 0; sub < SUB; ++sub) {
-                const uint32_t js = j * SUB + sub;
-                const uint32_t gbase = gb[sub];
-                // this half of the row (members in the lane's order c ^ x), its largest component
-                float2 v[HALF];
-                float m = 0.f;
-#pragma unroll
-                for (uint32_t c = 0; c < HALF; ++c) {
-                    const uint32_t mo = member_off(part * HALF + c);
+            for (uint32_t c = 0; c < HALF; c += P0 ? 2 : 1) {
+                const uint32_t mo = member_off(part * HALF + c);
+                if constexpr (P0) {
+                    const float4 f = *reinterpret_cast<const float4 *>(rs + (gbase ^ mo));
+                    v[c] = make_float2(f.x, f.y);
+                    v[c + 1] = make_float2(f.z, f.w);
+                    m = max_abs2(m, f.z, f.w);
+                } else {
                     v[c] = rs[gbase ^ (XP ? (mo ^ cx) : mo)];
-                    m = max_abs2(m, v[c].x, v[c].y);
                 }
-                max_part[part][row] = m;
-                fence_proxy_async_smem();         // reads of the raw stage before its refill
-                if (!named_bar_and(1, 256, okf)) { stop = true; break; }
-                if (sub == SUB - 1 && tid == 0) mbar_arrive(smem_u32(&empty[s]));
-                m = fmaxf(max_part[0][row], max_part[1][row]);
-                int ex = 0;
-                frexpf(m, &ex);                   // m < 2^ex (m = 0: ex = 0)
-                ex = max(ex, -100);               // keep 2^(8-ex) finite
-                const float sc = ldexpf(1.f, 8 - ex);      // |x * sc| < 256
-                const float2 scale = make_float2(sc, sc);
-                const uint32_t ab = js & 1u;
-                const bool oka = mbar_wait_or_abort(smem_u32(&a_empty[ab]), ((js >> 1) & 1u) ^ 1u, abort);
-                if (!named_bar_and(1, 256, oka)) { stop = true; break; }
-                tc_fence_after();
-                // slot js & 3 was last read by the epilogue of subtile js - 4, which finished
-                // before the MMAs of subtile js - 2 were issued, whose completion released
-                // a_empty[ab]
-                if (part == 0) row_scale[js & 3u][row] = ldexpf(bsc, ex - 8);
-                if constexpr (XP) xor_unpermute(v, xl, a.xt);   // back in member order (x < HALF)
-                // three 9-bit slices, one FP16 pair (re, im) per 32-bit TMEM column, stored
-                // eight members at a time
-                const uint32_t arow = tmem + S::A_COL0 + ab * S::A_SET + (((warp & 3u) * 32u) << 16) +
-                                      part * HALF;
+                m = max_abs2(m, v[c].x, v[c].y);
+            }
+            max_part[part][row] = m;
+            fence_proxy_async_smem();         // reads of the raw stage before its refill
+            if (!named_bar_and(1, 256, okf)) break;
+            if (tid == 0) mbar_arrive(smem_u32(&empty[s]));
+            m = fmaxf(max_part[0][row], max_part[1][row]);
+            int ex = 0;
+            frexpf(m, &ex);                   // m < 2^ex (m = 0: ex = 0)
+            ex = max(ex, -100);               // keep 2^(8-ex) finite
+            const float sc = ldexpf(1.f, 8 - ex);      // |x * sc| < 256
+            const float2 scale = make_float2(sc, sc);
+            const uint32_t ab = j & 1u;
+            const bool oka = mbar_wait_or_abort(smem_u32(&a_empty[ab]), ((j >> 1) & 1u) ^ 1u, abort);
+            if (!named_bar_and(1, 256, oka)) break;
+            tc_fence_after();
+            // slot j & 3 was last read by the epilogue of tile j - 4, which finished
+            // before the MMAs of tile j - 2 were issued, whose completion released
+            // a_empty[ab]
+            if (part == 0) row_scale[j & 3u][row] = ldexpf(bsc, ex - 8);
+            if constexpr (XP) xor_unpermute(v, xl, a.xt);   // back in member order (x < HALF)
+            // three 9-bit slices, one FP16 pair (re, im) per 32-bit TMEM column, stored
+            // eight members at a time
+            const uint32_t arow = tmem + S::A_COL0 + ab * S::A_SET + (((warp & 3u) * 32u) << 16) +
+                                  part * HALF;
 #pragma unroll
-                for (uint32_t c0 = 0; c0 < HALF; c0 += 8) {
-                    uint32_t w1[8], w2[8], w3[8];
+            for (uint32_t c0 = 0; c0 < HALF; c0 += 8) {
+                uint32_t w1[8], w2[8], w3[8];
 #pragma unroll
-                    for (uint32_t c = 0; c < 8; ++c) slices(v[c0 + c], scale, w1[c], w2[c], w3[c]);
-                    tmem_st8_async(arow + c0, w1);
-                    tmem_st8_async(arow + S::A_COLS + c0, w2);
-                    tmem_st8_async(arow + 2 * S::A_COLS + c0, w3);
-                }
-                tmem_wait_st();
-                tc_fence_before();
-                named_bar(1, 256);                // also: max_part is free for the next subtile
-                if (tid == 0) {
-                    mbar_arrive(smem_u32(&a_full[ab]));
-                    mbar_arrive(smem_u32(&scale_full[js & 3u]));
-                }
+                for (uint32_t c = 0; c < 8; ++c) slices(v[c0 + c], scale, w1[c], w2[c], w3[c]);
+                tmem_st8_async(arow + c0, w1);
+                tmem_st8_async(arow + S::A_COLS + c0, w2);
+                tmem_st8_async(arow + 2 * S::A_COLS + c0, w3);
+            }
+            tmem_wait_st();
+            tc_fence_before();
+            named_bar(1, 256);                // also: max_part is free for the next tile
+            if (tid == 0) {
+                mbar_arrive(smem_u32(&a_full[ab]));
+                mbar_arrive(smem_u32(&scale_full[j & 3u]));
             }
         }
     } else if (warp < S::W_STORE) {
@@ -580,9 +587,7 @@ __global__ void __launch_bounds__(608, 1) apply_tc(const __grid_constant__ TcArg
         const uint32_t quad = warp & 3u;          // TMEM lanes 32*quad .. 32*quad+31
         const uint32_t row = quad * 32u + lane;
         const uint32_t part = (warp - S::W_EPI) >> 2;
-        uint32_t gb[SUB];
-#pragma unroll
-        for (uint32_t sub = 0; sub < SUB; ++sub) gb[sub] = group_base(sub * S::ROWS + row);
+        const uint32_t gbase = group_base(row);
         const uint32_t xl = (lane >> a.xs) & ((1u << a.xt) - 1u);
         uint32_t cx = 0;
 #pragma unroll
@@ -593,44 +598,46 @@ __global__ void __launch_bounds__(608, 1) apply_tc(const __grid_constant__ TcArg
         for (unsigned long long t = first; t < tend && ok; t += step, ++j) {
             const uint32_t ob = j % NOUT;
             float2 *out = reinterpret_cast<float2 *>(smem + S::OFF_OUT + ob * S::TILE_BYTES);
+            const uint32_t b = j & 1u;
+            ok = ok && mbar_wait_or_abort(smem_u32(&d_full[b]), (j >> 1) & 1u, abort);
+            ok = ok && mbar_wait_or_abort(smem_u32(&scale_full[j & 3u]), (j >> 2) & 1u, abort);
+            ok = ok && mbar_wait_or_abort(smem_u32(&out_free[ob]), ((j / NOUT) & 1u) ^ 1u, abort);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc_fence_after();
+            const float osc1 = row_scale[j & 3u][row];
+            const float2 osc = make_float2(osc1, osc1);
+            const uint32_t lane_addr = tmem + b * S::ACC + ((quad * 32u) << 16) + part * HALF * 2u;
+            float2 o[XP ? HALF : 1];
 #pragma unroll
-            for (uint32_t sub = 0; sub < SUB; ++sub) {
-                const uint32_t js = j * SUB + sub, b = js & 1u;
-                ok = ok && mbar_wait_or_abort(smem_u32(&d_full[b]), (js >> 1) & 1u, abort);
-                ok = ok && mbar_wait_or_abort(smem_u32(&scale_full[js & 3u]), (js >> 2) & 1u, abort);
-                if (sub == 0) ok = ok && mbar_wait_or_abort(smem_u32(&out_free[ob]), ((j / NOUT) & 1u) ^ 1u, abort);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
-                tc_fence_after();
-                const uint32_t gbase = gb[sub];
-                const float osc1 = row_scale[js & 3u][row];
-                const float2 osc = make_float2(osc1, osc1);
-                const uint32_t lane_addr = tmem + b * S::ACC + ((quad * 32u) << 16) + part * HALF * 2u;
-                float2 o[XP ? HALF : 1];
+            for (uint32_t c0 = 0; c0 < 2u * HALF; c0 += 16) {
+                float d0[16], d12[16];
+                tmem_ld16x2(lane_addr + c0, lane_addr + KD + c0, d0, d12);
 #pragma unroll
-                for (uint32_t c0 = 0; c0 < 2u * HALF; c0 += 16) {
-                    float d0[16], d12[16];
-                    tmem_ld16x2(lane_addr + c0, lane_addr + KD + c0, d0, d12);
-#pragma unroll
-                    for (uint32_t i = 0; i < 16; i += 2) {
-                        const float2 x = __fmul2_rn(__fadd2_rn(make_float2(d0[i], d0[i + 1]),
-                                                               make_float2(d12[i], d12[i + 1])), osc);
-                        // in member order each chunk of eight members is written as soon as it
-                        // is formed (fewer live registers than holding the half row)
-                        if constexpr (XP) o[(c0 + i) / 2] = x;
-                        else out[gbase ^ member_off(part * HALF + (c0 + i) / 2)] = x;
+                for (uint32_t i = 0; i < 16; i += P0 ? 4 : 2) {
+                    const float2 x = __fmul2_rn(__fadd2_rn(make_float2(d0[i], d0[i + 1]),
+                                                           make_float2(d12[i], d12[i + 1])), osc);
+                    if constexpr (P0) {
+                        const float2 y = __fmul2_rn(__fadd2_rn(make_float2(d0[i + 2], d0[i + 3]),
+                                                               make_float2(d12[i + 2], d12[i + 3])), osc);
+                        *reinterpret_cast<float4 *>(out + (gbase ^ member_off(part * HALF + (c0 + i) / 2))) =
+                            make_float4(x.x, x.y, y.x, y.y);
+                        continue;
                     }
-                }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&d_empty[b]));
-                if constexpr (XP) {
-                    xor_unpermute(o, xl, a.xt);   // o[c] = member c ^ x (x < HALF)
-#pragma unroll
-                    for (uint32_t c = 0; c < HALF; ++c) out[gbase ^ member_off(part * HALF + c) ^ cx] = o[c];
+                    // in member order each chunk of eight members is written as soon as it
+                    // is formed (fewer live registers than holding the half row)
+                    if constexpr (XP) o[(c0 + i) / 2] = x;
+                    else out[gbase ^ member_off(part * HALF + (c0 + i) / 2)] = x;
                 }
             }
-            if (!ok) break;
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&d_empty[b]));
+            if constexpr (XP) {
+                xor_unpermute(o, xl, a.xt);   // o[c] = member c ^ x (x < HALF)
+#pragma unroll
+                for (uint32_t c = 0; c < HALF; ++c) out[gbase ^ member_off(part * HALF + c) ^ cx] = o[c];
+            }
             fence_proxy_async_smem();             // the bulk store reads them
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&out_full[ob]));
@@ -711,24 +718,20 @@ sv_status encode_rows_map(void *buf, unsigned long long bytes, uint32_t seg_byte
 
 template <int K>
 sv_status launch_tc_t(sv_state *s, const svi::Gate &g) {
-    using S = TcShape<K, 1>;
-    using S2 = TcShape<K, 2>;
+    using S = TcShape<K>;
     constexpr uint32_t D = S::D;
     static std::once_flag once;
     static cudaError_t init_err = cudaSuccess;
     std::call_once(once, [] {
-        init_err = cudaFuncSetAttribute(apply_tc<K, false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)S::SMEM);
-        if (init_err == cudaSuccess)
-            init_err = cudaFuncSetAttribute(apply_tc<K, true, 1>,
-                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
+        auto allow = [](auto kernel) {
+            if (init_err == cudaSuccess)
+                init_err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
+        };
+        allow(apply_tc<K, false>);
+        allow(apply_tc<K, true>);
         if constexpr (K == 5) {
-            if (init_err == cudaSuccess)
-                init_err = cudaFuncSetAttribute(apply_tc<K, false, 1, false, true>,
-                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
-            if (init_err == cudaSuccess)
-                init_err = cudaFuncSetAttribute(apply_tc<K, false, 2, false, true>,
-                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S2::SMEM);
+            allow(apply_tc<K, false, false, true>);
+            allow(apply_tc<K, false, false, true, true>);
         }
     });
     if (init_err != cudaSuccess)
@@ -738,15 +741,9 @@ sv_status launch_tc_t(sv_state *s, const svi::Gate &g) {
     // 8-byte accesses: bank pair = tile bits 0..3; targets there get lane-dependent order
     uint32_t tl = 0;
     while (tl < (uint32_t)K && p.lp[tl] < 4u) ++tl;
-    // width 5 on states of at least 13 qubits: two subtiles per stage (segments twice as
-    // long, half the per-stage work) with the swizzled tensor-map staging, whatever the
-    // targets (no XOR member order); otherwise one subtile, XOR order for bank-bit targets
-    // (one subtile while every SM has at most eight tiles, up to 22 qubits: a pass is then a few
-    // tiles' latency, and a second subtile adds to it: 18 qubits 7.25 -> 5.54 us per pass, 20
-    // qubits 7.83 -> 7.34, 22 qubits 15.1 -> 14.4; from 23 qubits two subtiles are as fast or faster)
-    const bool swz = K == 5 && s->n >= S2::TB;
-    const bool wide = swz && p.ntiles > 8ull * (unsigned long long)s->num_sms;
-    if (wide) p = make_plan(s->n, K, g.t, S2::TB);
+    // width 5 on states of at least 13 qubits: the swizzled tensor-map staging, whatever the
+    // targets (no XOR member order); otherwise XOR order for bank-bit targets
+    const bool swz = K == 5 && s->n >= K + 8u;
     if (swz) tl = 0;
     TcArgs<K> a;
     a.box_rows = a.boxes = 0;
@@ -776,6 +773,13 @@ sv_status launch_tc_t(sv_state *s, const svi::Gate &g) {
     a.psi = s->buf;
     a.err = reinterpret_cast<int *>(s->ws + svi::WS_ERR);
     a.ntiles = p.ntiles;
+    // Two tiles in flight per SM (64 KiB at K = 5, 10 MB in all) keep HBM busy; more of them queue up
+    // in front of the stores: 28 qubits, targets 6-10, 694 us per pass with four tiles in flight, 641
+    // with two; targets 7 and 24-27 699 and 640.  Tiles in 1 KiB pieces (five high targets)
+    // have longer latencies and want all stages: targets 23-27 636 us with four, 671 with two.
+    // (Two 32 KiB tiles per stage and transfer, the form for more than 22 qubits before: 657-669 us,
+    // 24 qubits 47-48.5 against 45-46 us.)
+    a.depth = K == 5 && p.h < K ? 2u : S::NS;
     a.L = p.L;
     a.h = p.h;
     for (int j = 0; j < SV_MAX_K; ++j) a.hi[j] = p.hi[j];
@@ -783,31 +787,25 @@ sv_status launch_tc_t(sv_state *s, const svi::Gate &g) {
     a.xs = 4u - tl;
     a.xt = std::min(tl, (uint32_t)K - 1u);   // permute within a worker's half of the members
     const unsigned grid = (unsigned)std::min<unsigned long long>(p.ntiles, (unsigned long long)s->num_sms);
-    cudaError_t e = cudaSuccess;
     // with eight worker warps per role the permutation costs less than even 2-way conflicts
-    if (swz && !wide) {
-        if constexpr (K == 5) e = launch_pass(apply_tc<K, false, 1, false, true>, dim3(grid), S::THREADS, S::SMEM, s->stream, a);
-    } else if (swz) {
-        if constexpr (K == 5) e = launch_pass(apply_tc<K, false, 2, false, true>, dim3(grid), S2::THREADS, S2::SMEM, s->stream, a);
-    } else if (a.xt >= 1) {
-        e = launch_pass(apply_tc<K, true, 1>, dim3(grid), S::THREADS, S::SMEM, s->stream, a);
-    } else {
-        e = launch_pass(apply_tc<K, false, 1>, dim3(grid), S::THREADS, S::SMEM, s->stream, a);
-    }
-    SV_CUDA(e);
+    auto kernel = a.xt >= 1 ? apply_tc<K, true> : apply_tc<K, false>;
+    if constexpr (K == 5)
+        if (swz) kernel = p.lp[3] == 3 ? apply_tc<K, false, false, true, true> : apply_tc<K, false, false, true>;
+    SV_CUDA(launch_pass(kernel, dim3(grid), S::THREADS, S::SMEM, s->stream, a));
     return SV_OK;
 }
 
 // Batched launches (sv_batch_apply): complex64 gates on states of at least 13 qubits (12 for
 // widths 4 and 5) run as width-5 gates (a narrower gate widened by identity qubits, chosen as in
-// widen_gate) with one MMA subtile per stage and the swizzled tensor-map staging (SW), like single
-// states.
+// widen_gate) with the swizzled tensor-map staging (SW), like single states.
 static cudaError_t tc_batch_setup() {
     static std::once_flag once;
     static cudaError_t err = cudaSuccess;
     std::call_once(once, [] {
-        err = cudaFuncSetAttribute(apply_tc<5, false, 1, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)TcShape<5, 1, true>::SMEM);
+        constexpr int smem = (int)TcShape<5, true>::SMEM;
+        err = cudaFuncSetAttribute(apply_tc<5, false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (err == cudaSuccess)
+            err = cudaFuncSetAttribute(apply_tc<5, false, true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     });
     return err;
 }
@@ -839,7 +837,7 @@ static void widen_targets(uint32_t n, uint32_t k, const uint32_t *t, uint32_t (&
         }
 }
 
-size_t tc_batch_image_bytes() { return TcShape<5, 1, true>::B_SET; }
+size_t tc_batch_image_bytes() { return TcShape<5, true>::B_SET; }
 
 sv_status launch_tc_pack(const sv_batch_launch *L, const size_t *tab_off, uint32_t ngates, const void *utab,
                          void *images, float *bscale) {
@@ -863,7 +861,7 @@ sv_status launch_tc_pack(const sv_batch_launch *L, const size_t *tab_off, uint32
 }
 
 sv_status launch_tc_batch(const sv_batch_launch &L) {
-    using S = TcShape<5, 1, true>;
+    using S = TcShape<5, true>;
     const cudaError_t e0 = tc_batch_prepare();
     if (e0 != cudaSuccess)
         return svi::set_error(SV_ERR_CUDA, std::string("batched tensor-core kernel setup: ") + cudaGetErrorString(e0));
@@ -887,12 +885,14 @@ sv_status launch_tc_batch(const sv_batch_launch &L) {
     for (int j = 0; j < 5; ++j) a.lp[j] = p.lp[j];
     a.xs = 0;
     a.xt = 0;
+    a.depth = S::NS;
     a.images = static_cast<const unsigned char *>(L.images);
     a.bscale = L.bscale;
     a.tps = (uint32_t)__builtin_ctzll(p.ntiles);
     a.n = L.n;
     const unsigned grid = (unsigned)std::min<unsigned long long>(a.ntiles, (unsigned long long)L.num_sms);
-    SV_CUDA(launch_pass(apply_tc<5, false, 1, true, true>, dim3(grid), S::THREADS, S::SMEM, L.stream, a));
+    SV_CUDA(launch_pass(p.lp[3] == 3 ? apply_tc<5, false, true, true, true> : apply_tc<5, false, true, true>,
+                        dim3(grid), S::THREADS, S::SMEM, L.stream, a));
     return SV_OK;
 }
 
@@ -901,19 +901,19 @@ sv_status launch_tc_batch(const sv_batch_launch &L) {
 namespace svi {
 
 // Width 4 and 5, and on states of at least 13 qubits every dense width (narrower gates run
-// as width-5 ones, U (x) I, on the swizzled two-subtile kernel: at 30 qubits its passes
+// as width-5 ones, U (x) I, on the swizzled kernel: at 30 qubits its passes
 // take 2.59-2.74 ms against 2.74 for the width-2/3 CUDA-core kernel).
 bool tc_eligible(const sv_state *s, const Gate &g) {
     if (s->dtype != SV_C64 || (s->policy & SV_POLICY_NO_TENSOR_CORES)) return false;
     if (g.k == 4 || g.k == 5) return s->n >= g.k + 7;
-    return g.k >= 1 && s->n >= svk::TcShape<5, 2>::TB;
+    return g.k >= 1 && s->n >= svk::TcShape<5>::TB + 1;
 }
 
 // Width-4 gates run as width-5 ones (U (x) I) where the state allows: the k = 5 kernel
 // moves a tile with half the per-tile overhead of the k = 4 one for the same bytes.
 sv_status launch_apply_tc(sv_state *s, const Gate &g) {
     if (g.k == 5) return svk::launch_tc_t<5>(s, g);
-    if (s->n >= svk::TcShape<5, 1>::TB) return svk::launch_tc_t<5>(s, widen_gate(g, s->n, 5));
+    if (s->n >= svk::TcShape<5>::TB) return svk::launch_tc_t<5>(s, widen_gate(g, s->n, 5));
     return svk::launch_tc_t<4>(s, g);
 }
 
