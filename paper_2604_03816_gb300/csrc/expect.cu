@@ -23,9 +23,9 @@
 // products and keep the general kernel.
 //
 // Measured, a transverse-field Ising chain on 26 qubits, complex64 (25 ZZ and 26 X terms):
-// 10.48 ms with one FP64 weight per amplitude and one pass per X-part -> 0.73 ms: z_sum 0.10 ms
-// (5.3 TB/s; 25 FP32 operations per amplitude), four x_sum passes of 0.12-0.16 ms (3.4-4.6
-// TB/s; 40 instructions per amplitude with twelve terms, then the latency of 16 warps per SM).
+// 10.48 ms with one FP64 weight per amplitude and one pass per X-part -> 0.58 ms: z_sum 0.10 ms
+// (5.3 TB/s; 25 FP32 operations per amplitude), four x_sum passes of about 0.11 ms (4.8
+// TB/s; the latency of 24 warps per SM).
 // complex128 is bound by the FP64 pipe.
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -298,15 +298,21 @@ __device__ __forceinline__ R pair_any(const C (&v)[16], uint32_t signs, uint32_t
     return odd ? pair_sum<R, XR, true, false>(v, signs) : pair_sum<R, XR, false, false>(v, signs);
 }
 
-template <typename R>
-__global__ void __launch_bounds__(THREADS, 2) x_sum(const __grid_constant__ XArgs a) {
+// PLAIN: every term is a plain flip (at most four per set): running sums in registers, the sets
+// unrolled.  Without the sums' 32 KiB three blocks fit an SM (complex64), 24 warps to hide latency:
+// a 26-qubit field of 26 X terms and its ZZ chain 693 -> 577 us (two blocks: 641).
+template <typename R, bool PLAIN>
+constexpr int x_blocks = PLAIN && sizeof(R) == 4 ? 3 : 2;
+template <typename R, bool PLAIN>
+__global__ void __launch_bounds__(THREADS, x_blocks<R, PLAIN>) x_sum(const __grid_constant__ XArgs a) {
     using C = typename Geo<R>::C;
     using S = typename Sum<R>::T;
     constexpr uint32_t TILE = (1u << Geo<R>::T) * (uint32_t)sizeof(C);
     constexpr uint32_t NT = (1u << Geo<R>::T) / 16u;           // threads that hold amplitudes
     extern __shared__ __align__(1024) unsigned char smem[];    // two tiles, then the sums
     __shared__ __align__(8) unsigned long long full[2];
-    S *sums = reinterpret_cast<S *>(smem + 2 * TILE);          // [term][NT]
+    S *sums = reinterpret_cast<S *>(smem + 2 * TILE);          // [term][NT] (not PLAIN)
+    S racc[PLAIN ? X_SETS * 4 : 1];                            // PLAIN: [set][register bit]
     const uint32_t tid = threadIdx.x, lane = tid & 31u;
     const uint32_t nseg = 1u << a.h, seg_amps = 1u << a.L;
     const uint32_t nact = 1u << (a.tb - 4u);
@@ -317,8 +323,12 @@ __global__ void __launch_bounds__(THREADS, 2) x_sum(const __grid_constant__ XArg
         svk::fence_mbar_init();
     }
     const uint32_t nterms = a.nterms;
-    if (act)
+    if (PLAIN) {
+#pragma unroll
+        for (uint32_t t = 0; t < (PLAIN ? X_SETS * 4 : 1); ++t) racc[t].clear();
+    } else if (act) {
         for (uint32_t t = 0; t < nterms; ++t) sums[t * NT + tid].clear();
+    }
     const unsigned long long my_z = lane < nterms ? a.term[lane].z : 0ull;
     svk::SegLanes sl;
     sl.init(a.L, a.h, a.hi, lane);
@@ -355,26 +365,46 @@ __global__ void __launch_bounds__(THREADS, 2) x_sum(const __grid_constant__ XArg
         const C *tile = reinterpret_cast<const C *>(smem + s * TILE);
         // bit i: (-1)^{|base & z_i|}, lane i's term
         const uint32_t tile_signs = __ballot_sync(0xffffffffu, __popcll(sl.base(t) & my_z) & 1);
-        if (act)
+        // the sixteen amplitudes of a register set
+        auto read_set = [&](uint32_t set, C (&v)[16]) {
+            uint32_t g = tid;
+            uint32_t rb[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                g = svk::insert_zero32(g, a.rbit[set][q]);
+                rb[q] = 1u << a.rbit[set][q];
+                rb[q] = sizeof(R) == 4 ? svk::swz128(rb[q]) : svk::swz128_16(rb[q]);
+            }
+            g = sizeof(R) == 4 ? svk::swz128(g) : svk::swz128_16(g);
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                uint32_t o = g;
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if ((k >> q) & 1) o ^= rb[q];
+                v[k] = tile[o];
+            }
+        };
+        if constexpr (PLAIN) {
+            if (act) {
+#pragma unroll
+                for (uint32_t set = 0; set < X_SETS; ++set) {
+                    if (set >= a.nsets) break;
+                    C v[16];
+                    read_set(set, v);
+                    const R x[4] = {pair_sum<R, 1, false, false>(v, 0), pair_sum<R, 2, false, false>(v, 0),
+                                    pair_sum<R, 4, false, false>(v, 0), pair_sum<R, 8, false, false>(v, 0)};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int32_t i = a.plain[set][q];
+                        if (i >= 0) racc[set * 4 + q].add(flip(x[q], ((tile_signs >> i) & 1u) << 31));
+                    }
+                }
+            }
+        } else if (act) {
             for (uint32_t set = 0; set < a.nsets; ++set) {
-                uint32_t g = tid;
-                uint32_t rb[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    g = svk::insert_zero32(g, a.rbit[set][q]);
-                    rb[q] = 1u << a.rbit[set][q];
-                    rb[q] = sizeof(R) == 4 ? svk::swz128(rb[q]) : svk::swz128_16(rb[q]);
-                }
-                g = sizeof(R) == 4 ? svk::swz128(g) : svk::swz128_16(g);
                 C v[16];
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    uint32_t o = g;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        if ((k >> q) & 1) o ^= rb[q];
-                    v[k] = tile[o];
-                }
+                read_set(set, v);
                 auto accumulate = [&](R x, uint32_t i) {
                     S acc = sums[i * NT + tid];
                     acc.add(flip(x, ((tile_signs >> i) & 1u) << 31));
@@ -406,6 +436,7 @@ __global__ void __launch_bounds__(THREADS, 2) x_sum(const __grid_constant__ XArg
                     accumulate(x, i);
                 }
             }
+        }
         svk::fence_proxy_async_smem();        // reads of this tile before its refill
         __syncthreads();
         const unsigned long long t2 = t + 2ull * gridDim.x;
@@ -417,9 +448,17 @@ __global__ void __launch_bounds__(THREADS, 2) x_sum(const __grid_constant__ XArg
             uint32_t g = tid;
 #pragma unroll
             for (int q = 0; q < 4; ++q) g = svk::insert_zero32(g, a.rbit[set][q]);
-            for (uint32_t i = a.first[set] - a.nplain[set]; i < a.last[set]; ++i) {
-                const double v = sums[i * NT + tid].value() * a.term[i].coef;
+            auto weigh = [&](const S &sum, uint32_t i) {
+                const double v = sum.value() * a.term[i].coef;
                 acc += (__popc(g & a.term[i].zt) & 1) ? -v : v;
+            };
+            if constexpr (PLAIN) {
+                // register indices stay constants: each set picks its own four
+#pragma unroll
+                for (uint32_t t = 0; t < X_SETS * 4; ++t)
+                    if (t / 4 == set && a.plain[set][t % 4] >= 0) weigh(racc[t], (uint32_t)a.plain[set][t % 4]);
+            } else {
+                for (uint32_t i = a.first[set] - a.nplain[set]; i < a.last[set]; ++i) weigh(sums[i * NT + tid], i);
             }
         }
     const double r = block_sum(acc);
@@ -468,10 +507,6 @@ struct Partials {
         return SV_OK;
     }
 };
-
-int blocks_for(const sv_state *s, unsigned long long ntiles) {
-    return (int)std::min<unsigned long long>(ntiles, 2ull * (unsigned long long)s->num_sms);
-}
 
 // The Z strings t[0 .. n) on `states` states of nq qubits at psi, tables in `tables`: every pass
 // asks `reserve` where its partials go (blocks per state, state by state) and says with `ran`
@@ -648,7 +683,12 @@ sv_status x_pass(sv_state *s, Partials &P, const std::vector<Term> &t, std::vect
                                               (uint32_t)sizeof(typename Geo<R>::C) << L, &a.tmap, &a.box_rows, &a.boxes);
     if (st != SV_OK) return st;
     a.ntiles = 1ull << (s->n - a.tb);
-    const int nb = blocks_for(s, a.ntiles);
+    uint32_t flips = 0;
+    for (uint32_t q = 0; q < ns; ++q) flips += a.nplain[q];
+    const bool plain = flips == total;
+    // as many blocks as the device holds
+    const int nb = (int)std::min<unsigned long long>(a.ntiles, (unsigned long long)(plain ? x_blocks<R, true> : x_blocks<R, false>) *
+                                                                   (unsigned long long)s->num_sms);
     const sv_status rs = P.reserve(nb);
     if (rs != SV_OK) return rs;
     a.partial = P.part();
@@ -658,10 +698,13 @@ sv_status x_pass(sv_state *s, Partials &P, const std::vector<Term> &t, std::vect
     static std::once_flag once;
     static cudaError_t err = cudaSuccess;
     std::call_once(once, [] {
-        err = cudaFuncSetAttribute(x_sum<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        err = cudaFuncSetAttribute(x_sum<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (err == cudaSuccess)
+            err = cudaFuncSetAttribute(x_sum<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * tile_bytes));
     });
     SV_CUDA(err);
-    SV_CUDA(svk::launch_pass(x_sum<R>, dim3(nb), THREADS, smem, s->stream, a));
+    SV_CUDA(plain ? svk::launch_pass(x_sum<R, true>, dim3(nb), THREADS, 2 * tile_bytes, s->stream, a)
+                           : svk::launch_pass(x_sum<R, false>, dim3(nb), THREADS, smem, s->stream, a));
     P.used += nb;
     return SV_OK;
 }
