@@ -22,12 +22,12 @@
 //
 // What bounds it: issue and the integer pipe (about 160 instructions per amplitude, 4250 cycles
 // per 2048 amplitudes where HBM needs 3030).  So the workers do not meet: two transform groups of
-// four warps take alternate subtiles, whole rows per warp (eight warps on one subtile exchanged
+// four warps take alternate tiles, whole rows per warp (eight warps on one tile exchanged
 // row maxima and met twice: 2430 cycles more), the epilogue's hand over by counted arrivals, and
 // the short forms of the split and of the scaling (rows whose exponents allow them, a vote per warp)
 // save a quarter of the integer instructions.  More workers do not help (16 epilogue warps: the
-// same time; 16 transform warps: 5% slower).  28-qubit grid circuit: 238.5 -> 196 ms, with the stores of
-// SUB = 2 by halves 175.6 ms.
+// same time; 16 transform warps: 5% slower).  28-qubit grid circuit: 238.5 -> 196 ms, with a store warp and
+// one swizzled tile per stage 169.8 ms.
 //
 // Gates on fewer than four qubits are widened to four (U (x) I on extra qubits chosen
 // above bit 4, so a warp's rows stay contiguous in shared memory).
@@ -53,21 +53,19 @@
 
 namespace svk {
 
-// SUB: MMA subtiles (128 groups each) per TMA stage.  SUB = 2 doubles the contiguous
-// segments of launches whose targets sit above the low index bits (4 KiB instead of 2).
-template <int SUB = 1>
-struct Tc64S {
+// One tile is one MMA (128 groups): 32 KiB.
+struct Tc64 {
     static constexpr uint32_t K = 4;
     static constexpr uint32_t D = 16;                     // amplitudes per group
     static constexpr uint32_t KD = 32;                    // real K = N
-    static constexpr uint32_t ROWS = 128;                 // groups per MMA subtile (MMA M)
-    static constexpr uint32_t TB = 11 + (SUB == 2 ? 1u : 0u);   // tile bits
-    static constexpr uint32_t TILE_BYTES = SUB * ROWS * D * 16u;  // 32 or 64 KB
+    static constexpr uint32_t ROWS = 128;                 // groups per tile (MMA M)
+    static constexpr uint32_t TB = 11;                    // tile bits
+    static constexpr uint32_t TILE_BYTES = ROWS * D * 16u;
     static constexpr uint32_t B_BYTES = KD * KD * 2u;     // one FP16 digit slice of R
     static constexpr uint32_t NB = 12;                    // B_j and B_j 2^-9, j = 0..5
     static constexpr uint32_t SBO = (KD / 8u) * 128u;
-    static constexpr uint32_t NS = SUB == 2 ? 2u : 4u;    // raw stages
-    static constexpr uint32_t NOUT = SUB == 2 ? 1u : 2u;  // output staging tiles (two subtiles)
+    static constexpr uint32_t NS = 4;                     // raw stages
+    static constexpr uint32_t NOUT = 2;                   // output staging tiles
     static constexpr uint32_t NACC = 5;                   // D0, D1, D2, D3, D45
     static constexpr uint32_t ACC = NACC * KD;            // TMEM columns of one D set
     static constexpr uint32_t A_COLS = KD / 2u;           // TMEM columns of one A digit slice
@@ -82,24 +80,21 @@ struct Tc64S {
     // warps 0-7 transform, 8 producer, 9 MMA issuer, 10-17 epilogue, 18 TMA stores
     static constexpr uint32_t W_PROD = 8, W_MMA = 9, W_EPI = 10, W_STORE = 18;
 };
-using Tc64 = Tc64S<1>;
 
 struct Tc64Args {
-    // swizzled launches (SW): the state as a 2-D tensor of 128-byte rows (8 amplitudes),
-    // `boxes` boxes of box_rows rows per segment, 128-byte swizzle in shared memory
+    // the state as a 2-D tensor of 128-byte rows (8 amplitudes), `boxes` boxes of box_rows rows per
+    // segment, 128-byte swizzle in shared memory
     CUtensorMap tmap;
     // U on the fixed-point grid of its largest entry: (re, im) of entry (r, c), row-major; the
     // prologue cuts each into six digits (expand_b64)
     alignas(16) longlong2 bx[16 * 16];
     uint32_t box_rows, boxes;
     int b_exp;               // max |U| < 2^b_exp
-    void *psi;
     int *err;
     unsigned long long ntiles;
     uint32_t L, h;
     uint32_t hi[SV_MAX_K];
     uint32_t lp[4];
-    uint32_t sb;             // the highest tile bit below L that is no target
 };
 
 // Digit-pair word -> FP16 pair of digits: the patterns read 2048 + 2u, and
@@ -188,29 +183,26 @@ __device__ __forceinline__ void cut_members(const uint4 (&v)[4], uint32_t emax, 
     }
 }
 
-// The pipelines count tiles (j: raw stage) and MMA subtiles (js = j SUB + sub: A and D buffers, row
-// exponents, output staging).
-// SW: tiles move by 2-D tensor-map copies with the 128-byte swizzle and the roles address
-// them through it, so a warp's lanes reach different banks whatever the targets.  The swizzle is applied to the group base and the target
-// bits, which then combine by XOR.
-template <int SUB = 1, bool SW = false>
+// The pipelines count this CTA's tiles (j).
+// Tiles move by 2-D tensor-map copies with the 128-byte swizzle and the roles address
+// them through it, so a warp's lanes reach different banks whatever the targets.  The swizzle is
+// applied to the group base and the target bits, which then combine by XOR.  (1-D bulk copies where
+// at most one target is among bits 0-2: the same time, 8% more with one.)
 __global__ void __launch_bounds__(608, 1) apply_tc64(const __grid_constant__ Tc64Args a) {
-    using S = Tc64S<SUB>;
+    using S = Tc64;
     constexpr uint32_t KD = S::KD, NS = S::NS;
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) unsigned long long full[NS], empty[NS];
     __shared__ __align__(8) unsigned long long a_full[2], a_empty[2], d_full[2], d_empty[2];
-    __shared__ __align__(8) unsigned long long scale_full[4];   // row exponents, subtile js -> js & 3
-    __shared__ __align__(8) unsigned long long out_full[2], out_free[2];   // staged subtiles
+    __shared__ __align__(8) unsigned long long scale_full[4];   // row exponents, tile j -> j & 3
+    __shared__ __align__(8) unsigned long long out_full[2], out_free[2];   // staged tiles
     __shared__ int row_exp[4][128];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
     unsigned char *sB = smem;
-    double2 *psi = reinterpret_cast<double2 *>(a.psi);
     const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     const uint32_t seg_amps = 1u << a.L;
-    const uint32_t seg_bytes = seg_amps * 16u;
     const uint32_t nseg = 1u << a.h;
 
     if (tid == 0) pass_trigger();
@@ -221,7 +213,7 @@ __global__ void __launch_bounds__(608, 1) apply_tc64(const __grid_constant__ Tc6
     if (tid == 0) {
         for (uint32_t s = 0; s < NS; ++s) {
             mbar_init(smem_u32(&full[s]), 1);
-            mbar_init(smem_u32(&empty[s]), 4 * SUB);     // one transform group per subtile
+            mbar_init(smem_u32(&empty[s]), 4);            // one transform group
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&a_full[b]), 4);       // one transform group
@@ -247,20 +239,19 @@ __global__ void __launch_bounds__(608, 1) apply_tc64(const __grid_constant__ Tc6
     const uint32_t tmem = tmem_slot;
     volatile int *abort = &abort_flag;
     const unsigned long long first = blockIdx.x, step = gridDim.x;
-    // this CTA's subtiles
-    const uint32_t nsub = a.ntiles > first ? (uint32_t)((a.ntiles - first + step - 1) / step) * SUB : 0u;
+    const uint32_t ntile = a.ntiles > first ? (uint32_t)((a.ntiles - first + step - 1) / step) : 0u;
 
     auto group_base = [&](uint32_t row) {
         uint32_t g = row;
 #pragma unroll
         for (int j = 0; j < 4; ++j) g = insert_zero32(g, a.lp[j]);
-        return SW ? swz128_16(g) : g;
+        return swz128_16(g);
     };
-    // tile offset of target j (swizzled with SW; four registers), and of group member c:
+    // tile offset of target j (swizzled; four registers), and of group member c:
     // the XOR of the offsets of its set bits; a member's index is group base XOR offset
     uint32_t tb[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) tb[j] = SW ? swz128_16(1u << a.lp[j]) : 1u << a.lp[j];
+    for (int j = 0; j < 4; ++j) tb[j] = swz128_16(1u << a.lp[j]);
     auto member_off = [&](uint32_t c) {
         uint32_t o = 0;
 #pragma unroll
@@ -285,24 +276,19 @@ __global__ void __launch_bounds__(608, 1) apply_tc64(const __grid_constant__ Tc6
             __syncwarp();
             if (lane < nseg) {
                 double2 *dst = reinterpret_cast<double2 *>(smem + S::OFF_RAW + s * S::TILE_BYTES);
-                if constexpr (SW) {
-                    // segment = `boxes` boxes of box_rows 128-byte rows (8 amplitudes each)
-                    const int32_t row0 = (int32_t)((sl.base(t) + sl.my_off) >> 3);
-                    const uint32_t d0 = smem_u32(dst + (size_t)lane * seg_amps);
-                    for (uint32_t bx = 0; bx < a.boxes; ++bx)
-                        tma_load_2d(d0 + bx * a.box_rows * 128u, &a.tmap, 0, row0 + (int32_t)(bx * a.box_rows), bar);
-                } else {
-                    bulk_g2s(smem_u32(dst + (size_t)lane * seg_amps), psi + sl.base(t) + sl.my_off,
-                             seg_bytes, bar);
-                }
+                // segment = `boxes` boxes of box_rows 128-byte rows (8 amplitudes each)
+                const int32_t row0 = (int32_t)((sl.base(t) + sl.my_off) >> 3);
+                const uint32_t d0 = smem_u32(dst + (size_t)lane * seg_amps);
+                for (uint32_t bx = 0; bx < a.boxes; ++bx)
+                    tma_load_2d(d0 + bx * a.box_rows * 128u, &a.tmap, 0, row0 + (int32_t)(bx * a.box_rows), bar);
             }
         }
     } else if (warp == S::W_MMA) {
         // ------------------------------------------------------------ MMA issuer
         if (lane == 0) {
             const uint32_t B0 = smem_u32(sB);
-            for (uint32_t js = 0; js < nsub; ++js) {
-                const uint32_t b = js & 1u, u = js >> 1;
+            for (uint32_t j = 0; j < ntile; ++j) {
+                const uint32_t b = j & 1u, u = j >> 1;
                 if (!mbar_wait_or_abort(smem_u32(&a_full[b]), u & 1u, abort)) break;
                 if (!mbar_wait_or_abort(smem_u32(&d_empty[b]), (u & 1u) ^ 1u, abort)) break;
                 tc_fence_after();
@@ -330,19 +316,19 @@ __global__ void __launch_bounds__(608, 1) apply_tc64(const __grid_constant__ Tc6
         }
     } else if (warp < S::W_PROD) {
         // ------------------------------------------------------------ digit transform
-        // Two groups of four warps take alternate subtiles, one warp per TMEM lane quadrant and
+        // Two groups of four warps take alternate tiles, one warp per TMEM lane quadrant and
         // whole rows each, so that no warp waits for another.  Rolled loops over four members at
         // a time keep the code small (the roles run different code on every SM sub-partition).
         const uint32_t quad = warp & 3u, grp = warp >> 2;
         const uint32_t row = quad * 32u + lane;
         const uint32_t lo_off[4] = {0u, tb[0], tb[1], tb[0] ^ tb[1]};
+        const uint32_t gbase = group_base(row);
         const uint32_t arow = tmem + S::A_COL0 + grp * S::A_SET + ((quad * 32u) << 16);
-        for (uint32_t js = grp; js < nsub; js += 2) {
-            const uint32_t j = js / SUB, sub = js % SUB, s = j % NS;
+        for (uint32_t j = grp; j < ntile; j += 2) {
+            const uint32_t s = j % NS;
             const bool okf = mbar_wait_or_abort(smem_u32(&full[s]), (j / NS) & 1u, abort);
             if (!__all_sync(0xffffffffu, okf)) break;
             const double2 *rs = reinterpret_cast<const double2 *>(smem + S::OFF_RAW + s * S::TILE_BYTES);
-            const uint32_t gbase = group_base(sub * S::ROWS + row);
             uint32_t em = 0, mn = 0x7FFFFFFFu;    // largest and smallest |high word| of the row
 #pragma unroll 1
             for (uint32_t c0 = 0; c0 < 16u; c0 += 4) {
@@ -369,14 +355,14 @@ __global__ void __launch_bounds__(608, 1) apply_tc64(const __grid_constant__ Tc6
                 if (near) cut_members<true>(va, emax, w);
                 else cut_members<false>(va, emax, w);
                 if (c0 == 0) {
-                    // the A buffer is free once the MMAs of subtile js - 2 have completed
+                    // the A buffer is free once the MMAs of tile j - 2 have completed
                     oka = __all_sync(0xffffffffu,
-                                     mbar_wait_or_abort(smem_u32(&a_empty[grp]), ((js >> 1) & 1u) ^ 1u, abort));
+                                     mbar_wait_or_abort(smem_u32(&a_empty[grp]), ((j >> 1) & 1u) ^ 1u, abort));
                     if (!oka) break;
                     tc_fence_after();
-                    // slot js & 3 was last read by the epilogue of subtile js - 4, which finished
-                    // before the MMAs of subtile js - 2
-                    row_exp[js & 3u][row] = (int)emax;
+                    // slot j & 3 was last read by the epilogue of tile j - 4, which finished
+                    // before the MMAs of tile j - 2
+                    row_exp[j & 3u][row] = (int)emax;
                 }
 #pragma unroll
                 for (int i = 0; i < 6; ++i) tmem_st4_async(arow + i * S::A_COLS + c0, w[i]);
@@ -389,7 +375,7 @@ __global__ void __launch_bounds__(608, 1) apply_tc64(const __grid_constant__ Tc6
             if (lane == 0) {
                 mbar_arrive(smem_u32(&empty[s]));
                 mbar_arrive(smem_u32(&a_full[grp]));
-                mbar_arrive(smem_u32(&scale_full[js & 3u]));
+                mbar_arrive(smem_u32(&scale_full[j & 3u]));
             }
         }
     } else if (warp < S::W_STORE) {
@@ -398,17 +384,17 @@ __global__ void __launch_bounds__(608, 1) apply_tc64(const __grid_constant__ Tc6
         const uint32_t quad = warp & 3u;
         const uint32_t row = quad * 32u + lane;
         const uint32_t part = (warp - S::W_EPI) >> 2;
-        for (uint32_t js = 0; js < nsub; ++js) {
-            const uint32_t b = js & 1u;
-            double2 *out = reinterpret_cast<double2 *>(smem + S::OFF_OUT + (SUB == 1 ? b * S::TILE_BYTES : 0u));
-            const uint32_t gbase = group_base(js % SUB * S::ROWS + row);
-            bool ok = mbar_wait_or_abort(smem_u32(&d_full[b]), (js >> 1) & 1u, abort);
-            ok = ok && mbar_wait_or_abort(smem_u32(&scale_full[js & 3u]), (js >> 2) & 1u, abort);
-            ok = ok && mbar_wait_or_abort(smem_u32(&out_free[b]), ((js >> 1) & 1u) ^ 1u, abort);
+        const uint32_t gbase = group_base(row);
+        for (uint32_t j = 0; j < ntile; ++j) {
+            const uint32_t b = j & 1u;
+            double2 *out = reinterpret_cast<double2 *>(smem + S::OFF_OUT + b * S::TILE_BYTES);
+            bool ok = mbar_wait_or_abort(smem_u32(&d_full[b]), (j >> 1) & 1u, abort);
+            ok = ok && mbar_wait_or_abort(smem_u32(&scale_full[j & 3u]), (j >> 2) & 1u, abort);
+            ok = ok && mbar_wait_or_abort(smem_u32(&out_free[b]), ((j >> 1) & 1u) ^ 1u, abort);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
-            const int p = row_exp[js & 3u][row] + a.b_exp - 1078;   // out = Z 2^p
+            const int p = row_exp[j & 3u][row] + a.b_exp - 1078;   // out = Z 2^p
             const uint32_t lane_addr = tmem + b * S::ACC + ((quad * 32u) << 16);
             const bool p_safe = __all_sync(0xffffffffu, p >= -1022 && p <= 960);
             // eight columns (four members) of the five accumulators per step, both steps
@@ -443,29 +429,19 @@ __global__ void __launch_bounds__(608, 1) apply_tc64(const __grid_constant__ Tc6
         }
     } else {
         // ------------------------------------------------------------ TMA stores
-        // One subtile at a time.  With SUB = 2 the two of a tile are the halves of its staging
-        // that differ in bit sb, the highest tile bit that is no target: pieces of 2^sb amplitudes,
-        // one per segment unless targets sit right below L.
         SegLanes sl;
         sl.init(a.L, a.h, a.hi, lane);
-        for (uint32_t js = 0; js < nsub; ++js) {
-            const uint32_t ob = js & 1u;
-            const unsigned long long t = first + (unsigned long long)(js / SUB) * step;
-            const double2 *out = reinterpret_cast<const double2 *>(smem + S::OFF_OUT + (SUB == 1 ? ob * S::TILE_BYTES : 0u));
-            const bool ok = mbar_wait_or_abort(smem_u32(&out_full[ob]), (js >> 1) & 1u, abort);
+        for (uint32_t j = 0; j < ntile; ++j) {
+            const uint32_t ob = j & 1u;
+            const unsigned long long t = first + (unsigned long long)j * step;
+            const double2 *out = reinterpret_cast<const double2 *>(smem + S::OFF_OUT + ob * S::TILE_BYTES);
+            const bool ok = mbar_wait_or_abort(smem_u32(&out_full[ob]), (j >> 1) & 1u, abort);
             if (!__all_sync(0xffffffffu, ok)) break;
             if (lane < nseg) {
-                if constexpr (SW) {
-                    const int32_t row0 = (int32_t)((sl.base(t) + sl.my_off) >> 3);
-                    const uint32_t s0 = smem_u32(out + (size_t)lane * seg_amps);
-                    for (uint32_t bx = 0; bx < a.boxes; ++bx)
-                        tma_store_2d(&a.tmap, 0, row0 + (int32_t)(bx * a.box_rows), s0 + bx * a.box_rows * 128u);
-                } else if constexpr (SUB == 2) {
-                    for (uint32_t o = ob << a.sb; o < seg_amps; o += 2u << a.sb)
-                        bulk_s2g(psi + sl.base(t) + sl.my_off + o, smem_u32(out + (size_t)lane * seg_amps + o), 16u << a.sb);
-                } else {
-                    bulk_s2g(psi + sl.base(t) + sl.my_off, smem_u32(out + (size_t)lane * seg_amps), seg_bytes);
-                }
+                const int32_t row0 = (int32_t)((sl.base(t) + sl.my_off) >> 3);
+                const uint32_t s0 = smem_u32(out + (size_t)lane * seg_amps);
+                for (uint32_t bx = 0; bx < a.boxes; ++bx)
+                    tma_store_2d(&a.tmap, 0, row0 + (int32_t)(bx * a.box_rows), s0 + bx * a.box_rows * 128u);
             }
             bulk_commit();
             bulk_wait_read_all();                 // the staging is free again
@@ -483,18 +459,10 @@ __global__ void __launch_bounds__(608, 1) apply_tc64(const __grid_constant__ Tc6
 
 sv_status launch_tc64(sv_state *s, const svi::Gate &g0) {
     using S = Tc64;
-    using S2 = Tc64S<2>;
     static std::once_flag once;
     static cudaError_t init_err = cudaSuccess;
     std::call_once(once, [] {
-        init_err = cudaFuncSetAttribute(apply_tc64<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)S::SMEM);
-        if (init_err == cudaSuccess)
-            init_err = cudaFuncSetAttribute(apply_tc64<2>,
-                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S2::SMEM);
-        if (init_err == cudaSuccess)
-            init_err = cudaFuncSetAttribute(apply_tc64<1, true>,
-                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
+        init_err = cudaFuncSetAttribute(apply_tc64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
     });
     if (init_err != cudaSuccess)
         return svi::set_error(SV_ERR_CUDA, std::string("tensor-core kernel setup: ") +
@@ -505,27 +473,12 @@ sv_status launch_tc64(sv_state *s, const svi::Gate &g0) {
         gw = svi::widen_gate(g0, s->n, 4);
         g = &gw;
     }
-    Plan p = make_plan(s->n, 4, g->t, S::TB);
-    // 16-byte accesses: bank group = tile bits 0..2; the lowest targets there (at most
-    // two, the ones inside a group of four members) get a lane-dependent order
-    uint32_t tl = 0;
-    while (tl < 3u && p.lp[tl] < 3u) ++tl;
-    // without the member-order variant and with three or four targets above the low bits
-    // (segments of 4 KiB or less), two MMA subtiles per 64 KiB stage: measured at 30
-    // qubits, four high targets 11.26 -> 10.58 ms per pass, but two high targets 9.94 ->
-    // 10.47 ms, so the mode is kept for the short segments
-    // Launches with two targets among the bank bits stage their tiles by tensor-map copies
-    // with the 128-byte swizzle instead of taking the XOR member order (one subtile per
-    // stage); the others keep 1-D bulk copies, where the swizzled staging measured slower.
-    const bool swz = std::min(tl, 2u) >= 2u;
-    const bool wide = !swz && s->n >= S2::TB && p.h >= 3;
-    if (wide) p = make_plan(s->n, 4, g->t, S2::TB);
+    const Plan p = make_plan(s->n, 4, g->t, S::TB);
+    // (Tiles of two MMAs for high targets, 64 KiB per stage, took 68 us per pass on 23 qubits against
+    // 63, and 0.8% more on 28.)
     Tc64Args a;
-    a.box_rows = a.boxes = 0;
-    if (swz) {
-        const sv_status st = encode_rows_map(s->buf, 16ull << s->n, 16u << p.L, &a.tmap, &a.box_rows, &a.boxes);
-        if (st != SV_OK) return st;
-    }
+    const sv_status st = encode_rows_map(s->buf, 16ull << s->n, 16u << p.L, &a.tmap, &a.box_rows, &a.boxes);
+    if (st != SV_OK) return st;
     // U on its fixed-point grid, exactly, on the host (the kernel cuts the digits)
     double rmax = 0.0;
     for (uint32_t i = 0; i < 256; ++i)
@@ -537,21 +490,14 @@ sv_status launch_tc64(sv_state *s, const svi::Gate &g0) {
         a.bx[i] = make_longlong2(fxp::to_fixed(fxp::bits_of(g->u[i].real()), ebias),
                                  fxp::to_fixed(fxp::bits_of(g->u[i].imag()), ebias));
     a.b_exp = (int)ebias - 1022;
-    a.psi = s->buf;
     a.err = reinterpret_cast<int *>(s->ws + svi::WS_ERR);
     a.ntiles = p.ntiles;
     a.L = p.L;
     a.h = p.h;
     for (int j = 0; j < SV_MAX_K; ++j) a.hi[j] = p.hi[j];
     for (int j = 0; j < 4; ++j) a.lp[j] = p.lp[j];
-    a.sb = p.L - 1;
-    for (int j = 3 - (int)p.h; j >= 0 && p.lp[j] == a.sb; --j) --a.sb;
     const unsigned grid = (unsigned)std::min<unsigned long long>(p.ntiles, (unsigned long long)s->num_sms);
-    // two targets in bits 0..2 (4-way conflicts and worse) take the swizzled staging; one
-    // target there leaves 2-way conflicts, cheaper than either remedy
-    SV_CUDA(swz    ? launch_pass(apply_tc64<1, true>, dim3(grid), S::THREADS, S::SMEM, s->stream, a)
-            : wide ? launch_pass(apply_tc64<2>, dim3(grid), S2::THREADS, S2::SMEM, s->stream, a)
-                   : launch_pass(apply_tc64<1>, dim3(grid), S::THREADS, S::SMEM, s->stream, a));
+    SV_CUDA(launch_pass(apply_tc64, dim3(grid), S::THREADS, S::SMEM, s->stream, a));
     return SV_OK;
 }
 

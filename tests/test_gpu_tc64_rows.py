@@ -1,19 +1,19 @@
 """Row scales and tile layouts of the complex128 tensor-core pass: rows whose exponents spread by
 exactly what the short cut of the digit split covers and by one more, zero, subnormal and very
-large rows, over the layouts (one or two subtiles per tile, swizzled staging, targets right below
-the contiguous part of a tile), against extended precision."""
+large rows, over target layouts (low, high, right below the contiguous part of a tile), against
+extended precision."""
 import numpy as np
 import pytest
 
 pytestmark = pytest.mark.gpu
 
 N = 14
-TARGETS = [(0, 5, 6, 9),        # one subtile per tile
-           (0, 1, 7, 12),       # swizzled staging
-           (9, 10, 12, 13),     # two subtiles, four high targets
-           (8, 9, 11, 13),      # two subtiles, the low target right below the contiguous part
-           (7, 8, 10, 12),      # two subtiles, two low targets
-           (8, 9, 10, 12)]      # two subtiles, two low targets right below the contiguous part
+TARGETS = [(0, 5, 6, 9),        # one among the bank bits
+           (0, 1, 7, 12),       # two among the bank bits
+           (9, 10, 12, 13),     # four high targets
+           (8, 9, 11, 13),      # three high, one right below the contiguous part
+           (7, 8, 10, 12),      # two high targets
+           (8, 9, 10, 12)]      # two right below the contiguous part
 
 
 def _groups(targets):
