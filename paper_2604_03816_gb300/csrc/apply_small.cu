@@ -2,7 +2,7 @@
 //
 // A state of 12 qubits is 32 KiB (complex64) or 64 KiB (complex128): a pass per gate is all
 // launch latency, fill and drain (6-8 us for work of well under one).  Measured on the 12-qubit
-// brickwork circuit, pass per gate -> this: 350 gates in complex128 2169 -> 269 us, 21 width-5
+// brickwork circuit, pass per gate -> this: 350 gates in complex128 2169 -> 251 us, 21 width-5
 // gates in complex64 208 -> 66 us.  Here one cluster of up
 // to 16 CTAs keeps the state on chip and runs the gates one after the other, as many per
 // launch as fit the kernel's parameters (28 KiB: 350 unfused gates, or three dense width-5
@@ -21,7 +21,8 @@
 //
 // What bounds it: complex128 the FP64 pipe (4 2^k FP64 operations per amplitude and gate at
 // about 1.9 per clock and SM: 0.5 us for a one-qubit gate on 12 qubits over 16 SMs); complex64
-// the barriers (0.1-0.4 us) and, at width 5, shared-memory reads (64 8-byte reads per output).
+// the barriers (0.1-0.4 us) and, at width 5, the host, which needs about 12 us to classify and pack
+// the three matrices of a launch that runs 7.6 (two threads per amplitude: the same time).
 #include <cuda_runtime.h>
 
 #include <algorithm>
