@@ -355,13 +355,6 @@ __global__ void __launch_bounds__(THREADS, x_blocks<R, PLAIN>) x_sum(const __gri
     for (unsigned long long t = blockIdx.x; t < a.ntiles; t += gridDim.x, ++j) {
         const uint32_t s = j & 1u;
         const bool ok = svk::mbar_wait_bounded(svk::smem_u32(&full[s]), (j >> 1) & 1u);
-        if (!__syncthreads_and(ok)) {
-            // the copy may still be in flight: wait once more (bounded) before the memory goes
-            if (tid == 0) atomicOr(a.err, 8);
-            (void)svk::mbar_wait_bounded(svk::smem_u32(&full[s]), (j >> 1) & 1u);
-            (void)svk::mbar_wait_bounded(svk::smem_u32(&full[s ^ 1u]), ((j + 1u) >> 1) & 1u);
-            return;
-        }
         const C *tile = reinterpret_cast<const C *>(smem + s * TILE);
         // bit i: (-1)^{|base & z_i|}, lane i's term
         const uint32_t tile_signs = __ballot_sync(0xffffffffu, __popcll(sl.base(t) & my_z) & 1);
@@ -386,7 +379,7 @@ __global__ void __launch_bounds__(THREADS, x_blocks<R, PLAIN>) x_sum(const __gri
             }
         };
         if constexpr (PLAIN) {
-            if (act) {
+            if (act && ok) {
 #pragma unroll
                 for (uint32_t set = 0; set < X_SETS; ++set) {
                     if (set >= a.nsets) break;
@@ -401,7 +394,7 @@ __global__ void __launch_bounds__(THREADS, x_blocks<R, PLAIN>) x_sum(const __gri
                     }
                 }
             }
-        } else if (act) {
+        } else if (act && ok) {
             for (uint32_t set = 0; set < a.nsets; ++set) {
                 C v[16];
                 read_set(set, v);
@@ -438,7 +431,13 @@ __global__ void __launch_bounds__(THREADS, x_blocks<R, PLAIN>) x_sum(const __gri
             }
         }
         svk::fence_proxy_async_smem();        // reads of this tile before its refill
-        __syncthreads();
+        if (__syncthreads_or(!ok)) {
+            // the copy may still be in flight: wait once more (bounded) before the memory goes
+            if (tid == 0) atomicOr(a.err, 8);
+            (void)svk::mbar_wait_bounded(svk::smem_u32(&full[s]), (j >> 1) & 1u);
+            (void)svk::mbar_wait_bounded(svk::smem_u32(&full[s ^ 1u]), ((j + 1u) >> 1) & 1u);
+            return;
+        }
         const unsigned long long t2 = t + 2ull * gridDim.x;
         if (tid < 32 && t2 < a.ntiles) load(t2, s);
     }
