@@ -23,7 +23,7 @@
 // products and keep the general kernel.
 //
 // Measured, a transverse-field Ising chain on 26 qubits, complex64 (25 ZZ and 26 X terms):
-// 10.48 ms with one FP64 weight per amplitude and one pass per X-part -> 0.58 ms: z_sum 0.10 ms
+// 10.48 ms with one FP64 weight per amplitude and one pass per X-part -> 0.56 ms: z_sum 0.10 ms
 // (5.3 TB/s; 25 FP32 operations per amplitude), four x_sum passes of about 0.11 ms (4.8
 // TB/s; the latency of 24 warps per SM).
 // complex128 is bound by the FP64 pipe.
@@ -300,7 +300,8 @@ __device__ __forceinline__ R pair_any(const C (&v)[16], uint32_t signs, uint32_t
 
 // PLAIN: every term is a plain flip (at most four per set): running sums in registers, the sets
 // unrolled.  Without the sums' 32 KiB three blocks fit an SM (complex64), 24 warps to hide latency:
-// a 26-qubit field of 26 X terms and its ZZ chain 693 -> 577 us (two blocks: 641).
+// a 26-qubit field of 26 X terms and its ZZ chain 693 -> 577 us (two blocks: 641), and 560
+// with one block barrier per tile instead of two.
 template <typename R, bool PLAIN>
 constexpr int x_blocks = PLAIN && sizeof(R) == 4 ? 3 : 2;
 template <typename R, bool PLAIN>
