@@ -319,9 +319,9 @@ sv_status sv_gate_structure(const sv_gate *g, uint32_t *kind, uint32_t *control_
  * 4 and 5 on states of at least k + 7 qubits, and of any width on states of at least 13
  * qubits, run on the tensor cores, complex128 gates of width <= 4 on states of at least 11
  * qubits too, structured gates on the structure-aware kernels, everything else on the CUDA
- * cores; circuits on states of up to 12 qubits on one kernel that keeps the state on chip and
- * runs many gates per launch, whatever their width, unless a flag other than
- * SV_POLICY_STAGED_PROBS is set). */
+ * cores; circuits on states of up to 12 qubits (11 where the device schedules no cluster of 16
+ * CTAs) on one kernel that keeps the state on chip and runs many gates per launch, whatever their
+ * width, unless a flag other than SV_POLICY_STAGED_PROBS is set). */
 #define SV_POLICY_NO_TENSOR_CORES 1u   /* always use the CUDA-core kernels */
 #define SV_POLICY_DENSE_ONLY 2u        /* ignore gate structure: every gate a dense pass */
 /* sv_probs into page-locked host memory goes through a device buffer of the probabilities'

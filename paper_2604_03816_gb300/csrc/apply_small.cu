@@ -30,6 +30,7 @@
 #include <mutex>
 
 #include "ptx.cuh"
+#include "small_fit.h"
 #include "sv_internal.h"
 
 namespace svm {
@@ -42,9 +43,6 @@ __device__ __forceinline__ double2 mk(double a, double b) { return make_double2(
 __device__ __forceinline__ float fmar(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fmar(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-constexpr uint32_t MAX_N = 12;            // qubits
-constexpr uint32_t THREADS = 256;         // one amplitude each: 2^12 = 16 CTAs x 256
-constexpr uint32_t MAX_C = 4;             // log2 of the largest cluster
 constexpr uint32_t BLOB = 28 * 1024;      // ops, then their entries
 
 enum OpKind : uint32_t { OP_DIAG = 0, OP_MONO = 1, OP_DENSE = 2 };
@@ -305,8 +303,7 @@ sv_status Builder<R>::flush() {
     std::memcpy(a.blob + ob, data, used);
     a.psi = s->buf;
     a.n = s->n;
-    // at least 32 amplitudes per CTA, at most one per thread
-    a.c = s->n > 5 ? std::min(max_c, s->n - 5u) : 0u;
+    a.c = cluster_log2(s->n, max_c);
     a.nops = (uint32_t)ops.size();
     a.blob_bytes = (uint32_t)ob + used;
     ops.clear();
@@ -333,8 +330,11 @@ sv_status Builder<R>::flush() {
 namespace svi {
 
 bool small_state(const sv_state *s) {
-    return s->n <= svm::MAX_N &&
-           !(s->policy & (SV_POLICY_NO_TENSOR_CORES | SV_POLICY_DENSE_ONLY | SV_POLICY_TWO_GATE_PASSES));
+    if (s->n > svm::MAX_N || (s->policy & (SV_POLICY_NO_TENSOR_CORES | SV_POLICY_DENSE_ONLY | SV_POLICY_TWO_GATE_PASSES)))
+        return false;
+    uint32_t max_c = 0;
+    const cudaError_t e = s->dtype == SV_C64 ? svm::setup<float>(&max_c) : svm::setup<double>(&max_c);
+    return e == cudaSuccess && svm::state_fits(s->n, max_c);
 }
 
 template <typename R>

@@ -199,7 +199,7 @@ size_t launch_run(sv_state *s, const std::vector<Gate> &gates, const Structure *
 bool struct_preferred(const sv_state *s, const Structure &st);
 sv_status launch_apply_struct(sv_state *s, const Structure &st);
 uint64_t struct_bytes(const sv_state *s, const Structure &st);   // 2 s per amplitude it touches
-// States of up to 12 qubits without kernel-selection flags: gates [begin, end) in as few
+// States of up to 12 qubits (small_fit.h) without kernel-selection flags: gates [begin, end) in as few
 // launches as their matrices allow (apply_small.cu); *bytes is added to as by launch_apply.
 bool small_state(const sv_state *s);
 sv_status launch_small(sv_state *s, const std::vector<Gate> &gates, size_t begin, size_t end, uint64_t *bytes);
