@@ -30,6 +30,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <mutex>
 #include <type_traits>
@@ -489,6 +490,29 @@ struct DiagPlan {
     }
 };
 
+// The factors of a run are multiplied before they meet an amplitude, so the product of any of them
+// has to stay inside FP32: a run ends before a gate with which the largest or the smallest nonzero
+// product could pass 2^+-64 (gate by gate, 0 times 1e20 twice is 0; times their product, NaN).
+// Unitary gates never come near.
+struct Range {
+    double hi = 1.0, lo = 1.0;
+    bool add(const Gate &g) {
+        const uint32_t D = 1u << g.k;
+        double h = 1.0, l = 1.0;
+        for (uint32_t r = 0; r < D; ++r) {
+            const cplx z = g.u[(size_t)r * D + r];
+            const double m = std::max(std::fabs(z.real()), std::fabs(z.imag()));
+            if (!(m <= 0x1p64) || !(std::fabs(z.real()) <= m) || !(std::fabs(z.imag()) <= m)) return false;   // NaN too
+            h = std::max(h, m);
+            if (m > 0.0) l = std::min(l, m);
+        }
+        if (!(hi * h <= 0x1p64) || !(lo * l >= 0x1p-64)) return false;
+        hi *= h;
+        lo *= l;
+        return true;
+    }
+};
+
 uint64_t qubit_mask(const Gate &g) {
     uint64_t m = 0;
     for (uint32_t j = 0; j < g.k; ++j) m |= 1ull << g.t[j];
@@ -636,15 +660,16 @@ size_t launch_run(sv_state *s, const std::vector<Gate> &gates, const Structure *
         // the longer of a run inside the low bits and one with tables per tile
         size_t low_end = begin, i = begin;
         double low_share = 0.0;
+        Range low_range, range;
         while (low_end < end && low_end - begin < svr::MAX_GATES && kind(low_end) == SV_STRUCT_DIAGONAL &&
-               !(qubit_mask(gates[low_end]) >> T)) {
+               !(qubit_mask(gates[low_end]) >> T) && low_range.add(gates[low_end])) {
             low_share += touched(s, st[low_end - begin]);
             ++low_end;
         }
         DiagPlan plan;
         plan.T = T;
         for (; i < end && i - begin < svr::MAX_GATES && kind(i) == SV_STRUCT_DIAGONAL; ++i) {
-            if (!plan.add((uint32_t)(i - begin), qubit_mask(gates[i]))) break;
+            if (!range.add(gates[i]) || !plan.add((uint32_t)(i - begin), qubit_mask(gates[i]))) break;
             share += touched(s, st[i - begin]);
         }
         if (low_end - begin >= 2 && low_end >= i && run_pays(s, low_share, false)) {
