@@ -17,7 +17,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "plan.h"
 #include "ptx.cuh"
@@ -142,17 +141,16 @@ template <typename R, int K>
 sv_status launch_apply_t(sv_state *s, const svi::Gate &g) {
     constexpr uint32_t TB = tile_bits<R, K>();
     using C = typename C2<R>::T;
-    static std::once_flag once;
-    static int blocks_per_sm = 1;
-    static cudaError_t init_err = cudaSuccess;
-    std::call_once(once, [] {
+    struct Setup { cudaError_t err; int blocks_per_sm; };
+    static PerDevice<Setup> setup;
+    const auto [init_err, blocks_per_sm] = setup.get(current_device(), [] {
         const int maxb = int((1u << TB) * sizeof(C));
-        init_err = cudaFuncSetAttribute(apply_tile<R, K>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, maxb);
-        if (init_err == cudaSuccess)
-            init_err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm,
-                                                                     apply_tile<R, K>, 256, maxb);
-        if (blocks_per_sm < 1) blocks_per_sm = 1;
+        Setup r = {cudaSuccess, 1};
+        r.err = cudaFuncSetAttribute(apply_tile<R, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxb);
+        if (r.err == cudaSuccess)
+            r.err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r.blocks_per_sm, apply_tile<R, K>, 256, maxb);
+        if (r.blocks_per_sm < 1) r.blocks_per_sm = 1;
+        return r;
     });
     if (init_err != cudaSuccess)
         return svi::set_error(SV_ERR_CUDA, std::string("apply kernel setup: ") +

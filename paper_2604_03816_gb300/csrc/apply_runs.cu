@@ -32,7 +32,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <mutex>
 #include <type_traits>
 
 #include "ptx.cuh"
@@ -595,14 +594,12 @@ sv_status launch_diag_run(sv_state *s, const std::vector<Gate> &gates, size_t be
     a.ntiles = 1ull << (s->n - plan.T);
     SV_CUDA(svk::launch_pass(diag_tables<R>, dim3(ta.ntabs), 1u << TAB_Q, 0, s->stream, ta));
     const size_t smem = ((size_t)a.ntabs << TAB_Q) * sizeof(C) + (2u << BIN_Q) * sizeof(C) + ((size_t)a.ntabs << BIN_Q) * 2;
-    static std::once_flag once;
-    static cudaError_t err = cudaSuccess;
-    std::call_once(once, [] {
-        err = cudaFuncSetAttribute(apply_diag_run<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)(((size_t)MAX_TABS << TAB_Q) * sizeof(C) + (2u << BIN_Q) * sizeof(C) +
-                                         ((size_t)MAX_TABS << BIN_Q) * 2));
-    });
-    SV_CUDA(err);
+    static svk::PerDevice<cudaError_t> setup;
+    SV_CUDA(setup.get(svk::current_device(), [] {
+        return cudaFuncSetAttribute(apply_diag_run<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)(((size_t)MAX_TABS << TAB_Q) * sizeof(C) + (2u << BIN_Q) * sizeof(C) +
+                                          ((size_t)MAX_TABS << BIN_Q) * 2));
+    }));
     const unsigned grid = (unsigned)std::min<unsigned long long>(a.ntiles, 3ull * s->num_sms);
     SV_CUDA(svk::launch_pass(apply_diag_run<R>, dim3(grid), THREADS, smem, s->stream, a));
     return SV_OK;
@@ -633,12 +630,10 @@ sv_status launch_swap_run(sv_state *s, const uint8_t (&pi)[SV_MAX_QUBITS]) {
     }
     a.ntiles = 1ull << nr;
     const size_t smem = 2 * sizeof(C) * (size_t)((1u << a.h) * ((1u << a.a) + 1u));
-    static std::once_flag once;
-    static cudaError_t err = cudaSuccess;
-    std::call_once(once, [] {
-        err = cudaFuncSetAttribute(apply_swap_run<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, 72 * 1024);
-    });
-    SV_CUDA(err);
+    static svk::PerDevice<cudaError_t> setup;
+    SV_CUDA(setup.get(svk::current_device(), [] {
+        return cudaFuncSetAttribute(apply_swap_run<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, 72 * 1024);
+    }));
     // an odd stride: which of a pair of tiles does the work depends on the tile number's low
     // bits first, and an even stride gave half of the blocks three quarters of it (1.45 -> 0.94 ms,
     // and 0.84 with a tile's place formed by the lanes together)

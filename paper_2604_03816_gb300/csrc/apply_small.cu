@@ -27,7 +27,6 @@
 
 #include <algorithm>
 #include <cstring>
-#include <mutex>
 
 #include "ptx.cuh"
 #include "small_fit.h"
@@ -263,13 +262,13 @@ struct Builder {
 // Cluster size (log2) for this device: 16 CTAs where the device schedules them, else 8.
 template <typename R>
 static cudaError_t setup(uint32_t *max_c) {
-    static std::once_flag once;
-    static cudaError_t err = cudaSuccess;
-    static uint32_t mc = 3;
-    std::call_once(once, [] {
+    struct Setup { cudaError_t err; uint32_t max_c; };
+    static svk::PerDevice<Setup> setup;
+    const Setup done = setup.get(svk::current_device(), [] {
         const int smem = int((2u << MAX_N) * 2u * sizeof(R) + BLOB);
-        err = cudaFuncSetAttribute(apply_small<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (err != cudaSuccess) return;
+        Setup r = {cudaSuccess, 3};
+        r.err = cudaFuncSetAttribute(apply_small<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (r.err != cudaSuccess) return r;
         if (cudaFuncSetAttribute(apply_small<R>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
             cudaLaunchAttribute at;
             at.id = cudaLaunchAttributeClusterDimension;
@@ -282,12 +281,13 @@ static cudaError_t setup(uint32_t *max_c) {
             cfg.attrs = &at;
             cfg.numAttrs = 1;
             int nc = 0;
-            if (cudaOccupancyMaxActiveClusters(&nc, apply_small<R>, &cfg) == cudaSuccess && nc > 0) mc = MAX_C;
+            if (cudaOccupancyMaxActiveClusters(&nc, apply_small<R>, &cfg) == cudaSuccess && nc > 0) r.max_c = MAX_C;
         }
         (void)cudaGetLastError();
+        return r;
     });
-    *max_c = mc;
-    return err;
+    *max_c = done.max_c;
+    return done.err;
 }
 
 template <typename R>

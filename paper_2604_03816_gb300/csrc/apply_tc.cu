@@ -720,12 +720,12 @@ template <int K>
 sv_status launch_tc_t(sv_state *s, const svi::Gate &g) {
     using S = TcShape<K>;
     constexpr uint32_t D = S::D;
-    static std::once_flag once;
-    static cudaError_t init_err = cudaSuccess;
-    std::call_once(once, [] {
-        auto allow = [](auto kernel) {
-            if (init_err == cudaSuccess)
-                init_err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
+    static PerDevice<cudaError_t> setup;
+    const cudaError_t init_err = setup.get(current_device(), [] {
+        cudaError_t e = cudaSuccess;
+        auto allow = [&e](auto kernel) {
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
         };
         allow(apply_tc<K, false>);
         allow(apply_tc<K, true>);
@@ -733,6 +733,7 @@ sv_status launch_tc_t(sv_state *s, const svi::Gate &g) {
             allow(apply_tc<K, false, false, true>);
             allow(apply_tc<K, false, false, true, true>);
         }
+        return e;
     });
     if (init_err != cudaSuccess)
         return svi::set_error(SV_ERR_CUDA, std::string("tensor-core kernel setup: ") +
@@ -799,15 +800,14 @@ sv_status launch_tc_t(sv_state *s, const svi::Gate &g) {
 // widths 4 and 5) run as width-5 gates (a narrower gate widened by identity qubits, chosen as in
 // widen_gate) with the swizzled tensor-map staging (SW), like single states.
 static cudaError_t tc_batch_setup() {
-    static std::once_flag once;
-    static cudaError_t err = cudaSuccess;
-    std::call_once(once, [] {
+    static PerDevice<cudaError_t> setup;
+    return setup.get(current_device(), [] {
         constexpr int smem = (int)TcShape<5, true>::SMEM;
-        err = cudaFuncSetAttribute(apply_tc<5, false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (err == cudaSuccess)
-            err = cudaFuncSetAttribute(apply_tc<5, false, true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaError_t e = cudaFuncSetAttribute(apply_tc<5, false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(apply_tc<5, false, true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        return e;
     });
-    return err;
 }
 
 // Also looks up the tensor-map encoder, so that a launch inside a stream capture finds it.

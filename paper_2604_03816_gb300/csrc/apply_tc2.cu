@@ -55,7 +55,6 @@
 #include <cmath>
 #include <cstring>
 #include <memory>
-#include <mutex>
 
 #include "ptx.cuh"
 #include "sv_internal.h"
@@ -537,14 +536,13 @@ bool tc2_pair_fits(const sv_state *s, const Gate &g0, const Gate &g1) {
 // adds no targets among the bank-selecting bits), then one launch.
 sv_status launch_apply_tc2(sv_state *s, const Gate &g0_in, const Gate &g1_in) {
     using S = svk::Tc2Shape;
-    static std::once_flag once;
-    static cudaError_t init_err = cudaSuccess;
-    std::call_once(once, [] {
-        init_err = cudaFuncSetAttribute(svk::apply_tc2<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)S::SMEM);
-        if (init_err == cudaSuccess)
-            init_err = cudaFuncSetAttribute(svk::apply_tc2<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)S::SMEM);
+    static svk::PerDevice<cudaError_t> setup;
+    const cudaError_t init_err = setup.get(svk::current_device(), [] {
+        cudaError_t e = cudaFuncSetAttribute(svk::apply_tc2<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)S::SMEM);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(svk::apply_tc2<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
+        return e;
     });
     if (init_err != cudaSuccess)
         return set_error(SV_ERR_CUDA, std::string("two-gate tensor-core kernel setup: ") + cudaGetErrorString(init_err));

@@ -42,7 +42,6 @@
 
 #include <algorithm>
 #include <cmath>
-#include <mutex>
 #include <type_traits>
 
 #include "fixed_point.h"
@@ -459,10 +458,9 @@ __global__ void __launch_bounds__(608, 1) apply_tc64(const __grid_constant__ Tc6
 
 sv_status launch_tc64(sv_state *s, const svi::Gate &g0) {
     using S = Tc64;
-    static std::once_flag once;
-    static cudaError_t init_err = cudaSuccess;
-    std::call_once(once, [] {
-        init_err = cudaFuncSetAttribute(apply_tc64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
+    static PerDevice<cudaError_t> setup;
+    const cudaError_t init_err = setup.get(current_device(), [] {
+        return cudaFuncSetAttribute(apply_tc64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
     });
     if (init_err != cudaSuccess)
         return svi::set_error(SV_ERR_CUDA, std::string("tensor-core kernel setup: ") +

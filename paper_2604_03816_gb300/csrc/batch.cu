@@ -164,24 +164,25 @@ constexpr uint32_t BATCH_TB_MIN = 10, BATCH_TB_MAX = 13;
 
 template <typename R, int K>
 struct BatchKernel {
-    // The dynamic shared-memory limit is set for the largest tile once; the resident CTAs
-    // per SM are measured per tile size.
+    // The dynamic shared-memory limit is set for the largest tile once per device; the resident
+    // CTAs per SM are measured per tile size.
     static cudaError_t prepare(uint32_t tb, int *blocks_per_sm) {
-        static std::once_flag once;
-        static int bps[BATCH_TB_MAX + 1] = {};
-        static cudaError_t err = cudaSuccess;
-        std::call_once(once, [] {
+        struct Setup { cudaError_t err; int bps[BATCH_TB_MAX + 1]; };
+        static PerDevice<Setup> setup;
+        const Setup done = setup.get(current_device(), [] {
             using C = typename BC2<R>::T;
-            err = cudaFuncSetAttribute(apply_batch_tile<R, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       int((1u << BATCH_TB_MAX) * sizeof(C)));
-            for (uint32_t t = BATCH_TB_MIN; t <= BATCH_TB_MAX && err == cudaSuccess; ++t) {
-                err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps[t], apply_batch_tile<R, K>, 256,
-                                                                    int((1u << t) * sizeof(C)));
-                if (bps[t] < 1) bps[t] = 1;
+            Setup r = {};
+            r.err = cudaFuncSetAttribute(apply_batch_tile<R, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         int((1u << BATCH_TB_MAX) * sizeof(C)));
+            for (uint32_t t = BATCH_TB_MIN; t <= BATCH_TB_MAX && r.err == cudaSuccess; ++t) {
+                r.err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r.bps[t], apply_batch_tile<R, K>, 256,
+                                                                      int((1u << t) * sizeof(C)));
+                if (r.bps[t] < 1) r.bps[t] = 1;
             }
+            return r;
         });
-        *blocks_per_sm = bps[tb];
-        return err;
+        *blocks_per_sm = done.bps[tb];
+        return done.err;
     }
     static sv_status launch(const sv_batch_launch &L) {
         using C = typename BC2<R>::T;

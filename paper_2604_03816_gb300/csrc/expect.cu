@@ -34,7 +34,6 @@
 #include <cmath>
 #include <cstring>
 #include <functional>
-#include <mutex>
 #include <type_traits>
 #include <vector>
 
@@ -695,14 +694,13 @@ sv_status x_pass(sv_state *s, Partials &P, const std::vector<Term> &t, std::vect
     a.err = reinterpret_cast<int *>(s->ws + WS_ERR);
     constexpr size_t tile_bytes = sizeof(typename Geo<R>::C) << Geo<R>::T;
     constexpr size_t smem = 2 * tile_bytes + X_TERMS * ((1u << Geo<R>::T) / 16) * sizeof(typename Sum<R>::T);
-    static std::once_flag once;
-    static cudaError_t err = cudaSuccess;
-    std::call_once(once, [] {
-        err = cudaFuncSetAttribute(x_sum<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (err == cudaSuccess)
-            err = cudaFuncSetAttribute(x_sum<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * tile_bytes));
-    });
-    SV_CUDA(err);
+    static svk::PerDevice<cudaError_t> setup;
+    SV_CUDA(setup.get(svk::current_device(), [] {
+        cudaError_t e = cudaFuncSetAttribute(x_sum<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(x_sum<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * tile_bytes));
+        return e;
+    }));
     SV_CUDA(plain ? svk::launch_pass(x_sum<R, true>, dim3(nb), THREADS, 2 * tile_bytes, s->stream, a)
                            : svk::launch_pass(x_sum<R, false>, dim3(nb), THREADS, smem, s->stream, a));
     P.used += nb;

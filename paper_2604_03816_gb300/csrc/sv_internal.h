@@ -11,6 +11,7 @@
 #include <utility>
 #include <vector>
 
+#include "per_device.h"
 #include "sv.h"
 
 namespace svi {
@@ -148,6 +149,12 @@ struct sv_batch_launch {
 };
 
 namespace svk {
+inline int current_device() {
+    int dev = 0;
+    (void)cudaGetDevice(&dev);
+    return dev;
+}
+
 // Launch a kernel that begins with pass_trigger() and calls pass_wait() before its first access
 // to memory that other kernels touch: its launch latency and prologue overlap the previous
 // kernel's tail.
