@@ -351,8 +351,8 @@ typedef struct {
     size_t l2_bytes;         /* chunk budget in bytes (0: 64 MiB) */
     uint32_t no_graph;       /* 1: launch directly instead of through the CUDA graph */
     uint32_t timing;         /* 1: time the passes with CUDA events (synchronises) */
-    uint32_t no_tensor_cores; /* 1: complex64 gates on the CUDA cores (default: on the tensor
-                                 cores when n >= 13, widths 4 and 5 when n >= 12) */
+    uint32_t no_tensor_cores; /* 1: complex64 width-4/5 gates on the CUDA cores too (default:
+                                 on the tensor cores when n >= 12) */
     uint32_t tile_bits;      /* CUDA-core passes: tiles of 2^tile_bits amplitudes per CTA,
                                 10..13 (0: 12 for complex64, 11 for complex128) */
 } sv_batch_opts;

@@ -796,9 +796,9 @@ sv_status launch_tc_t(sv_state *s, const svi::Gate &g) {
     return SV_OK;
 }
 
-// Batched launches (sv_batch_apply): complex64 gates on states of at least 13 qubits (12 for
-// widths 4 and 5) run as width-5 gates (a narrower gate widened by identity qubits, chosen as in
-// widen_gate) with the swizzled tensor-map staging (SW), like single states.
+// Batched launches (sv_batch_apply): complex64 gates of widths 4 and 5 on states of at least 12
+// qubits, the former widened by an identity qubit (chosen as in widen_gate), with the swizzled
+// tensor-map staging (SW) like single states.
 static cudaError_t tc_batch_setup() {
     static PerDevice<cudaError_t> setup;
     return setup.get(current_device(), [] {

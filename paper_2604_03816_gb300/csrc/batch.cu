@@ -346,12 +346,14 @@ static sv_status batch_launch(const sv_batch_launch &L) {
     }
 }
 
-// The tensor cores serve complex64 gates of width 4 and 5 on states of at least 12 qubits, and
-// narrower ones from 13 (one tile more): 18 qubits x 96 states, width 3: 141 us on the CUDA
-// cores, 79 widened.
-static bool batch_tc(sv_dtype dt, uint32_t n, uint32_t k) {
-    return dt == SV_C64 && n >= (k >= 4 ? 12u : 13u);
-}
+// The tensor cores serve complex64 gates of width 4 and 5 on states of at least 12 qubits.  Narrower
+// ones stay on the CUDA cores' FP32 multiply-adds: widened to 5, 2^(5-k) independent groups share one
+// fixed-point grid, so amplitudes far below a neighbouring group's lose their relative accuracy
+// and an infinity spreads to groups that the gate does not connect; and a pass of few or
+// small states costs more there (fills and drains and the operands' packing: 14 qubits x 2 states,
+// widths 1 / 2 / 3: 288 / 154 / 102 us per circuit on the CUDA cores, 472 / 252 / 153 widened; only
+// width 3 on large batches gains, 18 qubits x 96 states 141 -> 79 us per pass).
+static bool batch_tc(sv_dtype dt, uint32_t n, uint32_t k) { return dt == SV_C64 && n >= 12 && k >= 4; }
 
 static cudaError_t batch_prepare(sv_dtype dt, uint32_t k) {
     int bps = 0;
