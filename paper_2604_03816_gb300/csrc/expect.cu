@@ -17,9 +17,9 @@
 // One read of the state thus serves up to twelve single-qubit flips (26 qubits: 4 reads).
 //
 // Precision: p_k, re_k and im_k are formed as before (FP32 operations for complex64, runs of
-// eight FP32 pairs for x != 0); everything is then accumulated in two-float arithmetic (an
-// error-free sum and its error, about 48 bits) for complex64 and FP64 for complex128, and
-// weighted in FP64.  complex64 groups of more than four terms with one x != 0 had FP64
+// eight FP32 pairs for x != 0); complex64 then adds up to 128 tiles per thread in two-float
+// arithmetic (two_float.h) and everything beyond, weights included, in FP64 -- larger states take
+// several launches; complex128 is FP64 throughout.  complex64 groups of more than four terms with one x != 0 had FP64
 // products and keep the general kernel.
 //
 // Measured, a transverse-field Ising chain on 26 qubits, complex64 (25 ZZ and 26 X terms):
@@ -40,30 +40,13 @@
 #include "ptx.cuh"
 #include "reduce.cuh"
 #include "sv_internal.h"
+#include "two_float.h"
 
 namespace svx {
 
 using svk::block_sum;
 using svk::prob_of;
 
-// Running sums: two floats (s + e, error-free additions), or one double.
-struct SumF {
-    float s, e;
-    __device__ void clear() { s = e = 0.f; }
-    __device__ void add(float x) {
-        const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
-        e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b)));
-        s = t;
-    }
-    // (an infinite sum has no error term)
-    __device__ double value() const { return isfinite(s) ? (double)s + (double)e : (double)s; }
-};
-struct SumD {
-    double s;
-    __device__ void clear() { s = 0.0; }
-    __device__ void add(double x) { s += x; }
-    __device__ double value() const { return s; }
-};
 template <typename R> struct Sum;
 template <> struct Sum<float> { using T = SumF; };
 template <> struct Sum<double> { using T = SumD; };
@@ -109,7 +92,8 @@ struct ZArgs {
     double *partial;
     uint32_t t, nhi;
     uint32_t low;                              // 1: this pass adds table 0 (z_hi = 0)
-    unsigned long long ntiles;
+    unsigned long long ntiles;                 // of a state
+    unsigned long long begin, end;             // tiles of this launch
     unsigned long long zc[Z_CLASSES];          // z_hi of the classes
     unsigned long long zh[Z_TERMS];            // z_hi of the terms with z_lo = 0
     double ch[Z_TERMS];
@@ -144,12 +128,12 @@ __global__ void __launch_bounds__(THREADS, NC >= 2 ? 1 : 2) z_sum(const __grid_c
         for (uint32_t v = 0; v < NV; ++v) {
             const uint32_t i = v * THREADS + tid;
             next[v] = V{};
-            if (tile < a.ntiles && i < tile_vec) next[v] = psi[tile * tile_vec + i];
+            if (tile < a.end && i < tile_vec) next[v] = psi[tile * tile_vec + i];
         }
     };
-    load(blockIdx.x);
+    load(a.begin + blockIdx.x);
     uint32_t j = 0;
-    for (unsigned long long tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x, ++j) {
+    for (unsigned long long tile = a.begin + blockIdx.x; tile < a.end; tile += gridDim.x, ++j) {
         if ((j & 7u) == 0) {
             // weights and signs of the next eight tiles, one tile per warp
             const unsigned long long t = tile + (unsigned long long)warp * gridDim.x;
@@ -228,7 +212,7 @@ struct XArgs {
     CUtensorMap tmap;
     uint32_t box_rows, boxes, tb;             // tile bits
     uint32_t L, h, hi[SV_MAX_K];
-    unsigned long long ntiles;
+    unsigned long long begin, end;            // tiles of this launch
     double *partial;
     int *err;
     uint32_t nsets, first[X_SETS], last[X_SETS];   // other terms of set i: first[i] .. last[i] - 1
@@ -348,11 +332,11 @@ __global__ void __launch_bounds__(THREADS, x_blocks<R, PLAIN>) x_sum(const __gri
         }
     };
     if (tid < 32) {
-        load(blockIdx.x, 0);
-        if (blockIdx.x + (unsigned long long)gridDim.x < a.ntiles) load(blockIdx.x + gridDim.x, 1);
+        load(a.begin + blockIdx.x, 0);
+        if (a.begin + blockIdx.x + gridDim.x < a.end) load(a.begin + blockIdx.x + gridDim.x, 1);
     }
     uint32_t j = 0;
-    for (unsigned long long t = blockIdx.x; t < a.ntiles; t += gridDim.x, ++j) {
+    for (unsigned long long t = a.begin + blockIdx.x; t < a.end; t += gridDim.x, ++j) {
         const uint32_t s = j & 1u;
         const bool ok = svk::mbar_wait_bounded(svk::smem_u32(&full[s]), (j >> 1) & 1u);
         const C *tile = reinterpret_cast<const C *>(smem + s * TILE);
@@ -439,7 +423,7 @@ __global__ void __launch_bounds__(THREADS, x_blocks<R, PLAIN>) x_sum(const __gri
             return;
         }
         const unsigned long long t2 = t + 2ull * gridDim.x;
-        if (tid < 32 && t2 < a.ntiles) load(t2, s);
+        if (tid < 32 && t2 < a.end) load(t2, s);
     }
     double acc = 0.0;
     if (act)
@@ -471,6 +455,12 @@ namespace svi {
 namespace {
 
 struct Term { uint64_t x, z; double c; };
+
+// Tiles of one launch of nb blocks: all of them, in complex64 at most RUN_TILES per thread.
+template <typename R>
+unsigned long long run_tiles(unsigned long long nb) {
+    return sizeof(R) == 4 ? svx::RUN_TILES * nb : 1ull << SV_MAX_QUBITS;
+}
 
 // Block partials of several passes, summed in order by one kernel per full buffer; the sums
 // are fetched when their slots run out, and at the end.
@@ -554,22 +544,26 @@ sv_status z_passes(const void *psi, uint32_t nq, uint32_t states, int num_sms, c
             for (uint32_t c = 0; c < nc; ++c) ta.zc[1 + c] = a.zc[c] = cls[done + c];
             // as many blocks as the device holds, shared by the states
             const unsigned long long slots = (unsigned long long)(nc >= 2 ? 1 : 2) * (unsigned long long)num_sms;
-            const int nb = (int)std::min<unsigned long long>(a.ntiles, std::max<unsigned long long>(1, slots / states));
-            sv_status st = reserve(nb, &a.partial);
-            if (st != SV_OK) return st;
+            const unsigned long long blocks = std::max<unsigned long long>(1, slots / states);
             if (a.low || nc)
                 SV_CUDA(svk::launch_pass(z_table, dim3((unsigned)(((1u << T) + 127) / 128), ta.ntab), 128, 0, stream, ta));
-            const dim3 grid(nb, states);
-            cudaError_t e = cudaSuccess;
-            switch (nc) {
-                case 0: e = svk::launch_pass(z_sum<R, 0>, grid, THREADS, 0, stream, a); break;
-                case 1: e = svk::launch_pass(z_sum<R, 1>, grid, THREADS, 0, stream, a); break;
-                case 2: e = svk::launch_pass(z_sum<R, 2>, grid, THREADS, 0, stream, a); break;
-                default: e = svk::launch_pass(z_sum<R, 3>, grid, THREADS, 0, stream, a); break;
+            for (a.begin = 0; a.begin < a.ntiles; a.begin = a.end) {
+                a.end = std::min(a.ntiles, a.begin + run_tiles<R>(blocks));
+                const int nb = (int)std::min(blocks, a.end - a.begin);
+                const dim3 grid(nb, states);
+                sv_status st = reserve(nb, &a.partial);
+                if (st != SV_OK) return st;
+                cudaError_t e = cudaSuccess;
+                switch (nc) {
+                    case 0: e = svk::launch_pass(z_sum<R, 0>, grid, THREADS, 0, stream, a); break;
+                    case 1: e = svk::launch_pass(z_sum<R, 1>, grid, THREADS, 0, stream, a); break;
+                    case 2: e = svk::launch_pass(z_sum<R, 2>, grid, THREADS, 0, stream, a); break;
+                    default: e = svk::launch_pass(z_sum<R, 3>, grid, THREADS, 0, stream, a); break;
+                }
+                SV_CUDA(e);
+                st = ran(nb);
+                if (st != SV_OK) return st;
             }
-            SV_CUDA(e);
-            st = ran(nb);
-            if (st != SV_OK) return st;
             done += nc;
             first = false;
         }
@@ -681,16 +675,13 @@ sv_status x_pass(sv_state *s, Partials &P, const std::vector<Term> &t, std::vect
     const sv_status st = svk::encode_rows_map(s->buf, (unsigned long long)sizeof(typename Geo<R>::C) << s->n,
                                               (uint32_t)sizeof(typename Geo<R>::C) << L, &a.tmap, &a.box_rows, &a.boxes);
     if (st != SV_OK) return st;
-    a.ntiles = 1ull << (s->n - a.tb);
+    const unsigned long long ntiles = 1ull << (s->n - a.tb);
     uint32_t flips = 0;
     for (uint32_t q = 0; q < ns; ++q) flips += a.nplain[q];
     const bool plain = flips == total;
     // as many blocks as the device holds
-    const int nb = (int)std::min<unsigned long long>(a.ntiles, (unsigned long long)(plain ? x_blocks<R, true> : x_blocks<R, false>) *
-                                                                   (unsigned long long)s->num_sms);
-    const sv_status rs = P.reserve(nb);
-    if (rs != SV_OK) return rs;
-    a.partial = P.part();
+    const unsigned long long blocks = (unsigned long long)(plain ? x_blocks<R, true> : x_blocks<R, false>) *
+                                      (unsigned long long)s->num_sms;
     a.err = reinterpret_cast<int *>(s->ws + WS_ERR);
     constexpr size_t tile_bytes = sizeof(typename Geo<R>::C) << Geo<R>::T;
     constexpr size_t smem = 2 * tile_bytes + X_TERMS * ((1u << Geo<R>::T) / 16) * sizeof(typename Sum<R>::T);
@@ -701,9 +692,16 @@ sv_status x_pass(sv_state *s, Partials &P, const std::vector<Term> &t, std::vect
             e = cudaFuncSetAttribute(x_sum<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * tile_bytes));
         return e;
     }));
-    SV_CUDA(plain ? svk::launch_pass(x_sum<R, true>, dim3(nb), THREADS, 2 * tile_bytes, s->stream, a)
-                           : svk::launch_pass(x_sum<R, false>, dim3(nb), THREADS, smem, s->stream, a));
-    P.used += nb;
+    for (a.begin = 0; a.begin < ntiles; a.begin = a.end) {
+        a.end = std::min(ntiles, a.begin + run_tiles<R>(blocks));
+        const int nb = (int)std::min(blocks, a.end - a.begin);       // every block has a tile
+        const sv_status rs = P.reserve(nb);
+        if (rs != SV_OK) return rs;
+        a.partial = P.part();
+        SV_CUDA(plain ? svk::launch_pass(x_sum<R, true>, dim3(nb), THREADS, 2 * tile_bytes, s->stream, a)
+                      : svk::launch_pass(x_sum<R, false>, dim3(nb), THREADS, smem, s->stream, a));
+        P.used += nb;
+    }
     return SV_OK;
 }
 
