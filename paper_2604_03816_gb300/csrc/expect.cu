@@ -8,8 +8,9 @@
 //   * terms with z_lo = 0: sum over the tiles of w_hi(tile) (sum of p over the tile);
 //   * the others, by their distinct z_hi (a "class"; a nearest-neighbour chain has one): as
 //     the first kind, with the tiles' signs: w_c[k_lo] (sum over tiles of s(tile) p).
-// So an amplitude costs a few additions however many terms there are, where one weight per
-// term and amplitude was formed in FP64 before (25 chain terms on 26 qubits: 6.6 ms).
+// So an amplitude costs a few additions however many terms there are, where the general kernel forms
+// one weight per term and amplitude in FP64 (25 chain terms on 26 qubits: 6.6 ms).  Terms of many
+// classes go there all the same where that is cheaper (z_split.h).
 //
 // x != 0, x_sum.  A tile of 2^T amplitudes (the low index bits and up to five high ones) is
 // staged in shared memory by swizzled tensor-map copies; each thread takes 16 of them, four
@@ -41,6 +42,7 @@
 #include "reduce.cuh"
 #include "sv_internal.h"
 #include "two_float.h"
+#include "z_split.h"
 
 namespace svx {
 
@@ -58,7 +60,6 @@ template <> struct Geo<double> { static constexpr uint32_t T = 11, E = 8; using 
 // ---------------------------------------------------------------- Z strings
 
 constexpr uint32_t Z_TERMS = 512;    // terms per pass
-constexpr uint32_t Z_CLASSES = 3;    // mixed classes per pass
 constexpr uint32_t THREADS = 256;
 
 struct ZTableArgs {
@@ -742,6 +743,11 @@ sv_status x_group(sv_state *s, Partials &P, const std::vector<Term> &t) {
 
 }  // namespace
 
+std::vector<char> batch_z_split(uint32_t n, sv_dtype dtype, uint32_t states, const uint64_t *z, size_t nterms) {
+    const uint32_t T = std::min(n, dtype == SV_C64 ? svx::Geo<float>::T : svx::Geo<double>::T);
+    return svx::split_z(z, nterms, T, std::ldexp((double)states, (int)n), svx::Z_COST_BATCH[dtype]);
+}
+
 // Z strings on a batch: the tables (4 x 2^12 doubles) and `partial` (room for `room` doubles) are the
 // caller's; after each pass `fold` is called with the number of partials per state that lie there.
 sv_status batch_z_terms(const void *psi, uint32_t n, sv_dtype dtype, uint32_t states, int num_sms, cudaStream_t stream,
@@ -770,25 +776,35 @@ static sv_status expect_terms(sv_state *s, const uint64_t *x, const uint64_t *z,
         size_t e = i;
         while (e < nterms && t[e].x == t[i].x) ++e;
         sv_status st = SV_OK;
+        size_t g = i;                       // t[g] .. t[e - 1] take the general kernel
         if (t[i].x == 0 && !general) {
-            st = s->dtype == SV_C64 ? z_group<float>(s, P, &t[i], e - i) : z_group<double>(s, P, &t[i], e - i);
+            std::vector<uint64_t> zs;
+            for (size_t q = i; q < e; ++q) zs.push_back(t[q].z);
+            const uint32_t T = std::min(s->n, s->dtype == SV_C64 ? svx::Geo<float>::T : svx::Geo<double>::T);
+            const std::vector<char> to_general =
+                svx::split_z(zs.data(), zs.size(), T, std::ldexp(1.0, (int)s->n), svx::Z_COST_SINGLE[s->dtype]);
+            std::vector<Term> tiled, rest;
+            for (size_t q = i; q < e; ++q) (to_general[q - i] ? rest : tiled).push_back(t[q]);
+            std::copy(rest.begin(), rest.end(), std::copy(tiled.begin(), tiled.end(), t.begin() + i));
+            g = i + tiled.size();
+            if (g > i)
+                st = s->dtype == SV_C64 ? z_group<float>(s, P, &t[i], g - i) : z_group<double>(s, P, &t[i], g - i);
         } else if (!general && s->n >= 4 && __builtin_popcountll(t[i].x) <= 4 && (s->dtype == SV_C128 || e - i <= 4)) {
             xt.insert(xt.end(), t.begin() + i, t.begin() + e);
-        } else {
-            // general kernel, up to 32 terms per launch
-            for (size_t b = i; b < e && st == SV_OK; b += 32) {
-                uint64_t zz[32];
-                double cc[32];
-                const int m = (int)std::min<size_t>(32, e - b);
-                for (int q = 0; q < m; ++q) {
-                    zz[q] = t[b + q].z;
-                    cc[q] = t[b + q].c;
-                }
-                double *out;
-                st = P.fold();
-                if (st == SV_OK) st = P.slot(&out);
-                if (st == SV_OK) st = enqueue_expect_group(s, t[i].x, zz, cc, m, out);
+            g = e;
+        }
+        for (size_t b = g; b < e && st == SV_OK; b += 32) {      // up to 32 terms per launch
+            uint64_t zz[32];
+            double cc[32];
+            const int m = (int)std::min<size_t>(32, e - b);
+            for (int q = 0; q < m; ++q) {
+                zz[q] = t[b + q].z;
+                cc[q] = t[b + q].c;
             }
+            double *out;
+            st = P.fold();
+            if (st == SV_OK) st = P.slot(&out);
+            if (st == SV_OK) st = enqueue_expect_group(s, t[b].x, zz, cc, m, out);
         }
         if (st != SV_OK) return st;
         i = e;

@@ -229,6 +229,7 @@ sv_status enqueue_expect_group(sv_state *s, uint64_t x, const uint64_t *z, const
 sv_status batch_z_terms(const void *psi, uint32_t n, sv_dtype dtype, uint32_t states, int num_sms, cudaStream_t stream,
                         double *tables, double *partial, size_t room, const uint64_t *z, const double *c, size_t nterms,
                         const std::function<sv_status(int)> &fold);
+std::vector<char> batch_z_split(uint32_t n, sv_dtype dtype, uint32_t states, const uint64_t *z, size_t nterms);
 sv_status launch_topk(sv_state *s, uint32_t k, uint64_t *idx, double *p);
 sv_status enqueue_topk(sv_state *s, double *host_p, unsigned long long *host_i);
 sv_status launch_widen(sv_state *s, const void *src_c64, void *dst_c128);
