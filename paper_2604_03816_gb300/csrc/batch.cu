@@ -15,7 +15,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -23,9 +22,9 @@
 #include <mutex>
 #include <new>
 #include <string>
-#include <system_error>
 #include <thread>
 
+#include "group_threads.h"
 #include "plan.h"
 #include "ptx.cuh"
 #include "sv_internal.h"
@@ -775,43 +774,28 @@ sv_status sv_batch_apply(sv_batch *b, const sv_circuit *const *circuits, const s
         const uint32_t i0 = std::min(b->count, w * per), i1 = std::min(b->count, i0 + per);
         fill(i0, i1, cut[q], cut[q + 1]);
     };
-    std::atomic<uint32_t> ready[3];
-    for (std::atomic<uint32_t> &c : ready) c.store(0);
-    std::vector<std::thread> th;
-    try {
-        for (uint32_t w = 1; w < nt; ++w)
-            th.emplace_back([&, w] {
-                for (size_t q = 0; q < ngroups; ++q) {
-                    share(w, q);
-                    ready[q].fetch_add(1, std::memory_order_release);
-                }
-            });
-    } catch (const std::system_error &) {
-        // no more threads: the calling thread converts the rest
-    }
-    sv_status rc = SV_OK;
-    for (size_t q = 0; q < ngroups; ++q) {
-        share(0, q);
-        for (uint32_t w = (uint32_t)th.size() + 1; w < nt; ++w) share(w, q);
-        while (ready[q].load(std::memory_order_acquire) < th.size()) std::this_thread::yield();
-        if (rc != SV_OK) continue;           // the threads must still finish
+    auto enqueue_group = [&](size_t q) -> sv_status {
         const size_t from = goff[cut[q]], bytes = goff[cut[q + 1]] - from;
-        auto step = [&]() -> sv_status {
-            if (bytes)
-                SV_CUDA(cudaMemcpyAsync(static_cast<char *>(b->utab) + from, static_cast<char *>(b->utab_host) + from,
-                                        bytes, cudaMemcpyHostToDevice, b->stream));
-            if (q + 1 == ngroups) SV_CUDA(cudaEventRecord(b->staged, b->stream));
-            if (timing) SV_CUDA(cudaEventRecord(b->ev0, b->stream));
-            if (use_graph) {
-                SV_CUDA(cudaGraphLaunch(b->graphs[q], b->stream));
-                return SV_OK;
-            }
-            return enqueue_gates(b->stream, cut[q], cut[q + 1]);
-        };
-        rc = step();
-        if (q + 1 == ngroups) b->staged_pending = true;
+        if (bytes)
+            SV_CUDA(cudaMemcpyAsync(static_cast<char *>(b->utab) + from, static_cast<char *>(b->utab_host) + from,
+                                    bytes, cudaMemcpyHostToDevice, b->stream));
+        if (q + 1 == ngroups) {
+            SV_CUDA(cudaEventRecord(b->staged, b->stream));
+            b->staged_pending = true;
+        }
+        if (timing) SV_CUDA(cudaEventRecord(b->ev0, b->stream));
+        if (use_graph) {
+            SV_CUDA(cudaGraphLaunch(b->graphs[q], b->stream));
+            return SV_OK;
+        }
+        return enqueue_gates(b->stream, cut[q], cut[q + 1]);
+    };
+    sv_status rc = SV_OK;
+    try {
+        svk::in_groups(nt, ngroups, share, [&](size_t q) { return (rc = enqueue_group(q)) == SV_OK; });
+    } catch (const std::bad_alloc &) {
+        rc = set_error(SV_ERR_OOM, "sv_batch_apply: host allocation failed");
     }
-    for (std::thread &t : th) t.join();
     if (rc != SV_OK) {
         cudaStreamSynchronize(b->stream);    // the staging buffer may still be read
         return rc;
