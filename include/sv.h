@@ -533,7 +533,8 @@ sv_status sv_shard_unpack(sv_state *s, uint32_t bit, uint32_t value, uint64_t of
 sv_status sv_set_zero(sv_state *s);
 
 /* Testing aid (no counterpart in the paper): the next `count` allocations of a state
- * buffer (sv_alloc, sv_set_dtype, a promotion) fail as if device memory were exhausted,
+ * buffer (sv_alloc, sv_set_dtype, a promotion) or of the room for a batch's tensor-core
+ * operands (sv_batch_apply) fail as if device memory were exhausted,
  * so that tests can drive the out-of-memory paths without exhausting the GPU.  0 turns
  * it off.  Host only; process-wide. */
 sv_status sv_debug_fail_allocs(uint32_t count);

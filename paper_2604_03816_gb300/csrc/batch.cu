@@ -388,7 +388,8 @@ struct sv_batch {
     size_t partial_room = 0;
     double *results = nullptr;          // count
     void *images = nullptr;             // tensor-core operands of some gates (pack_images), then
-    size_t images_cap = 0;              // their scales: room for images_cap of them
+    size_t images_cap = 0;              // their scales: room for images_cap of them, of the
+    size_t images_asked = 0;            // images_asked that were wanted
     void *utab = nullptr;               // device matrix table
     size_t utab_cap = 0;
     void *utab_host = nullptr;          // pinned staging of the table
@@ -644,20 +645,23 @@ sv_status sv_batch_apply(sv_batch *b, const sv_circuit *const *circuits, const s
     if (ntc) {
         const size_t one = svk::tc_batch_image_bytes() + sizeof(float);
         size_t want = std::min<size_t>(ntc * chunk, (size_t(256) << 20) / one);
-        if (b->images_cap < want) {
+        // (not again for a request that was cut down before: what was granted then stays)
+        if (b->images_asked < want) {
             SV_CUDA(cudaStreamSynchronize(b->stream));
             if (b->images) cudaFree(b->images);
             b->images = nullptr;
-            b->images_cap = 0;
+            b->images_cap = b->images_asked = 0;
             drop_graphs(b);                 // they hold the old address
-            cudaError_t e = cudaMalloc(&b->images, want * one);
+            const size_t asked = want;
+            cudaError_t e = alloc_state_buffer(&b->images, want * one);
             while (e == cudaErrorMemoryAllocation && want > 1) {
                 (void)cudaGetLastError();
                 want /= 2;
-                e = cudaMalloc(&b->images, want * one);
+                e = alloc_state_buffer(&b->images, want * one);
             }
             SV_CUDA(e);
             b->images_cap = want;
+            b->images_asked = asked;
         }
     }
 

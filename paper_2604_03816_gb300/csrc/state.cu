@@ -63,10 +63,11 @@ static sv_status validate_gate(const sv_gate *g, uint32_t n, const char *who) {
     return SV_OK;
 }
 
-// Test hook: the next g_fail_allocs state-buffer allocations fail (sv_debug_fail_allocs).
+// Test hook: the next g_fail_allocs allocations of a state buffer or of a batch's operand room fail
+// (sv_debug_fail_allocs).
 static std::atomic<uint32_t> g_fail_allocs{0};
 
-static cudaError_t alloc_state_buffer(void **p, size_t bytes) {
+cudaError_t alloc_state_buffer(void **p, size_t bytes) {
     uint32_t left = g_fail_allocs.load();
     while (left > 0 && !g_fail_allocs.compare_exchange_weak(left, left - 1)) {
     }

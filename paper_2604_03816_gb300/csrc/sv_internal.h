@@ -241,6 +241,8 @@ sv_status read_results(sv_state *s, void *dst, size_t bytes);
 // The circuit's input gates fused again at width <= 4 when its schedule has width-5 gates
 // (built once per circuit), else its schedule: what complex128 runs on the tensor cores.
 const std::vector<Gate> &narrow_schedule(const sv_circuit *c);
+// cudaMalloc that sv_debug_fail_allocs can make fail.
+cudaError_t alloc_state_buffer(void **p, size_t bytes);
 // SV_ERR_STATE (with a message) when a failed reallocation left the state without a buffer.
 sv_status check_live(const sv_state *s, const char *who);
 sv_status enqueue_expect_sum(const void *psi, uint32_t n, sv_dtype dtype, const uint64_t *x,
