@@ -665,11 +665,15 @@ sv_status sv_batch_apply(sv_batch *b, const sv_circuit *const *circuits, const s
         }
     }
 
-    std::string key = std::to_string(b->n) + "/" + std::to_string(b->count) + "/" +
-                      std::to_string(b->dtype) + "/" + std::to_string(chunk) + "/" +
-                      (tc_ok ? "tc/" : "cc/") + std::to_string(tile_bits) + "/";
-    for (const Gate &g : c0->gates)
-        for (uint32_t j = 0; j < g.k; ++j) key += std::to_string(g.t[j]) + (j + 1 < g.k ? "," : ";");
+    // what the captured graphs depend on beside the batch (as bytes: texts took a few microseconds
+    // that nothing overlaps)
+    const uint32_t shape[3] = {chunk, (uint32_t)tc_ok, tile_bits};
+    std::string key(reinterpret_cast<const char *>(shape), sizeof(shape));
+    key.reserve(sizeof(shape) + G * (SV_MAX_K + 1) + 1);
+    for (const Gate &g : c0->gates) {
+        key.push_back((char)g.k);
+        for (uint32_t j = 0; j < g.k; ++j) key.push_back((char)g.t[j]);
+    }
 
     auto enqueue_gates = [&](cudaStream_t stream, size_t first_gate, size_t last_gate) -> sv_status {
         float *scales = reinterpret_cast<float *>(static_cast<char *>(b->images) +
@@ -737,14 +741,10 @@ sv_status sv_batch_apply(sv_batch *b, const sv_circuit *const *circuits, const s
     r.passes = (uint64_t)G * b->count;
     r.launches = (uint64_t)G * ((b->count + chunk - 1) / chunk);
     r.bytes = (uint64_t)G * b->count * 2ull * sbytes;
-    // Gates in up to three groups when the batch is one chunk: the first gates' matrices are
-    // converted, uploaded and their passes launched while host threads convert the rest (18
-    // qubits x 96 circuits: 0.9 ms of conversion and upload before the first pass, now 0.2).
-    // Several chunks need every gate first, and a timed call measures the passes alone.
-    std::vector<size_t> cut = {0, G};
-    if (chunk >= b->count && !timing && G >= 8) cut = {0, G / 8, G / 3, G};
+    // a timed call measures the passes alone: one group
+    const std::vector<size_t> cut = svk::group_cuts(G, tab, chunk >= b->count && !timing);
     const size_t ngroups = cut.size() - 1;
-    key += "|" + std::to_string(ngroups);
+    key.push_back((char)ngroups);
     if (use_graph && (b->graphs.size() != ngroups || b->graph_key != key)) {
         for (const Gate &g : c0->gates) SV_CUDA(use_tc(g) ? svk::tc_batch_prepare() : batch_prepare(b->dtype, g.k));
         drop_graphs(b);

@@ -11,6 +11,18 @@
 
 namespace svk {
 
+// Where a batch's gates are cut into groups (ends with the gate count): the first gates' matrices are
+// converted, uploaded and their passes launched while host threads convert the rest (18 qubits x
+// 96 circuits: 0.9 ms of conversion and upload before the first pass, 0.2 in three groups).  Only
+// when the batch is one chunk (several need every gate first), and when the table of all matrices is
+// large enough: a group costs one more copy and one more graph launch, and below 512 KiB one group
+// was faster on every batch tried (10 qubits x 2 states, 27 gates of two qubits: 121 us in three
+// groups, 94 in one; above, three: 16 qubits x 8, 18 gates of five qubits: 204 and 242).
+inline std::vector<size_t> group_cuts(size_t ngates, size_t table_bytes, bool one_chunk) {
+    if (!one_chunk || ngates < 8 || table_bytes < (size_t(512) << 10)) return {0, ngates};
+    return {0, ngates / 8, ngates / 3, ngates};
+}
+
 // share(w, q): worker w's part of group q, workers 0 .. nt - 1 (0 is the calling thread; where a thread
 // cannot be had it does that worker's part too).  step(q), once group q is prepared, in the
 // calling thread and in order; returns false to stop.  The threads have ended when this returns or

@@ -33,3 +33,10 @@ extern "C" int run_groups(unsigned workers, int groups, int at, int how, int *st
         if (p > 1) r = 2;
     return r;
 }
+
+// group_cuts into cut[0 .. 4); returns the number of groups.
+extern "C" int group_cuts(unsigned long gates, unsigned long table_bytes, int one_chunk, long *cut) {
+    const std::vector<size_t> c = svk::group_cuts(gates, table_bytes, one_chunk != 0);
+    for (size_t i = 0; i < c.size(); ++i) cut[i] = (long)c[i];
+    return (int)c.size() - 1;
+}
