@@ -383,11 +383,6 @@ namespace svi {
 
 namespace {
 
-// The share of the state a structured gate changes.
-double touched(const sv_state *s, const Structure &st) {
-    return (double)struct_bytes(s, st) / (double)(2ull * ((s->dtype == SV_C64 ? 8ull : 16ull) << s->n));
-}
-
 // A run moves the state once: 0.64 ms on 28 qubits in complex64, against 0.33-0.37 ms for a
 // gate that touches half of it, so it pays from a touched share of 1.25 on.  complex128 with two
 // tables per tile takes two products per amplitude on the FP64 pipe, against one per touched
@@ -467,7 +462,6 @@ struct DiagPlan {
     // Add gate number i with these qubits; false (and unchanged) if the run is full.
     bool add(uint32_t i, uint64_t q) {
         const uint64_t low = (1ull << T) - 1;
-        const std::vector<Table> before = tabs;
         Table *best = nullptr;
         for (Table &t : tabs) {
             if ((t.qubits & low) != (q & low) || __builtin_popcountll(t.qubits | q) > (int)svr::TAB_Q) continue;
@@ -480,10 +474,17 @@ struct DiagPlan {
             tabs.push_back(Table());
             best = &tabs.back();
         }
+        const uint64_t before = best->qubits;
+        if (before && (before | q) == before) {              // nothing new to pack
+            best->gates.push_back(i);
+            return true;
+        }
         best->qubits |= q;
         best->gates.push_back(i);
         if (pack()) return true;
-        tabs = before;
+        best->gates.pop_back();
+        best->qubits = before;
+        if (!before) tabs.pop_back();
         pack();
         return false;
     }
@@ -644,29 +645,34 @@ sv_status launch_swap_run(sv_state *s, const uint8_t (&pi)[SV_MAX_QUBITS]) {
 
 }  // namespace
 
-size_t launch_run(sv_state *s, const std::vector<Gate> &gates, const Structure *st, size_t begin, size_t end,
-                  sv_status *status) {
+size_t launch_run(sv_state *s, const std::vector<Gate> &gates, const Structure *st, const double *touched,
+                  size_t begin, size_t end, size_t *tried, sv_status *status) {
     *status = SV_OK;
+    *tried = 0;
     const uint32_t T = s->dtype == SV_C64 ? svr::tile_bits<float>() : svr::tile_bits<double>();
     if (s->n < T) return 0;
-    auto kind = [&](size_t i) { return st[i - begin].kind; };
+    const uint32_t kind = st[0].kind;
     double share = 0.0;
-    if (kind(begin) == SV_STRUCT_DIAGONAL) {
+    if (kind == SV_STRUCT_DIAGONAL) {
+        end = std::min(end, begin + svr::MAX_GATES);
+        for (size_t q = begin; q < end; ++q) share += touched[q - begin];
+        if (!run_pays(s, share, false)) return 0;       // not even all of them
+        share = 0.0;
         // the longer of a run inside the low bits and one with tables per tile
         size_t low_end = begin, i = begin;
         double low_share = 0.0;
         Range low_range, range;
-        while (low_end < end && low_end - begin < svr::MAX_GATES && kind(low_end) == SV_STRUCT_DIAGONAL &&
-               !(qubit_mask(gates[low_end]) >> T) && low_range.add(gates[low_end])) {
-            low_share += touched(s, st[low_end - begin]);
+        while (low_end < end && !(qubit_mask(gates[low_end]) >> T) && low_range.add(gates[low_end])) {
+            low_share += touched[low_end - begin];
             ++low_end;
         }
         DiagPlan plan;
         plan.T = T;
-        for (; i < end && i - begin < svr::MAX_GATES && kind(i) == SV_STRUCT_DIAGONAL; ++i) {
+        for (; i < end; ++i) {
             if (!range.add(gates[i]) || !plan.add((uint32_t)(i - begin), qubit_mask(gates[i]))) break;
-            share += touched(s, st[i - begin]);
+            share += touched[i - begin];
         }
+        *tried = std::max(i, low_end) - begin;
         if (low_end - begin >= 2 && low_end >= i && run_pays(s, low_share, false)) {
             *status = s->dtype == SV_C64 ? launch_low_run<float>(s, gates, begin, low_end)
                                          : launch_low_run<double>(s, gates, begin, low_end);
@@ -677,7 +683,7 @@ size_t launch_run(sv_state *s, const std::vector<Gate> &gates, const Structure *
                                      : launch_diag_run<double>(s, gates, begin, i, plan);
         return i - begin;
     }
-    if (kind(begin) == SV_STRUCT_MONOMIAL) {
+    if (kind == SV_STRUCT_MONOMIAL) {
         // the product of the run's bit permutations, as long as it only swaps pairs
         uint8_t pi[SV_MAX_QUBITS], good[SV_MAX_QUBITS];
         for (uint32_t q = 0; q < SV_MAX_QUBITS; ++q) pi[q] = (uint8_t)q;
@@ -685,13 +691,13 @@ size_t launch_run(sv_state *s, const std::vector<Gate> &gates, const Structure *
         size_t i = begin, upto = begin;
         double upto_share = 0.0;
         uint32_t perm[SV_MAX_K];
-        for (; i < end && kind(i) == SV_STRUCT_MONOMIAL && bit_permutation(gates[i], perm); ++i) {
+        for (; i < end && bit_permutation(gates[i], perm); ++i) {
             const Gate &g = gates[i];
             uint8_t to[SV_MAX_QUBITS];
             for (uint32_t q = 0; q < SV_MAX_QUBITS; ++q) to[q] = (uint8_t)q;
             for (uint32_t j = 0; j < g.k; ++j) to[g.t[j]] = (uint8_t)g.t[perm[j]];
             for (uint32_t q = 0; q < SV_MAX_QUBITS; ++q) pi[q] = to[pi[q]];   // this gate after the others
-            share += touched(s, st[i - begin]);
+            share += touched[i - begin];
             bool pairs = true;
             for (uint32_t q = 0; q < SV_MAX_QUBITS; ++q) pairs = pairs && pi[pi[q]] == q;
             if (pairs) {
@@ -700,6 +706,7 @@ size_t launch_run(sv_state *s, const std::vector<Gate> &gates, const Structure *
                 std::memcpy(good, pi, sizeof(pi));
             }
         }
+        *tried = i - begin;
         if (upto - begin < 2 || !run_pays(s, upto_share, false)) return 0;
         *status = s->dtype == SV_C64 ? launch_swap_run<float>(s, good) : launch_swap_run<double>(s, good);
         return upto - begin;
