@@ -106,7 +106,6 @@ __global__ void __launch_bounds__(256) apply_diag(const __grid_constant__ DiagAr
     using V = typename Vec<R, VEC>::T;
     constexpr int ILP = 4;
     __shared__ C tab[1 << SV_MAX_K];
-    svk::pass_trigger();
     if (threadIdx.x < (1u << a.k)) tab[threadIdx.x] = mk(a.d[2 * threadIdx.x], a.d[2 * threadIdx.x + 1]);
     __syncthreads();
     svk::pass_wait();
@@ -166,7 +165,6 @@ template <typename R, int K>
 __global__ void __launch_bounds__(256) apply_mono(const __grid_constant__ MonoArgs<R, K> a) {
     using C = typename Cx<R>::T;
     constexpr int D = 1 << K, ILP = mono_ilp<R, K>();
-    svk::pass_trigger();
     svk::pass_wait();
     C *psi = reinterpret_cast<C *>(a.psi);
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
@@ -210,7 +208,6 @@ template <typename R, int K>
 __global__ void __launch_bounds__(256) apply_ctrl(const __grid_constant__ CtrlArgs<R, K> a) {
     using C = typename Cx<R>::T;
     constexpr int D = 1 << K;
-    svk::pass_trigger();
     svk::pass_wait();
     C *psi = reinterpret_cast<C *>(a.psi);
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
