@@ -25,8 +25,7 @@
 // memory, read and written in rows of 2^a amplitudes.
 //
 // When: a run moves the whole state once, so it pays when its gates, one pass each, touch more
-// than that.  `touched` is the sum over the gates of the share of the state each changes; the
-// thresholds are at run_pays.
+// than that; the thresholds and what they were measured at stand at ONE_PRODUCT and least_gates.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -387,8 +386,15 @@ namespace {
 // gate that touches half of it, so it pays from a touched share of 1.25 on.  complex128 with two
 // tables per tile takes two products per amplitude on the FP64 pipe, against one per touched
 // amplitude: from 2.25 on.
-bool run_pays(const sv_state *s, double share, bool two_products) {
-    return share >= (s->dtype == SV_C128 && two_products ? 2.25 : 1.25);
+constexpr double ONE_PRODUCT = 1.25;
+double two_products(const sv_state *s) { return s->dtype == SV_C128 ? 2.25 : 1.25; }
+
+// A diagonal run is two launches, so below 20 qubits, where launches are what counts, two gates stay
+// two passes (two rotations on 15 qubits: 15.0 us, 18.4 as a run; complex128, inside the low bits, 19.4
+// and 22.7; on 20 qubits 19.0 and 18.4, 31 and 28).  Three gates: 17 us and 19 alone, the same in a
+// longer circuit; complex128 with two tables per tile 24 and 28, four gates 28 either way.
+size_t least_gates(const sv_state *s, bool two) {
+    return s->n >= 20 ? 2 : two && s->dtype == SV_C128 ? 4 : 3;
 }
 
 // Is the gate a permutation of its index bits?  Then out bit j of its targets comes from target
@@ -647,38 +653,31 @@ sv_status launch_swap_run(sv_state *s, const uint8_t (&pi)[SV_MAX_QUBITS]) {
 
 size_t launch_run(sv_state *s, const std::vector<Gate> &gates, const Structure *st, const double *touched,
                   size_t begin, size_t end, size_t *tried, sv_status *status) {
+    auto share = [&](size_t upto) { return touched[upto - begin] - touched[0]; };       // of gates begin .. upto - 1
     *status = SV_OK;
     *tried = 0;
     const uint32_t T = s->dtype == SV_C64 ? svr::tile_bits<float>() : svr::tile_bits<double>();
     if (s->n < T) return 0;
     const uint32_t kind = st[0].kind;
-    double share = 0.0;
     if (kind == SV_STRUCT_DIAGONAL) {
         end = std::min(end, begin + svr::MAX_GATES);
-        for (size_t q = begin; q < end; ++q) share += touched[q - begin];
-        if (!run_pays(s, share, false)) return 0;       // not even all of them
-        share = 0.0;
+        if (end - begin < least_gates(s, false) || share(end) < ONE_PRODUCT) return 0;     // not even all of them
         // the longer of a run inside the low bits and one with tables per tile
         size_t low_end = begin, i = begin;
-        double low_share = 0.0;
         Range low_range, range;
-        while (low_end < end && !(qubit_mask(gates[low_end]) >> T) && low_range.add(gates[low_end])) {
-            low_share += touched[low_end - begin];
-            ++low_end;
-        }
+        while (low_end < end && !(qubit_mask(gates[low_end]) >> T) && low_range.add(gates[low_end])) ++low_end;
+        const bool low = low_end - begin >= least_gates(s, false) && share(low_end) >= ONE_PRODUCT;
+        if (!low && share(end) < two_products(s)) return 0;
         DiagPlan plan;
         plan.T = T;
-        for (; i < end; ++i) {
-            if (!range.add(gates[i]) || !plan.add((uint32_t)(i - begin), qubit_mask(gates[i]))) break;
-            share += touched[i - begin];
-        }
+        while (i < end && range.add(gates[i]) && plan.add((uint32_t)(i - begin), qubit_mask(gates[i]))) ++i;
         *tried = std::max(i, low_end) - begin;
-        if (low_end - begin >= 2 && low_end >= i && run_pays(s, low_share, false)) {
+        if (low && low_end >= i) {
             *status = s->dtype == SV_C64 ? launch_low_run<float>(s, gates, begin, low_end)
                                          : launch_low_run<double>(s, gates, begin, low_end);
             return low_end - begin;
         }
-        if (i - begin < 2 || !run_pays(s, share, true)) return 0;
+        if (i - begin < least_gates(s, true) || share(i) < two_products(s)) return 0;
         *status = s->dtype == SV_C64 ? launch_diag_run<float>(s, gates, begin, i, plan)
                                      : launch_diag_run<double>(s, gates, begin, i, plan);
         return i - begin;
@@ -689,7 +688,6 @@ size_t launch_run(sv_state *s, const std::vector<Gate> &gates, const Structure *
         for (uint32_t q = 0; q < SV_MAX_QUBITS; ++q) pi[q] = (uint8_t)q;
         std::memcpy(good, pi, sizeof(pi));
         size_t i = begin, upto = begin;
-        double upto_share = 0.0;
         uint32_t perm[SV_MAX_K];
         for (; i < end && bit_permutation(gates[i], perm); ++i) {
             const Gate &g = gates[i];
@@ -697,17 +695,16 @@ size_t launch_run(sv_state *s, const std::vector<Gate> &gates, const Structure *
             for (uint32_t q = 0; q < SV_MAX_QUBITS; ++q) to[q] = (uint8_t)q;
             for (uint32_t j = 0; j < g.k; ++j) to[g.t[j]] = (uint8_t)g.t[perm[j]];
             for (uint32_t q = 0; q < SV_MAX_QUBITS; ++q) pi[q] = to[pi[q]];   // this gate after the others
-            share += touched[i - begin];
             bool pairs = true;
             for (uint32_t q = 0; q < SV_MAX_QUBITS; ++q) pairs = pairs && pi[pi[q]] == q;
             if (pairs) {
                 upto = i + 1;
-                upto_share = share;
                 std::memcpy(good, pi, sizeof(pi));
             }
         }
         *tried = i - begin;
-        if (upto - begin < 2 || !run_pays(s, upto_share, false)) return 0;
+        // one launch, like a pass: from the same share on at every size
+        if (upto - begin < 2 || share(upto) < ONE_PRODUCT) return 0;
         *status = s->dtype == SV_C64 ? launch_swap_run<float>(s, good) : launch_swap_run<double>(s, good);
         return upto - begin;
     }

@@ -587,25 +587,29 @@ static sv_status run_schedule(sv_state *s, const std::vector<Gate> &gates, size_
     // pass per gate)
     const bool runs = !small && !(s->policy & (SV_POLICY_DENSE_ONLY | SV_POLICY_TWO_GATE_PASSES));
     std::vector<Structure> structure;      // of the gates looked at so far
-    std::vector<double> share;             // and the share of the state each touches
+    std::vector<double> share = {0.0};     // and the shares of the state they touch, added up
     structure.reserve(runs ? end - begin : 0);
-    share.reserve(runs ? end - begin : 0);
+    share.reserve(runs ? end - begin + 1 : 1);
     auto kind_of = [&](size_t i) {
         while (structure.size() <= i) {
             structure.push_back(classify(gates[begin + structure.size()]));
             const Structure &t = structure.back();
-            share.push_back(t.kind == SV_STRUCT_DIAGONAL || t.kind == SV_STRUCT_MONOMIAL
-                                ? (double)struct_bytes(s, t) / (double)(2 * state_bytes(s)) : 0.0);
+            share.push_back(share.back() + (t.kind == SV_STRUCT_DIAGONAL || t.kind == SV_STRUCT_MONOMIAL
+                                                ? (double)struct_bytes(s, t) / (double)(2 * state_bytes(s)) : 0.0));
         }
         return structure[i].kind;
     };
     size_t next_try = 0;                   // the next gate that a run may start with
+    size_t alike = 0;                      // gates i .. alike - 1 are known to be of gate i's kind
     for (size_t i = 0; i < first.size() && st == SV_OK; ++i) {
         if (runs) {
             size_t e = i + 1;              // gates of one structured kind in a row, as far as a run goes
             const uint32_t kind = kind_of(i);
-            if (i >= next_try && (kind == SV_STRUCT_DIAGONAL || kind == SV_STRUCT_MONOMIAL))
+            if (i >= next_try && (kind == SV_STRUCT_DIAGONAL || kind == SV_STRUCT_MONOMIAL)) {
+                e = std::max(e, alike);
                 while (begin + e < end && e - i < RUN_GATES && kind_of(e) == kind) ++e;
+                alike = e;
+            }
             size_t tried = 0;
             const size_t m = e - i < 2 ? 0 : launch_run(s, gates, structure.data() + i, share.data() + i, begin + i,
                                                         begin + e, &tried, &st);

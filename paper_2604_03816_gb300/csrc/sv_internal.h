@@ -202,8 +202,8 @@ namespace svi {
 sv_status launch_apply(sv_state *s, const Gate &g, uint64_t *bytes = nullptr, int *kind = nullptr,
                        const Structure *st = nullptr);
 // Gates from `begin` on that share one pass (apply_runs.cu; st[i - begin]: gate i's structure, share[i -
-// begin]: the share of the state it touches; all of one kind): how many it ran, 0 if there is no run
-// there that pays -- then *tried is how many gates a plan in vain went over.
+// begin + 1] - share[i - begin]: the share of the state it touches; all of one kind): how many it ran, 0
+// if there is no run there that pays -- then *tried is how many gates a plan in vain went over.
 constexpr size_t RUN_GATES = 64;      // gates looked at for a run
 size_t launch_run(sv_state *s, const std::vector<Gate> &gates, const Structure *st, const double *share, size_t begin,
                   size_t end, size_t *tried, sv_status *status);
