@@ -45,20 +45,16 @@ FALLBACK_HBM_GBS = 6800.0
 # as null once those sources hash differently).
 KERNELS = {
     "c64": {"files": ("apply_tc.cu", "tc.cuh", "ptx.cuh", "plan.h"),
-            "sha256_prefix": "7bea4dcfbf277a2a", "n": 30,
-            "bytes_per_launch": (1.074020e9 + 1.012702e9) * 8,
-            "kernel": "fused-gate passes: apply_tc<5,0,0,1,0> 98.2% of GPU time "
-                      "(profiles/fused_pass_grid30q_k5_launches.md)",
-            "traffic_source": "apply_tc<5,0,0,1,0> ncu capture at 27q scaled to 30q "
-                              "(profiles/apply_tc5_c64_27q_ncu.md)"},
+            "sha256_prefix": "19796a3897b20f33", "n": 30,
+            "bytes_per_launch": (1.073791e9 + 1.012954e9) * 8,
+            "kernel": "fused-gate passes: apply_tc<5,0,0,1,0> 98.2% of GPU time",
+            "traffic_source": "apply_tc<5,0,0,1,0> ncu capture at 27q scaled to 30q"},
     "c128": {"files": ("apply_tc64.cu", "fixed_point.h", "tc.cuh", "ptx.cuh", "plan.h"),
-             "sha256_prefix": "09c53ac21ae52432", "n": 30,
-             "bytes_per_launch": (2.147576e9 + 2.085352e9) * 8,
-             "kernel": "fused-gate passes: apply_tc64 98.0% of GPU time "
-                       "(profiles/fused_pass_grid30q_c128_k4_launches.md); bound by issue and "
-                       "the integer ALU pipe, not HBM (profiles/apply_tc64_c128_27q_ncu.md)",
-             "traffic_source": "apply_tc64 ncu capture at 27q scaled to 30q "
-                               "(profiles/apply_tc64_c128_27q_ncu.md)"},
+             "sha256_prefix": "8e77802f2dbadecb", "n": 30,
+             "bytes_per_launch": (2.147615e9 + 2.085817e9) * 8,
+             "kernel": "fused-gate passes: apply_tc64 98.0% of GPU time; bound by issue and "
+                       "the integer ALU pipe, not HBM",
+             "traffic_source": "apply_tc64 ncu capture at 27q scaled to 30q"},
 }
 
 

@@ -258,7 +258,8 @@ sv_status sv_norm(sv_state *s, double *out);
 sv_status sv_probs(sv_state *s, void *out, int out_on_device);
 /* out = sum_t coef[t] <psi| P_t |psi> for Pauli strings P_t given by xmask[t] (X or Y
  * on those qubits) and zmask[t] (Z or Y): P|k> = i^{|x&z|} (-1)^{|k&z|} |k^x>.
- * Accumulated in FP64.  Synchronises. */
+ * Accumulated in FP64; complex64 forms products in FP32 and adds up to 128 of a thread's terms in two
+ * floats first, whose error stays below FP64's rounding of the sum.  Synchronises. */
 sv_status sv_expect(sv_state *s, const uint64_t *xmask, const uint64_t *zmask,
                     const double *coef, size_t nterms, double *out);
 /* Noisy simulation with density matrices (Section 9.5): rho on n <= 17 qubits is the
@@ -359,7 +360,7 @@ typedef struct {
 
 typedef struct {
     uint64_t passes;         /* fused gates x states */
-    uint64_t launches;       /* kernel launches (fused gates x chunks) */
+    uint64_t launches;       /* passes launched (fused gates x chunks) */
     uint64_t bytes;          /* algorithmic bytes: passes * 2 * 2^n * s */
     uint32_t chunk_states;
     uint32_t graph_reused;   /* 1 if a previously captured graph was replayed */
@@ -385,11 +386,15 @@ sv_status sv_batch_set_basis(sv_batch *b, uint64_t x);     /* every state to |x>
 /* Copy state i (2^n amplitudes) to host (synchronises) or device memory. */
 sv_status sv_batch_get_state(sv_batch *b, uint32_t i, void *dst, int dst_on_device);
 /* Apply circuits[i] to state i for all i < count (see above).  opts and rep may be NULL.
- * SV_ERR_ARG if a circuit does not share the structure of circuits[0]. */
+ * SV_ERR_ARG if a circuit does not share the structure of circuits[0].  complex64 gates of widths 4
+ * and 5 on the tensor cores have the precision stated at sv_apply_circuit, the others are FP32 (FP64)
+ * multiply-adds.  Device memory kept by the batch: the table of matrices and up to 256 MiB for
+ * the tensor cores' operands (less where memory is short). */
 sv_status sv_batch_apply(sv_batch *b, const sv_circuit *const *circuits, const sv_batch_opts *opts,
                          sv_batch_report *rep);
 /* out[i] = sum_t coef[t] <psi_i| P_t |psi_i> for every state (host array of count
- * doubles), FP64 accumulation.  Synchronises. */
+ * doubles), accumulated as in sv_expect; where many Z strings share little, complex64 weights runs of
+ * eight amplitudes in FP32 (coefficients as two floats), added in FP64.  Synchronises. */
 sv_status sv_batch_expect(sv_batch *b, const uint64_t *xmask, const uint64_t *zmask,
                           const double *coef, size_t nterms, double *out);
 sv_status sv_batch_sync(sv_batch *b);

@@ -49,12 +49,13 @@
 // in pairs instead measured the same within 1% (faster on 24-qubit states, slower on 28).
 // Targets among tile bits 0..3 (where 8-byte accesses pick their bank) would make the
 // lanes of a warp hit one bank.  Width-5 launches on states of 13 qubits or more, and
-// batched launches, avoid that with the swizzled staging (SW); the others (11- and
-// 12-qubit states) take each group's members in a lane-dependent XOR order (XP), undone
-// in registers.
+// batched launches, avoid that with the swizzled staging (SW); the others take each group's
+// members in a lane-dependent XOR order (XP), undone in registers.  The others are width 4 on 11
+// qubits (K = 4) and widths 4 and 5 on 12; circuits on such states run in apply_small.cu, so only
+// single gates, the server's requests and passes that a policy flag asks for come here.
 // So loads, slicing, MMAs and stores of consecutive tiles overlap.  With A in tensor
-// memory, shared memory holds only B, the raw stages and the output staging, so 4 (k = 5)
-// or 8 (k = 4) tiles of loads can be in flight per SM.  Every wait is bounded and any
+// memory, shared memory holds only B, the raw stages and the output staging: four tiles (k = 5) or
+// eight (k = 4), of which two loads are in flight except where launch_tc_t says more.  Every wait is bounded and any
 // role that gives up makes the others leave too (abort flag).
 #include <cuda.h>
 #include <cuda_fp16.h>

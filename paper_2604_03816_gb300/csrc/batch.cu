@@ -952,7 +952,7 @@ sv_status sv_batch_tune(sv_batch *b, const sv_gate *gates, size_t ngates, uint32
     std::memset(&r, 0, sizeof(r));
     double best = 1e300;
     // chunk budgets: L2-resident chunks suit the CUDA-core passes; the tensor-core passes
-    // (a fixed cost of about 20 us per launch) prefer few large launches
+    // (5 us of fill and drain per launch) prefer few large launches
     const size_t sbytes = (b->dtype == SV_C64 ? size_t(8) : size_t(16)) << b->n;
     const size_t l2s[3] = {size_t(64) << 20, size_t(512) << 20, sbytes * b->count};
     for (uint32_t k = kmin; k <= kmax; ++k) {

@@ -1,5 +1,6 @@
-// Read-only reductions over the state: norm (Eq. 1), Z-basis probabilities, Pauli
-// expectations and the top-k outcomes, plus the small initialisation kernels.
+// Read-only reductions over the state: norm (Eq. 1), Z-basis probabilities and the general Pauli
+// expectations (the ones that share reads are in expect.cu, the top-k outcomes in topk.cu), plus the
+// small initialisation kernels.
 //
 // Every reduction reads the state once with 16-byte vector loads from a fixed-size
 // grid (so the partial-sum layout, and therefore the FP64 result, is the same on every
